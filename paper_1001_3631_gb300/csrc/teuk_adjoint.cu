@@ -120,25 +120,46 @@ __global__ void adj_init_kernel(InstDev d, const double2* gbar, CoLevel out) {
 // over a strip of output columns [c0, c1): at half node h it forms mu(h) = C^T lam' from
 // the integer columns h and h+1 (the angular neighbours of lam'_Pi through shared
 // memory), then lam^n(h) = H^T mu from the half nodes h-1 and h (the angular neighbours
-// of mu_Pi through shared memory), so neither mu nor lam' is written to memory.  The
-// arithmetic of each node is that of the two gather passes in the same order
-// (corrector: integer node h, then h+1; predictor: half node h-1, then h).  Over the
+// of mu_Pi through shared memory), so neither mu nor lam' is written to memory.  Over the
 // source window the step also stores mu_Pi (half nodes) and lam'_Pi (integer nodes) into
 // one slot of a ring, from which adj_src_grad_kernel forms the source gradients of many
 // steps at once, off the step's critical path.
 
-// theta_cotangent with the angular neighbours given: lm, l0, lp the Pi cotangents of
-// rows j-1, j, j+1 of column node o.
-template <typename T, typename R>
-__device__ __forceinline__ Z<R> theta_cot3(const T* tab, size_t pl, size_t o, int j, int nth, Z<R> lm,
-                                           Z<R> l0, Z<R> lp, R g) {
-    R ep0 = cget<T, R>(tab, pl, C_EP, o), em0 = cget<T, R>(tab, pl, C_EM, o);
-    Z<R> r = zconjmul(cget<T, R>(tab, pl, C_E3R, o) - ep0 - em0, cget<T, R>(tab, pl, C_E3I, o), l0);
-    if (j >= 1) r = zadd(r, zscale(cget<T, R>(tab, pl, C_EP, o - 1), lm));
-    else r = zadd(r, zscale(g * em0, l0));
-    if (j + 1 < nth) r = zadd(r, zscale(cget<T, R>(tab, pl, C_EM, o + 1), lp));
-    else r = zadd(r, zscale(g * ep0, l0));
-    return r;
+// Real arithmetic of the FP64 reverse step: every operation a DFMA (DADD and DMUL take 19
+// clocks of the SM's FP64 pipe, DFMA 16; `one` is a factor the compiler cannot see).
+struct AdjLin {
+    using Zd = Z<double>;
+    double one;
+    __device__ __forceinline__ double sum(double a, double b) const { return __fma_rn(a, one, b); }
+    __device__ __forceinline__ Zd add(Zd a, Zd b) const { return {sum(a.x, b.x), sum(a.y, b.y)}; }
+    __device__ __forceinline__ Zd sub(Zd a, Zd b) const {
+        return {__fma_rn(b.x, -one, a.x), __fma_rn(b.y, -one, a.y)};
+    }
+    // s a + b
+    __device__ __forceinline__ Zd mac(Zd b, double s, Zd a) const { return {__fma_rn(s, a.x, b.x), __fma_rn(s, a.y, b.y)}; }
+    // conj(cr + i ci) a + b
+    __device__ __forceinline__ Zd cmac(Zd b, double cr, double ci, Zd a) const {
+        return {__fma_rn(cr, a.x, __fma_rn(ci, a.y, b.x)), __fma_rn(cr, a.y, __fma_rn(-ci, a.x, b.y))};
+    }
+};
+
+// g v for g = +-1 (flip: the sign bit if g < 0), without an FP64 operation
+__device__ __forceinline__ double pole_sign(double v, int flip) {
+    return __hiloint2double(__double2hiint(v) ^ flip, __double2loint(v));
+}
+
+// b + Th^T l at row j, Th the angular and zero-order part of one sub-step, ep (F_{j+1} - F_j)
+// - em (F_j - F_{j-1}) + E3 F with the ghost rows of the pole rule (flip: pole_sign of its
+// factor); lm, l, lp: l at the rows j-1, j, j+1.
+template <typename T>
+__device__ __forceinline__ Z<double> theta_cot(const AdjLin& A, Z<double> b, const T* tab, size_t pl, size_t o, int j,
+                                               int nth, Z<double> lm, Z<double> l, Z<double> lp, int flip) {
+    const double ep = cget<T, double>(tab, pl, C_EP, o), em = cget<T, double>(tab, pl, C_EM, o);
+    const double e3 = __fma_rn(em, -A.one, __fma_rn(ep, -A.one, cget<T, double>(tab, pl, C_E3R, o)));
+    b = A.cmac(b, e3, cget<T, double>(tab, pl, C_E3I, o), l);
+    const bool lo = j >= 1, hi = j + 1 < nth;
+    b = A.mac(b, lo ? cget<T, double>(tab, pl, C_EP, o - 1) : pole_sign(em, flip), lo ? lm : l);
+    return A.mac(b, hi ? cget<T, double>(tab, pl, C_EM, o + 1) : pole_sign(ep, flip), hi ? lp : l);
 }
 
 // The co-state of one node as stored: FP64 value, or FP32 (v, c) pairs with value v - c.
@@ -251,136 +272,136 @@ __device__ __forceinline__ void adj_wait_prev() { asm volatile("griddepcontrol.w
 // kMaxT: the largest block this instance serves (256: columns of up to 256 rows, with
 // the register budget of several blocks per SM; 512: up to 512 rows, one block per SM;
 // 1024: taller columns)
-template <typename T, typename R, int kMaxT>
+//
+// The FP64 co-state (FP64 and double-float instances).  Bound by the FP64 pipe, so the
+// cotangents of the undivided sums of the forward step (predict_x, correct_x) are formed
+// once a node and once a half node and shared by the two neighbours they enter:
+//   node i, l = lam':       cS = Th^T l_Pi, cD = -G l_Phi + conj(E2) l_Pi,
+//                           cSP = (dt/4) l_Phi + conj(E1) l_Pi, cDP = G l_Pi
+//     mu_Phi += cS +- cD, mu_Pi += cSP +- cDP  at the half nodes right (+) and left (-) of i
+//   half node h, mu:        cs = mu_Phi + Th^T mu_Pi, cd = -G mu_Phi + conj(E2) mu_Pi,
+//                           csP = (dt/2) mu_Phi + mu_Pi + conj(E1) mu_Pi, cdP = G mu_Pi
+//     lam_Phi += cs +- cd, lam_Pi += csP +- cdP  at the nodes right (+) and left (-) of h
+// 76 FP64 operations a node instead of 190 (4096 x 128: 195 -> 111 us a reverse step, double-float
+// instances 360 -> 204).  mu here is the cotangent of
+// 2 h, so the source window gets 2 mu_Pi.
+template <typename T, int kMaxT>
 __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin, const double2* gbar,
                                                          CoLevel lout, int strip, void* wh, void* wi) {
+    using Zd = Z<double>;
     extern __shared__ __align__(16) unsigned char adj_smem[];
     adj_release_next();
-    Z<R>* LB = (Z<R>*)adj_smem;                 // [2][pitch] lam'_Pi of a column
-    Z<R>* MB = LB + 2 * (size_t)d.pitch;        // [2][pitch] mu_Pi of a half node
+    Zd* LB = (Zd*)adj_smem;                    // [2][pitch] lam'_Pi of a column
+    Zd* MB = LB + 2 * (size_t)d.pitch;         // [2][pitch] mu_Pi of a half node
     const int j = threadIdx.x, nth = d.nth, nr = d.nr, pitch = d.pitch;
     const bool row_ok = j < nth;
     const int c0 = blockIdx.x * strip, c1 = min(nr, c0 + strip);   // output columns [c0, c1)
     const T* ci = (const T*)d.coef_i;
     const T* ch = (const T*)d.coef_h;
     const size_t pl = plane_elems(d);
-    const R g = (R)d.ghost, hdt = (R)(0.5 * d.dt);
-    constexpr bool kComp = sizeof(R) == 4;
+    const double hdt = 0.5 * d.dt, qdt = 0.25 * d.dt, w_e = 1.0 - d.f_e, w_e1 = d.f_e;
+    const int flip = d.ghost < 0.0 ? (int)0x80000000 : 0;
+    const AdjLin A{d.one};
     const SourceDev& s = d.src;
+    const Zd zero = {0, 0};
     // wh, wi: this step's ring slot of the window co-states (null: no source)
     // lam' = P lam^{n+1} at column col (zero at the boundary columns and outside)
     auto lam_at = [&](int col) {
-        CoNode<R> z{};
-        if (row_ok && col >= 1 && col <= nr - 2) z = co_load<R>(lin, node_index(d, col, j));
+        CoNode<double> z{};
+        if (row_ok && col >= 1 && col <= nr - 2) z = co_load<double>(lin, node_index(d, col, j));
         return z;
     };
-    auto nb3 = [&](const Z<R>* buf, int sl, Z<R>& lm, Z<R>& lp) {
-        const Z<R>* b = buf + (size_t)sl * pitch;
-        lm = j >= 1 ? b[j - 1] : Z<R>{0, 0};
-        lp = j + 1 < nth ? b[j + 1] : Z<R>{0, 0};
+    auto nb3 = [&](const Zd* buf, int sl, Zd& lm, Zd& lp) {
+        const Zd* b = buf + (size_t)sl * pitch;
+        lm = j >= 1 ? b[j - 1] : zero;
+        lp = j + 1 < nth ? b[j + 1] : zero;
+    };
+    // shares of node col (co-state L, its Pi part exchanged) of the half nodes to its right
+    // (rF, rP) and left (lF, lP)
+    auto node_shares = [&](const CoNode<double>& L, int col, Zd& rF, Zd& rP, Zd& lF, Zd& lP) {
+        rF = rP = lF = lP = zero;
+        if (!row_ok || col < 1 || col > nr - 2) return;
+        const size_t o = node_index(d, col, j);
+        Zd lm, lp;
+        nb3(LB, col & 1, lm, lp);
+        const double G = cget<T, double>(ci, pl, C_G, o);
+        const Zd cS = theta_cot<T>(A, zero, ci, pl, o, j, nth, lm, L.P, lp, flip);
+        const Zd cD = A.cmac(A.mac(zero, -G, L.F), cget<T, double>(ci, pl, C_E2R, o), cget<T, double>(ci, pl, C_E2I, o), L.P);
+        const Zd cSP = A.cmac(A.mac(zero, qdt, L.F), cget<T, double>(ci, pl, C_E1R, o), cget<T, double>(ci, pl, C_E1I, o), L.P);
+        const Zd cDP = A.mac(zero, G, L.P);
+        rF = A.add(cS, cD);
+        lF = A.sub(cS, cD);
+        rP = A.add(cSP, cDP);
+        lP = A.sub(cSP, cDP);
     };
     adj_wait_prev();
-    CoNode<R> l_cur = lam_at(c0 - 1), l_next;
+    // prologue: column c0 - 1
+    CoNode<double> l_cur = lam_at(c0 - 1), l_next;
     LB[(size_t)((c0 - 1) & 1) * pitch + j] = l_cur.P;
-    Z<R> mu_prevF = {0, 0}, mu_prevP = {0, 0};
+    __syncthreads();
+    Zd muF_part, muP_part, aF_part = zero, aP_part = zero, x, y;
+    node_shares(l_cur, c0 - 1, muF_part, muP_part, x, y);
     for (int h = c0 - 1; h <= c1 - 1; ++h) {
-        // A: lam' of column h+1
+        // column h+1: lam' and its shares; mu at half node h
         l_next = lam_at(h + 1);
         LB[(size_t)((h + 1) & 1) * pitch + j] = l_next.P;
         __syncthreads();
-        // C: mu at half node h = C^T lam' from the integer columns h (right neighbour of
-        // this half node, sign +1) and h+1 (left neighbour, sign -1)
-        Z<R> muF = {0, 0}, muP = {0, 0};
-        if (row_ok && h >= 0 && h <= nr - 2) {
-            for (int side = 0; side < 2; ++side) {
-                const int col = h + side;
-                if (col < 1 || col > nr - 2) continue;
-                const R sR = side == 0 ? R(1) : R(-1);
-                const size_t o = node_index(d, col, j);
-                const CoNode<R>& L = side == 0 ? l_cur : l_next;
-                Z<R> lm, lp;
-                nb3(LB, col & 1, lm, lp);
-                const R G = cget<T, R>(ci, pl, C_G, o);
-                const Z<R> tc = theta_cot3<T, R>(ci, pl, o, j, nth, lm, L.P, lp, g);
-                muF = zadd(muF, zscale(-sR * G, L.F));
-                muF = zadd(muF, zscale(sR, zconjmul(cget<T, R>(ci, pl, C_E2R, o), cget<T, R>(ci, pl, C_E2I, o), L.P)));
-                muF = zadd(muF, zscale(R(0.5), tc));
-                muP = zadd(muP, zscale((R)(0.5 * d.dt), L.F));
-                muP = zadd(muP, zscale(sR * G, L.P));
-                muP = zadd(muP, zscale(R(0.5), zconjmul(cget<T, R>(ci, pl, C_E1R, o), cget<T, R>(ci, pl, C_E1I, o), L.P)));
-            }
-            if (wh && h >= c0) {   // half-node window: mu_Pi (half node c0 - 1 is the
-                                   // previous block's)
-                const int a = h - s.h_lo, bb = j - s.j_lo;
-                if ((unsigned)a < (unsigned)s.nh && (unsigned)bb < (unsigned)s.nj)
-                    stv<R>(wh, (size_t)bb * s.nh + a, muP);
-            }
+        Zd muF_next, muP_next, muF, muP;
+        node_shares(l_next, h + 1, muF_next, muP_next, muF, muP);
+        const bool half_ok = row_ok && h >= 0 && h <= nr - 2;
+        muF = half_ok ? A.add(muF_part, muF) : zero;
+        muP = half_ok ? A.add(muP_part, muP) : zero;
+        if (wh && half_ok && h >= c0) {   // half-node window: the cotangent of h_Pi (half node c0 - 1 is
+                                          // the previous block's)
+            const int a = h - s.h_lo, bb = j - s.j_lo;
+            if ((unsigned)a < (unsigned)s.nh && (unsigned)bb < (unsigned)s.nj)
+                stv<double>(wh, (size_t)bb * s.nh + a, A.add(muP, muP));
         }
         MB[(size_t)(h & 1) * pitch + j] = muP;
         __syncthreads();
-        // F: lam^n at integer column h from the half nodes h-1 (this column is their right
-        // input, sign +1) and h (left input, sign -1)
+        // the shares of half node h of the nodes h (left) and h+1 (right)
+        Zd tF = zero, tP = zero, nF = zero, nP = zero;
+        if (half_ok) {
+            const size_t oh = node_index(d, h, j);
+            Zd mm, mp;
+            nb3(MB, h & 1, mm, mp);
+            const double G = cget<T, double>(ch, pl, C_G, oh);
+            const Zd cs = theta_cot<T>(A, muF, ch, pl, oh, j, nth, mm, muP, mp, flip);
+            const Zd cd = A.cmac(A.mac(zero, -G, muF), cget<T, double>(ch, pl, C_E2R, oh), cget<T, double>(ch, pl, C_E2I, oh), muP);
+            const Zd csP = A.cmac(A.mac(muP, hdt, muF), cget<T, double>(ch, pl, C_E1R, oh), cget<T, double>(ch, pl, C_E1I, oh), muP);
+            tF = A.sub(cs, cd);
+            nF = A.add(cs, cd);
+            tP = A.mac(csP, -G, muP);
+            nP = A.mac(csP, G, muP);
+        }
+        // lam^n at column h
         if (h >= c0 && row_ok) {
-            const int i = h;
-            const size_t o = node_index(d, i, j);
-            const bool interior = i >= 1 && i <= nr - 2;
-            Z<R> aF = {0, 0}, aP = {0, 0};
-            if constexpr (!kComp) {
-                if (interior) {
-                    aF = l_cur.F;
-                    aP = l_cur.P;
-                }
-            }
-            for (int side = 0; side < 2; ++side) {
-                const int hh = i - 1 + side;
-                if (hh < 0 || hh > nr - 2) continue;
-                const R sR = side == 0 ? R(1) : R(-1);
-                const size_t oh = node_index(d, hh, j);
-                const Z<R> MF = side == 0 ? mu_prevF : muF, MP = side == 0 ? mu_prevP : muP;
-                Z<R> mm, mp;
-                nb3(MB, hh & 1, mm, mp);
-                const R G = cget<T, R>(ch, pl, C_G, oh);
-                const Z<R> tc = theta_cot3<T, R>(ch, pl, oh, j, nth, mm, MP, mp, g);
-                aF = zadd(aF, zscale(R(0.5) - sR * G, MF));
-                aF = zadd(aF, zscale(sR, zconjmul(cget<T, R>(ch, pl, C_E2R, oh), cget<T, R>(ch, pl, C_E2I, oh), MP)));
-                aF = zadd(aF, zscale(R(0.5), tc));
-                aP = zadd(aP, zscale(R(0.5) * hdt, MF));
-                aP = zadd(aP, zscale(R(0.5) + sR * G, MP));
-                aP = zadd(aP, zscale(R(0.5), zconjmul(cget<T, R>(ch, pl, C_E1R, oh), cget<T, R>(ch, pl, C_E1I, oh), MP)));
+            const size_t o = node_index(d, h, j);
+            const bool interior = h >= 1 && h <= nr - 2;
+            Zd aF = A.add(aF_part, tF), aP = A.add(aP_part, tP);
+            if (interior) {
+                aF = A.add(l_cur.F, aF);
+                aP = A.add(l_cur.P, aP);
             }
             if (gbar) {   // transpose of the linear extraction between i_e and i_e + 1
-                if (i == d.i_e) aF = zadd(aF, zscale((R)(1.0 - d.f_e), gld<R>(gbar, j)));
-                if (i == d.i_e + 1) aF = zadd(aF, zscale((R)d.f_e, gld<R>(gbar, j)));
+                if (h == d.i_e) aF = zadd(aF, zscale(w_e, gld<double>(gbar, j)));
+                if (h == d.i_e + 1) aF = zadd(aF, zscale(w_e1, gld<double>(gbar, j)));
             }
-            if constexpr (kComp) {
-                float2 vF = {0.f, 0.f}, cF = {0.f, 0.f}, vP = {0.f, 0.f}, cP = {0.f, 0.f};
-                if (interior) {
-                    vF = l_cur.vF;
-                    cF = l_cur.cF;
-                    vP = l_cur.vP;
-                    cP = l_cur.cP;
-                }
-                kahan_node(vF, cF, aF);
-                kahan_node(vP, cP, aP);
-                if (TK_IN(d.status, o, pl)) {
-                    ((float2*)lout.F)[o] = vF;
-                    ((float2*)lout.Fc)[o] = cF;
-                    ((float2*)lout.P)[o] = vP;
-                    ((float2*)lout.Pc)[o] = cP;
-                }
-            } else if (TK_IN(d.status, o, pl)) {
-                stv<R>(lout.F, o, aF);
-                stv<R>(lout.P, o, aP);
+            if (TK_IN(d.status, o, pl)) {
+                stv<double>(lout.F, o, aF);
+                stv<double>(lout.P, o, aP);
             }
             if (wi) {   // integer-node window: lam'_Pi (zero off the interior columns)
-                const int a = i - s.i_lo, bb = j - s.j_lo;
+                const int a = h - s.i_lo, bb = j - s.j_lo;
                 if ((unsigned)a < (unsigned)s.ni && (unsigned)bb < (unsigned)s.nj)
-                    stv<R>(wi, (size_t)bb * s.ni + a, interior ? l_cur.P : Z<R>{0, 0});
+                    stv<double>(wi, (size_t)bb * s.ni + a, interior ? l_cur.P : zero);
             }
         }
         l_cur = l_next;
-        mu_prevF = muF;
-        mu_prevP = muP;
+        muF_part = muF_next;
+        muP_part = muP_next;
+        aF_part = nF;
+        aP_part = nP;
     }
 }
 
@@ -660,13 +681,13 @@ static void adj_dispatch(int prec, int t, F f) {
     if (prec == 0 || prec == 3) {
         const size_t sm = adj_smem<double>(t, false);
         if (prec == 0) {
-            if (t <= 256) f(adj_step_kernel<double, double, 256>, sm);
-            else if (t <= 512) f(adj_step_kernel<double, double, 512>, sm);
-            else f(adj_step_kernel<double, double, 1024>, sm);
+            if (t <= 256) f(adj_step_kernel<double, 256>, sm);
+            else if (t <= 512) f(adj_step_kernel<double, 512>, sm);
+            else f(adj_step_kernel<double, 1024>, sm);
         } else {
-            if (t <= 256) f(adj_step_kernel<DF, double, 256>, sm);
-            else if (t <= 512) f(adj_step_kernel<DF, double, 512>, sm);
-            else f(adj_step_kernel<DF, double, 1024>, sm);
+            if (t <= 256) f(adj_step_kernel<DF, 256>, sm);
+            else if (t <= 512) f(adj_step_kernel<DF, 512>, sm);
+            else f(adj_step_kernel<DF, 1024>, sm);
         }
     } else {
         const size_t sm = adj_smem<float>(t, true);

@@ -262,6 +262,7 @@ InstDev dev_of(const teuk_ctx* c, const Instance& I) {
     // behaviour theta^|m+s| of the spin-weighted harmonics, the paper's rule for even s
     d.ghost = (std::abs(I.p.m + I.p.s) % 2 == 0) ? 1.0 : -1.0;
     d.ghost_f = (float)d.ghost;
+    d.one = 1.0;
     for (int b = 0; b < 2; ++b)
         for (int k = 0; k < 2; ++k) d.buf[b][k] = I.state[b][k];
     d.coef_h = I.coef_h;

@@ -24,14 +24,15 @@ namespace teuk {
 constexpr int kNCoef = 9;        // coefficients per node and sub-step
 constexpr int kPitchAlign = 32;  // elements
 
-// Coefficient planes (same order at half and integer nodes; "s" is 1/2 for the
-// predictor and 1 for the corrector, i.e. the fraction of dt of the sub-step):
-//   0: g    = s dt b / dr*                       (D term of Eqs. 13-14)
-//   1,2: E1 = -s dt c_t                          (Pi coefficient of S_Pi)
-//   3,4: E2 = s dt P* / dr*,  P* = c_t b + p* - b b_{,r*}
-//   5:   ep = s dt w (1/dth^2 + cot/(2 dth))     (forward theta difference)
-//   6:   em = s dt w (1/dth^2 - cot/(2 dth))     (backward theta difference)
-//   7,8: E3 = s dt (q - w V)                     (zero-order term)
+// Coefficient planes (same order at half and integer nodes; sd is dt/2 for the predictor
+// and dt/4 for the corrector, kd is dt and dt/2: the sub-step's time step with the powers
+// of two of the undivided half-node sums folded in, see predict_x and correct_x):
+//   0: G    = kd b / dr*                         (D term of Eqs. 13-14)
+//   1,2: E1 = -sd c_t                            (Pi coefficient of S_Pi)
+//   3,4: E2 = kd P* / dr*,  P* = c_t b + p* - b b_{,r*}
+//   5:   ep = sd w (1/dth^2 + cot/(2 dth))       (forward theta difference)
+//   6:   em = sd w (1/dth^2 - cot/(2 dth))       (backward theta difference)
+//   7,8: E3 = sd (q - w V)                       (zero-order term)
 enum CoefIdx { C_G = 0, C_E1R, C_E1I, C_E2R, C_E2I, C_EP, C_EM, C_E3R, C_E3I };
 
 struct SourceDev {
@@ -87,6 +88,7 @@ struct InstDev {
     double drs, dth, dt;
     float ghost_f;            // +1 even |m + s|, -1 odd |m + s|
     double ghost;
+    double one;               // 1.0, as a value the compiler does not know (see Lin)
     void* buf[2][2];          // [ping-pong buffer][plane]
     const void* coef_h;       // [9][nr][pitch] (double or float)
     const void* coef_i;

@@ -113,13 +113,15 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
     const int jp = j + 1 < nth ? j + 1 : j, jm = j > 0 ? j - 1 : 0;
     const T g = (T)d.ghost;
     const T gp = top ? g : T(1), gm = bot ? g : T(1);
-    const T hdt = (T)(0.5 * d.dt), fdt = (T)d.dt;
+    const T hdt = (T)(0.5 * d.dt), fdt = (T)d.dt, qdt = (T)(0.25 * d.dt);
+    const Lin<T> A(d);
     const bool has_l = b > 0, has_r = b < r.nb - 1;
 
     using L = ResLayout<P>;
     unsigned char* sm = res_smem;
     const Planes<P> S = Planes<P>::at(sm, (unsigned)(ncol * pitch));
     HalfRec<T>* HR = (HalfRec<T>*)(sm + L::s_bytes(ncol, pitch));
+    HalfX<T>* HX = (HalfX<T>*)HR;   // expanded form (the smaller record in the same place)
     T* X = (T*)(sm + L::s_bytes(ncol, pitch) + L::hr_bytes(ncol, pitch));
     T* CF = (T*)(sm + L::s_bytes(ncol, pitch) + L::hr_bytes(ncol, pitch) + L::x_bytes(ncol, pitch));
     auto sidx = [&](int q, int jj) { return (size_t)q * pitch + jj; };
@@ -192,7 +194,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
         const int q = t - w1;
         if (!src_blk || q < 0 || q >= 2 * hs) return;
         const double2 f = (q & 1) ? source_factor<false>(d, step + q / 2, 0.5, d.dt)
-                                  : source_factor<false>(d, step + q / 2, 0.0, 0.5 * d.dt);
+                                  : source_factor<false>(d, step + q / 2, 0.0, kSplit ? 0.5 * d.dt : d.dt);
         sfac[ip][q / 2][2 * (q & 1)] = (T)f.x;
         sfac[ip][q / 2][2 * (q & 1) + 1] = (T)f.y;
     };
@@ -268,65 +270,93 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
             // P1: predictor (Eq. 13)
             for (int k = k0; k < nk; k += KT) {
                 if (!pact(k)) continue;
-                const int col = c0 - h + k;
-                const NodeV<P> ul = S.load(sidx(k, j)), ur = S.load(sidx(k + 1, j));
-                C dll, dlml, dlr, dlmr;
-                {
-                    const NodeV<P> dn = S.load_phi(sidx(k, jp)), upn = S.load_phi(sidx(k, jm));
-                    if constexpr (kSplit) {
+                if constexpr (kSplit) {
+                    const int col = c0 - h + k;
+                    const NodeV<P> ul = S.load(sidx(k, j)), ur = S.load(sidx(k + 1, j));
+                    C dll, dlml, dlr, dlmr;
+                    {
+                        const NodeV<P> dn = S.load_phi(sidx(k, jp)), upn = S.load_phi(sidx(k, jm));
                         ul.theta_split(gp, dn, gm, upn, dll, dlml);
-                    } else {
-                        dll = dn.dphi_sl(gp, ul);
-                        dlml = ul.dphi_sr(gm, upn);
                     }
-                }
-                {
-                    const NodeV<P> dn = S.load_phi(sidx(k + 1, jp)), upn = S.load_phi(sidx(k + 1, jm));
-                    if constexpr (kSplit) {
+                    {
+                        const NodeV<P> dn = S.load_phi(sidx(k + 1, jp)), upn = S.load_phi(sidx(k + 1, jm));
                         ur.theta_split(gp, dn, gm, upn, dlr, dlmr);
-                    } else {
-                        dlr = dn.dphi_sl(gp, ur);
-                        dlmr = ur.dphi_sr(gm, upn);
                     }
-                }
-                C s_h = C::zero();
-                if (src_blk) s_h = source_half<T>(sw, C{sfac[ip][s][0], sfac[ip][s][1]}, col, j);
-                T cf[kNCoef];
+                    C s_h = C::zero();
+                    if (src_blk) s_h = source_half<T>(sw, C{sfac[ip][s][0], sfac[ip][s][1]}, col, j);
+                    T cf[kNCoef];
 #pragma unroll
-                for (int q = 0; q < kNCoef; ++q) cf[q] = CF[sidx(k, j) * 2 * kNCoef + q];
-                const Half<T> hp = half_prep<P>(ul, ur);
-                const C Dp = C::half_sum(dll, dlr);
-                const C Dm = C::half_sum(dlml, dlmr);
-                HR[sidx(k, j)] = predictor<T, kSplit>(hp, Dp, Dm, cf, hdt, s_h);
+                    for (int q = 0; q < kNCoef; ++q) cf[q] = CF[sidx(k, j) * 2 * kNCoef + q];
+                    const Half<T> hp = half_prep<P>(ul, ur);
+                    const C Dp = C::half_sum(dll, dlr);
+                    const C Dm = C::half_sum(dlml, dlmr);
+                    HR[sidx(k, j)] = predictor<T>(hp, Dp, Dm, cf, hdt, s_h);
+                } else {
+                    // the sums of the rows above and below, as those rows form them
+                    const NodeV<P> ul = S.load(sidx(k, j)), ur = S.load(sidx(k + 1, j));
+                    const C sm = A.add(ul.F, ur.F);
+                    C s_p = A.add(S.load_phi(sidx(k, jp)).F, S.load_phi(sidx(k + 1, jp)).F);
+                    C s_m = A.add(S.load_phi(sidx(k, jm)).F, S.load_phi(sidx(k + 1, jm)).F);
+                    if (top) s_p = g * s_p;
+                    if (bot) s_m = g * s_m;
+                    T cf[kNCoef];
+#pragma unroll
+                    for (int q = 0; q < kNCoef; ++q) cf[q] = CF[sidx(k, j) * 2 * kNCoef + q];
+                    C s_h = C::zero();
+                    if (src_blk) s_h = source_half<T>(sw, C{sfac[ip][s][0], sfac[ip][s][1]}, c0 - h + k, j);
+                    HX[sidx(k, j)] = predict_x<T, true>(A, ul.F, ul.Pp, ur.F, ur.Pp, sm, s_p, s_m, cf, hdt, s_h);
+                }
             }
             __syncthreads();
             // P2: combine the half nodes on both sides of node k, publish the exchange entry
             for (int k = k0; k < nk; k += KT) {
                 if (!cact(k)) continue;
-                const HalfRec<T> Rh = HR[sidx(k, j)], Lh = HR[sidx(k - 1, j)];
-                const CRow<T> row = combine_lr<T, kSplit>(Rh, Lh);
-                T* xb = X + (size_t)k * (pitch + 2) * 4;
-                xpublish<P, kSplit>(xb, xb + 4 * (j + 1), row, Rh, Lh, g, row_ok, top, bot);
+                if constexpr (kSplit) {
+                    const HalfRec<T> Rh = HR[sidx(k, j)], Lh = HR[sidx(k - 1, j)];
+                    const CRow<T> row = combine_lr<T>(Rh, Lh);
+                    T* xb = X + (size_t)k * (pitch + 2) * 4;
+                    xpublish(xb, xb + 4 * (j + 1), row, g, row_ok, top, bot);
+                } else {
+                    unsigned char* xb = (unsigned char*)(X + (size_t)k * (pitch + 2) * 4);
+                    publish16<T>(xb, j, A.add(HX[sidx(k, j)].F, HX[sidx(k - 1, j)].F), g, row_ok, top, bot);
+                }
             }
             __syncthreads();
             // P3: corrector (Eq. 14) at node k, in place (this step's state is no longer read)
             for (int k = k0; k < nk; k += KT) {
                 const int col = c0 - h + k;
                 if (cact(k) && row_ok) {
-                    const HalfRec<T> Rh = HR[sidx(k, j)], Lh = HR[sidx(k - 1, j)];
-                    const CRow<T> row = combine_lr<T, kSplit>(Rh, Lh);
-                    C Hs_p, Hs_m, DpS_m;
-                    xread<P, kSplit>(X + (size_t)k * (pitch + 2) * 4 + 4 * (j + 1), Hs_p, Hs_m, DpS_m);
-                    C s_i = C::zero();
-                    if (src_blk) s_i = source_int<T>(sw, C{sfac[ip][s][2], sfac[ip][s][3]}, col, j);
-                    T cf[kNCoef];
+                    if constexpr (kSplit) {
+                        const HalfRec<T> Rh = HR[sidx(k, j)], Lh = HR[sidx(k - 1, j)];
+                        const CRow<T> row = combine_lr<T>(Rh, Lh);
+                        C Hs_p, Hs_m;
+                        xread(X + (size_t)k * (pitch + 2) * 4 + 4 * (j + 1), Hs_p, Hs_m);
+                        C s_i = C::zero();
+                        if (src_blk) s_i = source_int<T>(sw, C{sfac[ip][s][2], sfac[ip][s][3]}, col, j);
+                        T cf[kNCoef];
 #pragma unroll
-                    for (int q = 0; q < kNCoef; ++q) cf[q] = CF[sidx(k, j) * 2 * kNCoef + kNCoef + q];
-                    C dPhi, dPi;
-                    corrector_incr<P, kSplit>(row, Hs_p, Hs_m, DpS_m, cf, fdt, s_i, dPhi, dPi);
-                    NodeV<P> u = S.load(sidx(k, j));
-                    u.update(dPhi, dPi);
-                    S.store(sidx(k, j), u);
+                        for (int q = 0; q < kNCoef; ++q) cf[q] = CF[sidx(k, j) * 2 * kNCoef + kNCoef + q];
+                        C dPhi, dPi;
+                        corrector_incr<P>(row, Hs_p, Hs_m, cf, fdt, s_i, dPhi, dPi);
+                        NodeV<P> u = S.load(sidx(k, j));
+                        u.update(dPhi, dPi);
+                        S.store(sidx(k, j), u);
+                    } else {
+                        const HalfX<T> Rh = HX[sidx(k, j)], Lh = HX[sidx(k - 1, j)];
+                        const unsigned char* xb = (const unsigned char*)(X + (size_t)k * (pitch + 2) * 4);
+                        const C S_p = get16<T>(xb + 16 * (j + 2)), S_m = get16<T>(xb + 16 * j);
+                        C s_i = C::zero();
+                        if (src_blk) s_i = source_int<T>(sw, C{sfac[ip][s][2], sfac[ip][s][3]}, col, j);
+                        T cf[kNCoef];
+#pragma unroll
+                        for (int q = 0; q < kNCoef; ++q) cf[q] = CF[sidx(k, j) * 2 * kNCoef + kNCoef + q];
+                        C dPhi, dPi;
+                        correct_x<T, true>(A, Rh, Lh, A.add(Rh.F, Lh.F), S_p, S_m, cf, qdt, s_i, dPhi, dPi);
+                        NodeV<P> u = S.load(sidx(k, j));
+                        u.F = A.add(u.F, dPhi);
+                        u.Pp = A.add(u.Pp, dPi);
+                        S.store(sidx(k, j), u);
+                    }
                 }
                 // radial boundary condition: Phi = Pi = 0 at columns 0 and nr - 1
                 if (row_ok && k >= s && k < nk - s) {

@@ -60,10 +60,12 @@ __global__ void invert_tortoise_kernel(double M, double a, double rstar_min, dou
 
 struct Cplx { double re, im; };
 
-// The nine scaled coefficients (order of CoefIdx) of a sub-step that spans the
-// fraction sfrac of dt, at (r = r_+ + x, theta).
+// The nine scaled coefficients (order of CoefIdx) of a sub-step, at (r = r_+ + x, theta):
+// sd = sfrac dt scales the terms that act on sums, kd = kfrac dt those on radial
+// differences (teuk_internal.cuh).
 __device__ void node_coefficients(double M, double a, int s_, int m_, double x, double th,
-                                  double dth, double dt, double drs, double sfrac, double* out) {
+                                  double dth, double dt, double drs, double sfrac, double kfrac,
+                                  double* out) {
     double d = sqrt(M * M - a * a);
     double rp = M + d, rm = M - d;
     double s = (double)s_, m = (double)m_;
@@ -87,13 +89,13 @@ __device__ void node_coefficients(double M, double a, int s_, int m_, double x, 
     Cplx Pst = {ct.re * b + pst.re - bbr, ct.im * b + pst.im};
     double V = (m + s * cs) * (m + s * cs) / sn2 - s;
     double cot = cs / sn;
-    double sdt = sfrac * dt;
+    const double sdt = sfrac * dt, kdt = kfrac * dt;
     double i2 = 1.0 / (dth * dth), i1 = cot / (2.0 * dth);
-    out[C_G] = sdt * b / drs;
+    out[C_G] = kdt * b / drs;
     out[C_E1R] = -sdt * ct.re;
     out[C_E1I] = -sdt * ct.im;
-    out[C_E2R] = sdt * Pst.re / drs;
-    out[C_E2I] = sdt * Pst.im / drs;
+    out[C_E2R] = kdt * Pst.re / drs;
+    out[C_E2I] = kdt * Pst.im / drs;
     out[C_EP] = sdt * w * (i2 + i1);
     out[C_EM] = sdt * w * (i2 - i1);
     out[C_E3R] = sdt * (q.re - w * V);
@@ -112,13 +114,13 @@ __global__ void coef_kernel(double M, double a, int s, int m, double rstar_min, 
     double th = (j + 0.5) * dth;
     double c[kNCoef];
     if (j < nth && i < nr - 1) {
-        node_coefficients(M, a, s, m, x_half[i], th, dth, dt, drs, 0.5, c);
+        node_coefficients(M, a, s, m, x_half[i], th, dth, dt, drs, 0.5, 1.0, c);
         for (int k = 0; k < kNCoef; ++k) coef_h[k * pl + o] = (T)c[k];
     } else {
         for (int k = 0; k < kNCoef; ++k) coef_h[k * pl + o] = (T)0;
     }
     if (j < nth) {
-        node_coefficients(M, a, s, m, x_int[i], th, dth, dt, drs, 1.0, c);
+        node_coefficients(M, a, s, m, x_int[i], th, dth, dt, drs, 0.25, 0.5, c);
         for (int k = 0; k < kNCoef; ++k) coef_i[k * pl + o] = (T)c[k];
     } else {
         for (int k = 0; k < kNCoef; ++k) coef_i[k * pl + o] = (T)0;

@@ -14,9 +14,13 @@
 // (even |m + s|) or -1 (odd |m + s|): on the averaged state in the predictor, on the half-node
 // results in the corrector.
 //
-// Arithmetic, in differences so that the compensated FP32 state keeps its accuracy (a
-// difference of two (hi, c) pairs is formed as (hi_a - hi_b) - (c_a - c_b) before
-// anything cancels):
+// The FP64 and double-float kernels take the expanded form of teuk_step_common.cuh
+// (predict_x, correct_x), in which the rows exchange the radial sums s of the next half
+// node as well as S, so that no row reads another row's slot entries.
+//
+// Arithmetic of the FP32 paths, in differences so that the compensated FP32 state keeps its
+// accuracy (a difference of two (hi, c) pairs is formed as (hi_a - hi_b) - (c_a - c_b)
+// before anything cancels):
 //   predictor at (i+1/2, j), with Fb = (Phi_i + Phi_{i+1})/2, dF = Phi_{i+1} - Phi_i,
 //   Dp(j) = Fb(j+1) - Fb(j) and the same for Pi:
 //     dh_Phi = -g dF + (dt/2) Pb
@@ -26,7 +30,7 @@
 //     Delta Phi = -g d(h_Phi) + dt Pi~
 //     Delta Pi  =  g d(h_Pi) + E1 Pi~ + E2 d(h_Phi) + ep D+ - em D- + E3 Phi~ + dt tau(t_n+dt/2)
 //     u^{n+1} = u^n + Delta   (Kahan-compensated for the FP32_KAHAN state)
-// with the scaled coefficients g, E1, E2, ep, em, E3 of teuk_setup.cu (the two
+// with the scaled coefficients g, E1, E2, ep, em, E3 (see RTab2; the two
 // sub-steps differ only by the factor 1/2 versus 1 of dt).  This is Eqs. (13)-(14)
 // with S_Pi = -c_t Pi + P* Phi_* + w Theta[Phi] + q Phi + tau, rearranged, not
 // approximated.  The FP32 paths write the angular part ep D+ - em D- in the split form
@@ -211,6 +215,130 @@ struct StepShared {
 // slots are up to four times bigger than those of 256 rows).
 constexpr int kRingS = 6, kRingL = 4;
 
+// Waveform record of the level in buffer bin between columns i_e and i_e + 1, one row a
+// thread, read from the buffer itself.
+template <class P>
+__device__ __forceinline__ void record_level(const InstDev& d, int64_t step, int bin) {
+    const int j = threadIdx.x;
+    const Planes<P> in = Planes<P>::of(d, bin);
+    const size_t wi = (size_t)(step % d.wave_cap) * d.nth + j;
+    if (j >= d.nth || !TK_IN(d.status, d.i_e, d.nr - 1) || !TK_IN(d.status, wi, d.wave_cap * d.nth)) return;
+    const double2 w = wave_lerp(in.load(node_index(d, d.i_e, j)).phi64(),
+                                in.load(node_index(d, d.i_e + 1, j)).phi64(), d.f_e);
+    d.wave[wi] = w;
+    if (!isfinite(w.x) || !isfinite(w.y)) atomicOr(d.status, (unsigned)ST_NONFINITE);
+}
+
+// Columns of a work item in the expanded form (FP64, double-float), after the ring's first
+// fills.  At column c the half-node sum s of c-1/2 has been exchanged already: predictor at
+// c-1/2, S published together with the next half node's s (from column c+1, awaited here),
+// one barrier, corrector at c-1.  A slot is read by its own rows only and is refilled after
+// the next barrier, R columns ahead.  has_src: source terms meet this block; moving: from
+// the moving particle's tables.
+template <class P, int R, bool kMov, class SH, class SI, class MH, class MI>
+__device__ __forceinline__ void strip_columns_x(const InstDev& d, int64_t step, int bin, int c0, int c1,
+                                                ColumnRing<P, R>& ring, unsigned char* xb, bool has_src, bool moving,
+                                                SH src_h, SI src_i, MH msrc_h, MI msrc_i) {
+    using T = typename P::T;
+    using C = Cx<T>;
+    const Lin<T> A(d);
+    const int j = threadIdx.x, nth = d.nth;
+    const bool row_ok = j < nth, bot = j == 0, top = j == nth - 1;
+    const T g = (T)d.ghost, hdt = (T)(0.5 * d.dt), qdt = (T)(0.25 * d.dt);
+    const Planes<P> out = Planes<P>::of(d, 1 - bin);
+    // exchange entries: [column parity][S, s][threads + 2] of 16 bytes
+    const unsigned xs = 16u * (blockDim.x + 2u);
+    auto xS = [&](int c) { return xb + (c & 1) * 2u * xs; };
+    auto xs_ = [&](int c) { return xb + (c & 1) * 2u * xs + xs; };
+    auto nbr = [&](const unsigned char* x, C& p, C& m) {
+        p = get16<T>(x + 16 * (j + 2));
+        m = get16<T>(x + 16 * j);
+    };
+    auto node = [&](int slot) { return ring.planes(slot).load((size_t)j); };
+    // refill the slot that column col has left with column col + R
+    auto refill = [&](int col, int slot) {
+        if (threadIdx.x == 0 && col + R <= c1) ring.fill(d, bin, col + R, slot);
+    };
+    auto coefs = [&](bool half, int col, T* cf) {
+        if (!TK_IN(d.status, col, d.nr)) return;
+        if constexpr (P::kind == kDF) coefs_df(d, half, col, j, (DF*)cf);
+        else coefs64(d, half, col, j, (double*)cf);
+    };
+    auto term_h = [&](int h) { return kMov && moving ? msrc_h(h) : src_h(h); };
+    auto term_i = [&](int i) { return kMov && moving ? msrc_i(i) : src_i(i); };
+
+    // prologue: columns c0-1, c0, c0+1 in slots 0, 1, 2; the sums of c0-1/2 and c0+1/2
+    ring.wait(0);
+    NodeV<P> u_prev = node(0);
+    ring.wait(1);
+    NodeV<P> u_cur = node(1);
+    ring.wait(2);
+    NodeV<P> u_next = node(2);
+    C s0 = A.add(u_prev.F, u_cur.F), s = A.add(u_cur.F, u_next.F);
+    publish16<T>(xS(c0), j, s0, g, row_ok, top, bot);
+    publish16<T>(xs_(c0), j, s, g, row_ok, top, bot);
+    __syncthreads();
+    for (int k = 0; k < 3; ++k) refill(c0 - 1 + k, k);
+    HalfX<T> L;
+    {
+        C p, m;
+        nbr(xS(c0), p, m);
+        T cf[kNCoef];
+        coefs(true, c0 - 1, cf);
+        C src = C::zero();
+        if (has_src) src = term_h(c0 - 1);
+        L = predict_x<T, true>(A, u_prev.F, u_prev.Pp, u_cur.F, u_cur.Pp, s0, p, m, cf, hdt, src);
+    }
+    size_t o = node_index(d, c0, j);
+    // two instances of the loop: blocks without source nodes carry no source code
+    auto steady = [&](auto src_kind) {
+        constexpr bool kSrc = decltype(src_kind)::value;
+        int slot = 3 % R;   // of column c + 1
+#pragma unroll 2
+        for (int c = c0 + 1; c <= c1; ++c) {
+            // half node c-1/2 = (c-1, c): u_cur holds c-1, u_next column c
+            C p, m;
+            nbr(xs_(c - 1), p, m);
+            T cf[kNCoef];
+            coefs(true, c - 1, cf);
+            C src = C::zero();
+            if constexpr (kSrc) src = term_h(c - 1);
+            const HalfX<T> Rh = predict_x<T, kSrc>(A, u_cur.F, u_cur.Pp, u_next.F, u_next.Pp, s, p, m, cf, hdt, src);
+            const C S = A.add(Rh.F, L.F);
+            publish16<T>(xS(c), j, S, g, row_ok, top, bot);
+            const NodeV<P> u = u_cur;
+            u_cur = u_next;
+            if (c < c1) {
+                ring.wait(slot);
+                u_next = node(slot);
+                s = A.add(u_cur.F, u_next.F);
+                publish16<T>(xs_(c), j, s, g, row_ok, top, bot);
+            }
+            __syncthreads();
+            if (c < c1) refill(c + 1, slot);
+            C S_p, S_m;
+            nbr(xS(c), S_p, S_m);
+            T ci[kNCoef];
+            coefs(false, c - 1, ci);
+            C srcc = C::zero();
+            if constexpr (kSrc) srcc = term_i(c - 1);
+            C dPhi, dPi;
+            correct_x<T, kSrc>(A, Rh, L, S, S_p, S_m, ci, qdt, srcc, dPhi, dPi);
+            if (row_ok && TK_IN(d.status, o, plane_elems(d))) {
+                NodeV<P> v = u;
+                v.F = A.add(v.F, dPhi);
+                v.Pp = A.add(v.Pp, dPi);
+                out.store(o, v);
+            }
+            L = Rh;
+            o += d.pitch;
+            slot = slot + 1 == R ? 0 : slot + 1;
+        }
+    };
+    if (has_src) steady(std::true_type{});
+    else steady(std::false_type{});
+}
+
 // One work item: the columns [c0, c1) of one instance for one step, one thread per row.
 // Per column c: theta differences of Phi(c), dl = Phi(j+1) - Phi(j) and dlm = Phi(j) -
 // Phi(j-1), from the ring slot; predictor at the half node c-1/2; exchange of its
@@ -229,7 +357,7 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
                                            int c1, ColumnRing<P, R>& ring, typename P::T* xbuf) {
     using T = typename P::T;
     using C = Cx<T>;
-    constexpr bool kTabsPath = uses_1d_tables<P>();   // FP32 paths: coefficients from 1D tables
+    constexpr bool kSplit = split_angular<P>();
     const int j = threadIdx.x;
     const int nth = d.nth;
     const bool row_ok = j < nth;
@@ -258,7 +386,7 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
     if (src_blk) {
         const int w1 = blockDim.x > 32 ? 32 : 0;
         if (threadIdx.x == 0) {
-            const double2 f = source_factor<kMov>(d, step, 0.0, 0.5 * d.dt);
+            const double2 f = source_factor<kMov>(d, step, 0.0, kSplit ? 0.5 * d.dt : d.dt);
             sfac[0] = (T)f.x;
             sfac[1] = (T)f.y;
         }
@@ -304,101 +432,14 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
         }
     }
     const bool ex_blk = c0 - 1 <= d.i_e && d.i_e <= c1 - 1;
+    if constexpr (!kSplit) {
+        if ((c0 <= d.i_e && d.i_e < c1) || (c0 == 1 && d.i_e == 0)) record_level<P>(d, step, bin);
+    }
 
     // radial boundary condition: Phi = Pi = 0 at i = 0 and i = nr - 1
     if (row_ok && c0 == 1) out.store(node_index(d, 0, j), NodeV<P>::zero());
     if (row_ok && c1 == d.nr - 1) out.store(node_index(d, d.nr - 1, j), NodeV<P>::zero());
 
-    // own node of the column in slot s (rows past nth read slot padding: their results
-    // are never stored or exchanged)
-    auto node = [&](int s) { return ring.planes(s).load((size_t)j); };
-    // theta differences of Phi in the column in slot s (own node u): forward and backward
-    // (expanded angular form) or second and two-cell (split form, see split_angular)
-    constexpr bool kSplit = split_angular<P>();
-    auto theta_diffs = [&](int s, const NodeV<P>& u, C& dl, C& dlm) {
-        const Planes<P> pl = ring.planes(s);
-        const NodeV<P> dn = pl.load_phi((size_t)jp), upn = pl.load_phi((size_t)jm);
-        if constexpr (kSplit) {
-            u.theta_split(gp, dn, gm, upn, dl, dlm);
-        } else {
-            dl = dn.dphi_sl(gp, u);
-            dlm = u.dphi_sr(gm, upn);
-        }
-    };
-    // predictor at the half node h between columns h (ul) and h+1 (ur)
-    auto predict = [&](const NodeV<P>& ul, const NodeV<P>& ur, C dll, C dlr, C dlml, C dlmr,
-                       const T* cf, C src) {
-        const Half<T> hp = half_prep<P>(ul, ur);
-        const C Dp = C::half_sum(dll, dlr);     // Fb(j+1) - Fb(j)    (split: Fb(j+1) - 2 Fb(j) + Fb(j-1))
-        const C Dm = C::half_sum(dlml, dlmr);   // Fb(j) - Fb(j-1)    (split: Fb(j+1) - Fb(j-1))
-        return predictor<T, kSplit>(hp, Dp, Dm, cf, hdt, src);
-    };
-    // coefficients of column col: the half node col+1/2 into cfh and, on the FP32 paths
-    // (formed together in paired instructions), the node col into cfi
-    auto coefs = [&](int slot, int col, T* cfh, T* cfi) {
-        if constexpr (kTabsPath) {
-            float2 cf2[kNCoef];
-            form_coefs2(ring.tab2(slot), rt.t, cf2);
-#pragma unroll
-            for (int k = 0; k < kNCoef; ++k) {
-                cfh[k] = cf2[k].x;
-                cfi[k] = cf2[k].y;
-            }
-        } else if constexpr (P::kind == kDF) {
-            if (TK_IN(d.status, col, d.nr)) coefs_df(d, true, col, j, (DF*)cfh);
-        } else {
-            if (TK_IN(d.status, col, d.nr)) coefs64(d, true, col, j, (double*)cfh);
-        }
-    };
-    // corrector at column cc from the half nodes L = cc-1/2 and R = cc+1/2; xb is the
-    // exchange buffer of this column's parity, srcc the source term at (cc, j); cfi the
-    // node's coefficients on the FP32 paths (the FP64 path reads them here)
-    auto correct = [&](const HalfRec<T>& Rh, const HalfRec<T>& Lh, const NodeV<P>& uc,
-                       const T* cfi, int cc, T* xb, size_t o, C srcc) {
-        const CRow<T> row = combine_lr<T, kSplit>(Rh, Lh);
-        // publish this row's exchange entry (the split form needs Hs alone: its averaged
-        // differences are the row's own), then read the rows above and below
-        T* mine = xb + 4 * (j + 1);
-        xpublish<P, kSplit>(xb, mine, row, Rh, Lh, g, row_ok, top, bot);
-        __syncthreads();
-        C Hs_p, Hs_m, DpS_m;
-        xread<P, kSplit>(mine, Hs_p, Hs_m, DpS_m);
-        T cf[kNCoef];
-        if constexpr (kTabsPath) {
-#pragma unroll
-            for (int k = 0; k < kNCoef; ++k) cf[k] = cfi[k];
-        } else if constexpr (P::kind == kDF) {
-            if (TK_IN(d.status, cc, d.nr)) coefs_df(d, false, cc, j, (DF*)cf);
-        } else {
-            if (TK_IN(d.status, cc, d.nr)) coefs64(d, false, cc, j, (double*)cf);
-        }
-        C dPhi, dPi;
-        corrector_incr<P, kSplit>(row, Hs_p, Hs_m, DpS_m, cf, fdt, srcc, dPhi, dPi);
-        if (row_ok && TK_IN(d.status, o, plane_elems(d))) {
-            NodeV<P> u = uc;
-            u.update(dPhi, dPi);
-            out.store(o, u);
-        }
-    };
-    // waveform record of the input level between columns i_e (ul) and i_e + 1 (ur)
-    auto extract = [&](const NodeV<P>& ul, const NodeV<P>& ur) {
-        if (!row_ok) return;
-        double2 a = ul.phi64(), b = ur.phi64();
-        double f = d.f_e;
-        double2 w = wave_lerp(a, b, f);
-        const size_t wi = (size_t)(step % d.wave_cap) * nth + j;
-        if (TK_IN(d.status, wi, d.wave_cap * nth)) d.wave[wi] = w;
-        if (!isfinite(w.x) || !isfinite(w.y)) atomicOr(d.status, (unsigned)ST_NONFINITE);
-    };
-
-    // prologue: columns c0-1 (slot 0) and c0 (slot 1)
-    C dl_prev, dlm_prev, dl, dlm;
-    ring.wait(0);
-    NodeV<P> u_prev = node(0);
-    theta_diffs(0, u_prev, dl_prev, dlm_prev);
-    ring.wait(1);
-    NodeV<P> u_cur = node(1);
-    theta_diffs(1, u_cur, dl, dlm);
     // source terms at the half node h and the node i (source blocks only)
     auto src_h = [&](int h) { return source_half<T>(sw, sp_fac, h, j); };
     auto src_i = [&](int i) { return source_int<T>(sw, sc_fac, i, j); };
@@ -413,72 +454,146 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
         const T g = (unsigned)a < (unsigned)sw.ni ? gr[sw.nh + a] : T(0);
         return source_int<T>(sw, g * sc_fac, i, j);
     };
-    T cfh[kNCoef], cfi[kNCoef];
-    coefs(0, c0 - 1, cfh, cfi);
-    C s_first = C::zero();
-    if constexpr (kMov) {
-        if (gr) s_first = msrc_h(c0 - 1);
-        else if (src_blk) s_first = src_h(c0 - 1);
-    } else {
-        if (src_blk) s_first = src_h(c0 - 1);
-    }
-    HalfRec<T> L = predict(u_prev, u_cur, dl_prev, dl, dlm_prev, dlm, cfh, s_first);
-    if (ex_blk && d.i_e == c0 - 1) extract(u_prev, u_cur);
-    u_prev = u_cur;
-    dl_prev = dl;
-    dlm_prev = dlm;
-    size_t o = node_index(d, c0, j);               // output offset of the corrector's column
-
-    // steady state: column c arrives, predictor at c-1/2, corrector at c-1; the slots
-    // hold columns c-2 (sf, free once the column's barrier is passed), c-1 (sp) and c (sc).
-    // Three instances of the loop: blocks without source nodes carry no source code; the
-    // source blocks (circular orbit: kSrc = 1, moving particle: 2) load the next
-    // column's source terms one column ahead.
-    auto steady = [&](auto src_kind) {
-        constexpr int kSrc = decltype(src_kind)::value;
-        auto load_src = [&](int c, C& h, C& i) {
-            if constexpr (kSrc == 1) {
-                h = src_h(c);
-                i = src_i(c);
-            } else if constexpr (kSrc == 2 && kMov) {
-                h = msrc_h(c);
-                i = msrc_i(c);
+    if constexpr (kSplit) {
+        // own node of the column in slot s (rows past nth read slot padding: their results
+        // are never stored or exchanged)
+        auto node = [&](int s) { return ring.planes(s).load((size_t)j); };
+        // theta differences of Phi in the column in slot s (own node u): forward and backward
+        // (expanded angular form) or second and two-cell (split form, see split_angular)
+        auto theta_diffs = [&](int s, const NodeV<P>& u, C& dl, C& dlm) {
+            const Planes<P> pl = ring.planes(s);
+            const NodeV<P> dn = pl.load_phi((size_t)jp), upn = pl.load_phi((size_t)jm);
+            u.theta_split(gp, dn, gm, upn, dl, dlm);
+        };
+        // predictor at the half node h between columns h (ul) and h+1 (ur)
+        auto predict = [&](const NodeV<P>& ul, const NodeV<P>& ur, C dll, C dlr, C dlml, C dlmr,
+                           const T* cf, C src) {
+            const Half<T> hp = half_prep<P>(ul, ur);
+            const C Dp = C::half_sum(dll, dlr);     // Fb(j+1) - Fb(j)    (split: Fb(j+1) - 2 Fb(j) + Fb(j-1))
+            const C Dm = C::half_sum(dlml, dlmr);   // Fb(j) - Fb(j-1)    (split: Fb(j+1) - Fb(j-1))
+            return predictor<T>(hp, Dp, Dm, cf, hdt, src);
+        };
+        // coefficients of column col: the half node col+1/2 into cfh and, on the FP32 paths
+        // (formed together in paired instructions), the node col into cfi
+        auto coefs = [&](int slot, int col, T* cfh, T* cfi) {
+            float2 cf2[kNCoef];
+            form_coefs2(ring.tab2(slot), rt.t, cf2);
+#pragma unroll
+            for (int k = 0; k < kNCoef; ++k) {
+                cfh[k] = cf2[k].x;
+                cfi[k] = cf2[k].y;
             }
         };
-        C nxt_h = C::zero(), nxt_i = C::zero();
-        load_src(c0, nxt_h, nxt_i);
-        int sf = 0, sp = 1, sc = 2;
-#pragma unroll 2
-        for (int c = c0 + 1; c <= c1; ++c) {
-            const C s_h = nxt_h, s_i = nxt_i;
-            if constexpr (kSrc != 0) {
-                if (c < c1) load_src(c, nxt_h, nxt_i);
+        // corrector at column cc from the half nodes L = cc-1/2 and R = cc+1/2; xb is the
+        // exchange buffer of this column's parity, srcc the source term at (cc, j); cfi the
+        // node's coefficients on the FP32 paths (the FP64 path reads them here)
+        auto correct = [&](const HalfRec<T>& Rh, const HalfRec<T>& Lh, const NodeV<P>& uc,
+                           const T* cfi, int cc, T* xb, size_t o, C srcc) {
+            const CRow<T> row = combine_lr<T>(Rh, Lh);
+            // publish this row's exchange entry (the split form needs Hs alone: its averaged
+            // differences are the row's own), then read the rows above and below
+            T* mine = xb + 4 * (j + 1);
+            xpublish(xb, mine, row, g, row_ok, top, bot);
+            __syncthreads();
+            C Hs_p, Hs_m;
+            xread(mine, Hs_p, Hs_m);
+            C dPhi, dPi;
+            corrector_incr<P>(row, Hs_p, Hs_m, cfi, fdt, srcc, dPhi, dPi);
+            if (row_ok && TK_IN(d.status, o, plane_elems(d))) {
+                NodeV<P> u = uc;
+                u.update(dPhi, dPi);
+                out.store(o, u);
             }
-            ring.wait(sc);
-            u_cur = node(sc);
-            theta_diffs(sc, u_cur, dl, dlm);
-            coefs(sp, c - 1, cfh, cfi);
-            const HalfRec<T> Rh = predict(u_prev, u_cur, dl_prev, dl, dlm_prev, dlm, cfh, s_h);
-            correct(Rh, L, u_prev, cfi, c - 1, xbuf + (c & 1) * xstride, o, s_i);
-            if (threadIdx.x == 0 && c - 2 + R <= c1) ring.fill(d, bin, c - 2 + R, sf);
-            if (ex_blk && d.i_e == c - 1) extract(u_prev, u_cur);
-            L = Rh;
-            u_prev = u_cur;
-            dl_prev = dl;
-            dlm_prev = dlm;
-            o += pitch;
-            sf = sp;
-            sp = sc;
-            sc = sc + 1 == R ? 0 : sc + 1;
+        };
+        // waveform record of the input level between columns i_e (ul) and i_e + 1 (ur)
+        auto extract = [&](const NodeV<P>& ul, const NodeV<P>& ur) {
+            if (!row_ok) return;
+            double2 a = ul.phi64(), b = ur.phi64();
+            double f = d.f_e;
+            double2 w = wave_lerp(a, b, f);
+            const size_t wi = (size_t)(step % d.wave_cap) * nth + j;
+            if (TK_IN(d.status, wi, d.wave_cap * nth)) d.wave[wi] = w;
+            if (!isfinite(w.x) || !isfinite(w.y)) atomicOr(d.status, (unsigned)ST_NONFINITE);
+        };
+
+        // prologue: columns c0-1 (slot 0) and c0 (slot 1)
+        C dl_prev, dlm_prev, dl, dlm;
+        ring.wait(0);
+        NodeV<P> u_prev = node(0);
+        theta_diffs(0, u_prev, dl_prev, dlm_prev);
+        ring.wait(1);
+        NodeV<P> u_cur = node(1);
+        theta_diffs(1, u_cur, dl, dlm);
+        T cfh[kNCoef], cfi[kNCoef];
+        coefs(0, c0 - 1, cfh, cfi);
+        C s_first = C::zero();
+        if constexpr (kMov) {
+            if (gr) s_first = msrc_h(c0 - 1);
+            else if (src_blk) s_first = src_h(c0 - 1);
+        } else {
+            if (src_blk) s_first = src_h(c0 - 1);
         }
-    };
-    if constexpr (kMov) {
-        if (gr) steady(std::integral_constant<int, 2>{});
-        else if (src_blk) steady(std::integral_constant<int, 1>{});
-        else steady(std::integral_constant<int, 0>{});
+        HalfRec<T> L = predict(u_prev, u_cur, dl_prev, dl, dlm_prev, dlm, cfh, s_first);
+        if (ex_blk && d.i_e == c0 - 1) extract(u_prev, u_cur);
+        u_prev = u_cur;
+        dl_prev = dl;
+        dlm_prev = dlm;
+        size_t o = node_index(d, c0, j);               // output offset of the corrector's column
+
+        // steady state: column c arrives, predictor at c-1/2, corrector at c-1; the slots
+        // hold columns c-2 (sf, free once the column's barrier is passed), c-1 (sp) and c (sc).
+        // Three instances of the loop: blocks without source nodes carry no source code; the
+        // source blocks (circular orbit: kSrc = 1, moving particle: 2) load the next
+        // column's source terms one column ahead.
+        auto steady = [&](auto src_kind) {
+            constexpr int kSrc = decltype(src_kind)::value;
+            auto load_src = [&](int c, C& h, C& i) {
+                if constexpr (kSrc == 1) {
+                    h = src_h(c);
+                    i = src_i(c);
+                } else if constexpr (kSrc == 2 && kMov) {
+                    h = msrc_h(c);
+                    i = msrc_i(c);
+                }
+            };
+            C nxt_h = C::zero(), nxt_i = C::zero();
+            load_src(c0, nxt_h, nxt_i);
+            int sf = 0, sp = 1, sc = 2;
+    #pragma unroll 2
+            for (int c = c0 + 1; c <= c1; ++c) {
+                const C s_h = nxt_h, s_i = nxt_i;
+                if constexpr (kSrc != 0) {
+                    if (c < c1) load_src(c, nxt_h, nxt_i);
+                }
+                ring.wait(sc);
+                u_cur = node(sc);
+                theta_diffs(sc, u_cur, dl, dlm);
+                coefs(sp, c - 1, cfh, cfi);
+                const HalfRec<T> Rh = predict(u_prev, u_cur, dl_prev, dl, dlm_prev, dlm, cfh, s_h);
+                correct(Rh, L, u_prev, cfi, c - 1, xbuf + (c & 1) * xstride, o, s_i);
+                if (threadIdx.x == 0 && c - 2 + R <= c1) ring.fill(d, bin, c - 2 + R, sf);
+                if (ex_blk && d.i_e == c - 1) extract(u_prev, u_cur);
+                L = Rh;
+                u_prev = u_cur;
+                dl_prev = dl;
+                dlm_prev = dlm;
+                o += pitch;
+                sf = sp;
+                sp = sc;
+                sc = sc + 1 == R ? 0 : sc + 1;
+            }
+        };
+        if constexpr (kMov) {
+            if (gr) steady(std::integral_constant<int, 2>{});
+            else if (src_blk) steady(std::integral_constant<int, 1>{});
+            else steady(std::integral_constant<int, 0>{});
+        } else {
+            if (src_blk) steady(std::integral_constant<int, 1>{});
+            else steady(std::integral_constant<int, 0>{});
+        }
     } else {
-        if (src_blk) steady(std::integral_constant<int, 1>{});
-        else steady(std::integral_constant<int, 0>{});
+        strip_columns_x<P, R, kMov>(d, step, bin, c0, c1, ring, (unsigned char*)xbuf, src_blk, gr != nullptr,
+                                    src_h, src_i, msrc_h, msrc_i);
     }
     if (__syncthreads_or(ring.late)) {
         if (threadIdx.x == 0) {

@@ -179,6 +179,8 @@ struct PD {
     static constexpr bool kahan = false;
     static constexpr int kind = kDF, planes = 2, blocks256 = 2;
 };
+template <typename T> __host__ __device__ constexpr bool uses_pairs() { return false; }
+template <> __host__ __device__ constexpr bool uses_pairs<DF>() { return true; }
 // the FP32 paths that form their coefficients from 1D tables
 template <class P>
 __host__ __device__ constexpr bool uses_1d_tables() { return P::kind == kFP32 || P::kind == kKahan; }
@@ -207,18 +209,6 @@ struct NodeV {
     __device__ __forceinline__ Cx<T> dphi(const NodeV& o) const {
         if constexpr (P::kahan) return (F - o.F) - (Fc - o.Fc);
         else return F - o.F;
-    }
-    // gs Phi(this) - Phi(o) and Phi(this) - gs Phi(o) for gs = +-1 (an exact scaling, so
-    // these round exactly as dphi of the scaled node)
-    __device__ __forceinline__ Cx<T> dphi_sl(T gs, const NodeV& o) const {
-        const Cx<T> a = rmac(neg(o.F), gs, F);
-        if constexpr (P::kahan) return a - rmac(neg(o.Fc), gs, Fc);
-        else return a;
-    }
-    __device__ __forceinline__ Cx<T> dphi_sr(T gs, const NodeV& o) const {
-        const Cx<T> a = rmac(F, -gs, o.F);
-        if constexpr (P::kahan) return a - rmac(Fc, -gs, o.Fc);
-        else return a;
     }
     // Split theta differences of Phi at this node from the rows above (a, factor ga)
     // and below (b, factor gb): d2 = ga a - 2 this + gb b and d1 = ga a - gb b.  For
@@ -411,9 +401,123 @@ __device__ __forceinline__ Half<typename P::T> half_prep(const NodeV<P>& own, co
 template <class P>
 __host__ __device__ constexpr bool split_angular() { return P::kind == kFP32 || P::kind == kKahan; }
 
-// Predictor output at one half node, plus the inputs the corrector needs from it.
-// Expanded form: Dp = Fb(j+1) - Fb(j) (D1 unused); split form: Dp = Fb(j+1) - 2 Fb(j) +
-// Fb(j-1), D1 = Fb(j+1) - Fb(j-1).
+// ---------------------------------------------------------------- expanded form
+// FP64 and double-float step (HalfX, predict_x, correct_x).  What bounds it is the number
+// of operations: GB300's FP64 pipe retires one warp DFMA per SM in 16 clocks, so every
+// operation counts, and a double-float operation is 8 to 16 FP32 ones.  The half-node
+// state is therefore kept undivided, as 2 h = (u_i + u_{i+1}) + ..., the powers of two
+// folded into the coefficient tables (exactly; teuk_setup.cu), sums and differences are
+// formed once and shared, and the angular differences are taken of the sums s = Phi_i +
+// Phi_{i+1} and S = 2 h_R + 2 h_L, which the neighbouring rows exchange:
+//   predictor   s, sP, dF, dP (sums and differences of columns i, i+1)
+//     2 h_Phi = s + (dt/2) sP - G dF
+//     2 h_Pi  = sP + G dP + E1 sP + E2 dF + ep (s(j+1) - s(j)) - em (s(j) - s(j-1)) + E3 s + dt tau
+//   corrector   S, SP, D, DP (sums and differences of the half nodes R, L)
+//     Phi += (dt/4) SP - G D
+//     Pi  += G DP + E1 SP + E2 D + ep (S(j+1) - S(j)) - em (S(j) - S(j-1)) + E3 S + dt tau
+// 72 FP64 operations a node where the form in separate half-node increments had 124.  The
+// rounding error against extended precision is the same (60 x 128 grid, 1000 steps: 3.89e-15
+// both), because both increments of the state are formed apart and added once.  16384 x 256,
+// us per step before and after: FP64 947 -> 629, double-float 262 -> 205 (681 -> 506 paired
+// FP32 operations a node, and no register spills: the record of a half node is two complex
+// values instead of eight).
+
+// Complex sums and differences.  FP64: as DFMA with a factor one that the compiler cannot
+// see (DADD and DMUL take 19 clocks of the SM's FP64 pipe, DFMA 16; the rounding is the
+// sum's own).  A product is formed as DFMA with a zero addend for the same reason.
+template <typename T> struct Lin;
+template <> struct Lin<double> {
+    using C = Cx<double>;
+    double one;
+    __device__ __forceinline__ explicit Lin(const InstDev& d) : one(d.one) {}
+    __device__ __forceinline__ C add(C a, C b) const {
+        return {__fma_rn(a.re, one, b.re), __fma_rn(a.im, one, b.im)};
+    }
+    __device__ __forceinline__ C sub(C a, C b) const {
+        return {__fma_rn(b.re, -one, a.re), __fma_rn(b.im, -one, a.im)};
+    }
+    __device__ __forceinline__ C mul(double s, C a) const { return {__fma_rn(s, a.re, 0.0), __fma_rn(s, a.im, 0.0)}; }
+};
+template <> struct Lin<DF> {
+    using C = Cx<DF>;
+    __device__ __forceinline__ explicit Lin(const InstDev&) {}
+    __device__ __forceinline__ C add(C a, C b) const { return a + b; }
+    __device__ __forceinline__ C sub(C a, C b) const { return a - b; }
+    __device__ __forceinline__ C mul(DF s, C a) const { return s * a; }
+};
+
+template <> struct Lin<float> {   // (the FP32 paths take the split form)
+    __device__ __forceinline__ explicit Lin(const InstDev&) {}
+};
+
+// 2 h_Phi and 2 h_Pi at one half node
+template <typename T>
+struct HalfX { Cx<T> F, P; };
+
+// kSrc: src is a source term (else it is not read)
+template <typename T, bool kSrc>
+__device__ __forceinline__ HalfX<T> predict_x(const Lin<T>& A, Cx<T> F0, Cx<T> P0, Cx<T> F1, Cx<T> P1, Cx<T> s,
+                                              Cx<T> s_p, Cx<T> s_m, const T* cf, T hdt, Cx<T> src) {
+    const Cx<T> dF = A.sub(F1, F0), sP = A.add(P0, P1), dP = A.sub(P1, P0);
+    HalfX<T> h;
+    h.F = rmac(rmac(s, hdt, sP), -cf[C_G], dF);
+    Cx<T> a = rmac(sP, cf[C_G], dP);
+    a = cmac(a, cf[C_E1R], cf[C_E1I], sP);
+    a = cmac(a, cf[C_E2R], cf[C_E2I], dF);
+    a = cmac(a, cf[C_E3R], cf[C_E3I], s);
+    a = rmac(a, cf[C_EP], A.sub(s_p, s));
+    a = rmac(a, -cf[C_EM], A.sub(s, s_m));
+    if constexpr (kSrc) a = A.add(a, src);
+    h.P = a;
+    return h;
+}
+
+// Eq. (14) at one node: the increments of Phi and Pi from the half nodes R and L, with S =
+// R.F + L.F of this row and of the rows above and below
+template <typename T, bool kSrc>
+__device__ __forceinline__ void correct_x(const Lin<T>& A, const HalfX<T>& R, const HalfX<T>& L, Cx<T> S, Cx<T> S_p,
+                                          Cx<T> S_m, const T* cf, T qdt, Cx<T> src, Cx<T>& dPhi, Cx<T>& dPi) {
+    const Cx<T> D = A.sub(R.F, L.F), SP = A.add(R.P, L.P), DP = A.sub(R.P, L.P);
+    dPhi = rmac(A.mul(qdt, SP), -cf[C_G], D);
+    Cx<T> a;
+    if constexpr (kSrc) a = rmac(src, cf[C_G], DP);
+    else a = A.mul(cf[C_G], DP);
+    a = cmac(a, cf[C_E1R], cf[C_E1I], SP);
+    a = cmac(a, cf[C_E2R], cf[C_E2I], D);
+    a = cmac(a, cf[C_E3R], cf[C_E3I], S);
+    a = rmac(a, cf[C_EP], A.sub(S_p, S));
+    a = rmac(a, -cf[C_EM], A.sub(S, S_m));
+    dPi = a;
+}
+
+// A complex value as one 16-byte shared-memory entry
+__device__ __forceinline__ void put16(void* e, Cx<double> v) { *(double2*)e = make_double2(v.re, v.im); }
+__device__ __forceinline__ void put16(void* e, Cx<DF> v) {
+    *(float4*)e = make_float4(v.re.hi, v.im.hi, v.re.lo, v.im.lo);
+}
+template <typename T>
+__device__ __forceinline__ Cx<T> get16(const void* e) {
+    if constexpr (sizeof(Cx<T>) == sizeof(double2) && !uses_pairs<T>()) {
+        const double2 v = *(const double2*)e;
+        return {v.x, v.y};
+    } else {
+        const float4 v = *(const float4*)e;
+        return {T(v.x, v.z), T(v.y, v.w)};
+    }
+}
+// Publish this row's value (row j at entry j + 1 of x) and, for the pole rows, the ghost
+// rows' entries 0 and n_theta + 1 (the row times the pole factor g = +-1)
+template <typename T>
+__device__ __forceinline__ void publish16(unsigned char* x, int j, Cx<T> v, T g, bool row_ok, bool top, bool bot) {
+    unsigned char* mine = x + 16 * (j + 1);
+    if (row_ok) put16(mine, v);
+    if (top) put16(mine + 16, g * v);
+    if (bot) put16(x, g * v);
+}
+
+// ---------------------------------------------------------------- split form
+// Predictor output at one half node, plus the inputs the corrector needs from it
+// (Dp = Fb(j+1) - 2 Fb(j) + Fb(j-1), D1 = Fb(j+1) - Fb(j-1)).
 template <typename T>
 struct HalfRec { Cx<T> Fb, Pb, dF, dP, Dp, D1, hF, hP; };
 
@@ -422,17 +526,17 @@ template <typename T>
 struct CRow {
     Cx<T> Hs;        // (dh_Phi_R + dh_Phi_L)/2
     Cx<T> DpS;       // (Dp_R + Dp_L)/2
-    Cx<T> D1S;       // (D1_R + D1_L)/2 (split form)
+    Cx<T> D1S;       // (D1_R + D1_L)/2
     Cx<T> FC, PC;    // u~ = (h_R + h_L)/2 for Phi and Pi
     Cx<T> dFc, dPc;  // h_R - h_L for Phi and Pi
 };
 
-template <typename T, bool kSplit>
+template <typename T>
 __device__ __forceinline__ CRow<T> combine_lr(const HalfRec<T>& R, const HalfRec<T>& L) {
     CRow<T> c;
     c.Hs = Cx<T>::half_sum(R.hF, L.hF);
     c.DpS = Cx<T>::half_sum(R.Dp, L.Dp);
-    if constexpr (kSplit) c.D1S = Cx<T>::half_sum(R.D1, L.D1);
+    c.D1S = Cx<T>::half_sum(R.D1, L.D1);
     c.FC = half_sum_add(R.Fb, L.Fb, c.Hs);
     c.PC = half_sum_add(R.Pb, L.Pb, Cx<T>::half_sum(R.hP, L.hP));
     c.dFc = half_sum_add(R.dF, L.dF, R.hF - L.hF);
@@ -503,10 +607,9 @@ __device__ __forceinline__ void coefs_df(const InstDev& d, bool half, int i, int
     }
 }
 
-// Eq. (13) at the own half node, as an increment on the averaged state.  Dp, Dm: the
-// theta differences of the averaged state in the angular form of kSplit (expanded:
-// forward and backward differences; split: second and two-cell differences).
-template <typename T, bool kSplit>
+// Eq. (13) at the own half node, as an increment on the averaged state.  Dp, Dm: its second
+// and two-cell theta differences.
+template <typename T>
 __device__ __forceinline__ HalfRec<T> predictor(const Half<T>& h, Cx<T> Dp, Cx<T> Dm, const T* cf,
                                                 T hdt, Cx<T> src) {
     HalfRec<T> r;
@@ -515,13 +618,8 @@ __device__ __forceinline__ HalfRec<T> predictor(const Half<T>& h, Cx<T> Dp, Cx<T
     Cx<T> a = rmac(src, cf[C_G], h.dP);
     a = cmac(a, cf[C_E1R], cf[C_E1I], h.Pb);
     a = cmac(a, cf[C_E2R], cf[C_E2I], h.dF);
-    if constexpr (kSplit) {
-        a = rmac(a, cf[C_EP], Dp);
-        a = rmac(a, cf[C_EM], Dm);
-    } else {
-        a = rmac(a, cf[C_EP], Dp);
-        a = rmac(a, -cf[C_EM], Dm);
-    }
+    a = rmac(a, cf[C_EP], Dp);
+    a = rmac(a, cf[C_EM], Dm);
     a = cmac(a, cf[C_E3R], cf[C_E3I], h.Fb);
     r.hP = a;
     return r;
@@ -536,102 +634,41 @@ __device__ __forceinline__ double2 wave_lerp(double2 a, double2 b, double f) {
 }
 
 // ---------------------------------------------------------------- corrector
-// Exchange entry of one row for the corrector's theta neighbours: {Hs, DpS} (4 values of
-// T at e; the split form uses Hs alone).  Row j sits at entry j + 1 of its column's
-// buffer; entries 0 and n_theta + 1 hold the ghost rows of the pole rule:
-// row nth Hs = g Hs(nth-1); row -1 Hs = g Hs(0) and DpS = (Dp_R(-1) + Dp_L(-1))/2 =
-// (1 - g) (Fb_R + Fb_L)(0)/2.
-template <class P>
-__device__ __forceinline__ void xput(typename P::T* e, Cx<typename P::T> a, Cx<typename P::T> b) {
-    if constexpr (P::kind == kDF) {
-        ((float4*)e)[0] = make_float4(a.re.hi, a.re.lo, a.im.hi, a.im.lo);
-        ((float4*)e)[1] = make_float4(b.re.hi, b.re.lo, b.im.hi, b.im.lo);
-    } else if constexpr (sizeof(typename P::T) == 4) {
-        *(float4*)e = make_float4(a.re, a.im, b.re, b.im);
-    } else {
-        ((double2*)e)[0] = make_double2(a.re, a.im);
-        ((double2*)e)[1] = make_double2(b.re, b.im);
-    }
-}
-
-// Publish this row's entry (xb: the column's buffer, mine = xb + 4 (j + 1)) and, for the
-// pole rows, the ghost entries.
-template <class P, bool kSplit>
-__device__ __forceinline__ void xpublish(typename P::T* xb, typename P::T* mine, const CRow<typename P::T>& row,
-                                         const HalfRec<typename P::T>& Rh, const HalfRec<typename P::T>& Lh,
-                                         typename P::T g, bool row_ok, bool top, bool bot) {
-    using T = typename P::T;
-    using C = Cx<T>;
-    if constexpr (kSplit) {
-        if (row_ok) *(float2*)mine = make_float2(row.Hs.re, row.Hs.im);
-        if (top) *(float2*)(mine + 4) = make_float2(g * row.Hs.re, g * row.Hs.im);
-        if (bot) *(float2*)xb = make_float2(g * row.Hs.re, g * row.Hs.im);
-    } else {
-        if (row_ok) xput<P>(mine, row.Hs, row.DpS);
-        if (top) xput<P>(mine + 4, g * row.Hs, C::zero());
-        if (bot) xput<P>(xb, g * row.Hs, (T(1) - g) * C::half_sum(Rh.Fb, Lh.Fb));
-    }
+// Exchange entry of one row for the corrector's theta neighbours: Hs (the first two of the
+// entry's four floats).  Row j sits at entry j + 1 of its column's buffer; entries 0 and
+// n_theta + 1 hold the ghost rows of the pole rule, g Hs of the pole row.
+// xb: the column's buffer, mine = xb + 4 (j + 1).
+__device__ __forceinline__ void xpublish(float* xb, float* mine, const CRow<float>& row, float g, bool row_ok,
+                                         bool top, bool bot) {
+    if (row_ok) *(float2*)mine = make_float2(row.Hs.re, row.Hs.im);
+    if (top) *(float2*)(mine + 4) = make_float2(g * row.Hs.re, g * row.Hs.im);
+    if (bot) *(float2*)xb = make_float2(g * row.Hs.re, g * row.Hs.im);
 }
 
 // Read the entries of the rows above and below (after the barrier that follows xpublish).
-template <class P, bool kSplit>
-__device__ __forceinline__ void xread(const typename P::T* mine, Cx<typename P::T>& Hs_p,
-                                      Cx<typename P::T>& Hs_m, Cx<typename P::T>& DpS_m) {
-    if constexpr (kSplit) {
-        const float2 a = *(const float2*)(mine + 4), b = *(const float2*)(mine - 4);
-        Hs_p = {a.x, a.y};
-        Hs_m = {b.x, b.y};
-    } else if constexpr (P::kind == kDF) {
-        const float4 a = *(const float4*)(mine + 4);
-        const float4 b0 = ((const float4*)(mine - 4))[0], b1 = ((const float4*)(mine - 4))[1];
-        Hs_p = {DF(a.x, a.y), DF(a.z, a.w)};
-        Hs_m = {DF(b0.x, b0.y), DF(b0.z, b0.w)};
-        DpS_m = {DF(b1.x, b1.y), DF(b1.z, b1.w)};
-    } else if constexpr (sizeof(typename P::T) == 4) {
-        const float2 a = *(const float2*)(mine + 4);
-        const float4 b = *(const float4*)(mine - 4);
-        Hs_p = {a.x, a.y};
-        Hs_m = {b.x, b.y};
-        DpS_m = {b.z, b.w};
-    } else {
-        const double2 a = *(const double2*)(mine + 4);
-        const double2 b0 = ((const double2*)(mine - 4))[0], b1 = ((const double2*)(mine - 4))[1];
-        Hs_p = {a.x, a.y};
-        Hs_m = {b0.x, b0.y};
-        DpS_m = {b1.x, b1.y};
-    }
+__device__ __forceinline__ void xread(const float* mine, Cx<float>& Hs_p, Cx<float>& Hs_m) {
+    const float2 a = *(const float2*)(mine + 4), b = *(const float2*)(mine - 4);
+    Hs_p = {a.x, a.y};
+    Hs_m = {b.x, b.y};
 }
 
 // Eq. (14) at one node as increments (dPhi, dPi) from the row's combined half-node values,
 // the theta neighbours' exchange entries, the node's coefficients cf and source term.
-template <class P, bool kSplit>
+template <class P>
 __device__ __forceinline__ void corrector_incr(const CRow<typename P::T>& row, Cx<typename P::T> Hs_p,
-                                               Cx<typename P::T> Hs_m, Cx<typename P::T> DpS_m,
-                                               const typename P::T* cf, typename P::T fdt,
+                                               Cx<typename P::T> Hs_m, const typename P::T* cf, typename P::T fdt,
                                                Cx<typename P::T> srcc, Cx<typename P::T>& dPhi,
                                                Cx<typename P::T>& dPi) {
     using C = Cx<typename P::T>;
-    // expanded: Dplus = u~(j+1) - u~(j), Dminus = u~(j) - u~(j-1) of the corrector's
-    // averaged state u~ = (h_R + h_L)/2; split: its second and two-cell differences
-    C Dplus, Dminus;
-    if constexpr (kSplit) {
-        Dplus = row.DpS + ((Hs_p - row.Hs) - (row.Hs - Hs_m));
-        Dminus = row.D1S + (Hs_p - Hs_m);
-    } else {
-        Dplus = row.DpS + (Hs_p - row.Hs);
-        Dminus = DpS_m + (row.Hs - Hs_m);
-    }
+    // second and two-cell differences of the corrector's averaged state u~ = (h_R + h_L)/2
+    const C Dplus = row.DpS + ((Hs_p - row.Hs) - (row.Hs - Hs_m));
+    const C Dminus = row.D1S + (Hs_p - Hs_m);
     dPhi = rmac(rmac(C::zero(), -cf[C_G], row.dFc), fdt, row.PC);
     dPi = rmac(srcc, cf[C_G], row.dPc);
     dPi = cmac(dPi, cf[C_E1R], cf[C_E1I], row.PC);
     dPi = cmac(dPi, cf[C_E2R], cf[C_E2I], row.dFc);
-    if constexpr (kSplit) {
-        dPi = rmac(dPi, cf[C_EP], Dplus);
-        dPi = rmac(dPi, cf[C_EM], Dminus);
-    } else {
-        dPi = rmac(dPi, cf[C_EP], Dplus);
-        dPi = rmac(dPi, -cf[C_EM], Dminus);
-    }
+    dPi = rmac(dPi, cf[C_EP], Dplus);
+    dPi = rmac(dPi, cf[C_EM], Dminus);
     dPi = cmac(dPi, cf[C_E3R], cf[C_E3I], row.FC);
 }
 
