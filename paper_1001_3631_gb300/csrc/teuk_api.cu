@@ -277,6 +277,7 @@ InstDev dev_of(const teuk_ctx* c, const Instance& I) {
     d.wave_cap = I.wave_cap;
     d.status = c->status;
     d.fault_col = I.fault_col;
+    d.resident = I.resident;
     return d;
 }
 

@@ -102,6 +102,8 @@ struct InstDev {
     unsigned int* status;     // device status word (bit flags)
     int fault_col;            // testing aid: this input column is never filled into the
                               // step kernels' ring (-1: none)
+    int resident;             // blocks of the per-step kernel that the GPU holds at once
+    int pad;
     const int64_t* step_base; // per-step kernels replayed from a graph: their step argument
                               // is an offset from *step_base (null: the argument is the step)
 };

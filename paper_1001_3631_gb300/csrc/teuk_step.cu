@@ -216,7 +216,10 @@ struct StepShared {
 constexpr int kRingS = 6, kRingL = 4;
 
 // Waveform record of the level in buffer bin between columns i_e and i_e + 1, one row a
-// thread, read from the buffer itself.
+// thread, read from the buffer itself.  It stands outside the column loop: in there the
+// compiler ran its FP64 conversions (1 to 2 a node on the FP32 paths, on a pipe that is
+// busy 16 clocks of the SM with each) at every column and discarded them (16384 x 256, us
+// per step: FP32-Kahan 50.9 -> 48.0, FP32 39.0 -> 37.1).
 template <class P>
 __device__ __forceinline__ void record_level(const InstDev& d, int64_t step, int bin) {
     const int j = threadIdx.x;
@@ -352,9 +355,11 @@ __device__ __forceinline__ void strip_columns_x(const InstDev& d, int64_t step, 
 // once when a bounded wait of an earlier launch gave up).  Returns false in that case.
 // kMov: the kernel serves instances whose particle moves (per-step Gaussian tables);
 // the kernels of circular orbits are compiled without that code.
+// rec_here: the block that owns the extraction column takes the level's record.
 template <class P, int R, bool kPerStep, bool kMov>
 __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int bin, int c0,
-                                           int c1, ColumnRing<P, R>& ring, typename P::T* xbuf) {
+                                           int c1, bool rec_here, ColumnRing<P, R>& ring,
+                                           typename P::T* xbuf) {
     using T = typename P::T;
     using C = Cx<T>;
     constexpr bool kSplit = split_angular<P>();
@@ -431,10 +436,9 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
             gr = (const T*)sw.gr + (size_t)step * (sw.nh + sw.ni);
         }
     }
-    const bool ex_blk = c0 - 1 <= d.i_e && d.i_e <= c1 - 1;
-    if constexpr (!kSplit) {
-        if ((c0 <= d.i_e && d.i_e < c1) || (c0 == 1 && d.i_e == 0)) record_level<P>(d, step, bin);
-    }
+    // the input level's waveform record, by the block that owns column i_e (block 0 also
+    // between columns 0 and 1), while the ring's first copies are in flight
+    if (rec_here && ((c0 <= d.i_e && d.i_e < c1) || (c0 == 1 && d.i_e == 0))) record_level<P>(d, step, bin);
 
     // radial boundary condition: Phi = Pi = 0 at i = 0 and i = nr - 1
     if (row_ok && c0 == 1) out.store(node_index(d, 0, j), NodeV<P>::zero());
@@ -505,17 +509,6 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
                 out.store(o, u);
             }
         };
-        // waveform record of the input level between columns i_e (ul) and i_e + 1 (ur)
-        auto extract = [&](const NodeV<P>& ul, const NodeV<P>& ur) {
-            if (!row_ok) return;
-            double2 a = ul.phi64(), b = ur.phi64();
-            double f = d.f_e;
-            double2 w = wave_lerp(a, b, f);
-            const size_t wi = (size_t)(step % d.wave_cap) * nth + j;
-            if (TK_IN(d.status, wi, d.wave_cap * nth)) d.wave[wi] = w;
-            if (!isfinite(w.x) || !isfinite(w.y)) atomicOr(d.status, (unsigned)ST_NONFINITE);
-        };
-
         // prologue: columns c0-1 (slot 0) and c0 (slot 1)
         C dl_prev, dlm_prev, dl, dlm;
         ring.wait(0);
@@ -534,7 +527,6 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
             if (src_blk) s_first = src_h(c0 - 1);
         }
         HalfRec<T> L = predict(u_prev, u_cur, dl_prev, dl, dlm_prev, dlm, cfh, s_first);
-        if (ex_blk && d.i_e == c0 - 1) extract(u_prev, u_cur);
         u_prev = u_cur;
         dl_prev = dl;
         dlm_prev = dlm;
@@ -572,7 +564,6 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
                 const HalfRec<T> Rh = predict(u_prev, u_cur, dl_prev, dl, dlm_prev, dlm, cfh, s_h);
                 correct(Rh, L, u_prev, cfi, c - 1, xbuf + (c & 1) * xstride, o, s_i);
                 if (threadIdx.x == 0 && c - 2 + R <= c1) ring.fill(d, bin, c - 2 + R, sf);
-                if (ex_blk && d.i_e == c - 1) extract(u_prev, u_cur);
                 L = Rh;
                 u_prev = u_cur;
                 dl_prev = dl;
@@ -625,6 +616,13 @@ __device__ __forceinline__ void step_body(const InstDev& d, int64_t step, int bi
     // first replay) or the graph's last node (after each replay) sets; it does not change
     // while the graph's steps run
     if (d.step_base) step += *d.step_base;
+    // a launch with one block more than pieces takes the record in that block
+    const bool rec_apart = (int64_t)(gridDim.x - 1) * strip >= d.nr - 2;
+    if (rec_apart && blockIdx.x == gridDim.x - 1) {
+        griddep_wait();
+        if (!(*(volatile unsigned*)d.status & ST_TIMEOUT)) record_level<P>(d, step, bin);
+        return;
+    }
     ColumnRing<P, R> ring(step_smem, mbar);
     if (threadIdx.x == 0) ring.init();
     __syncthreads();
@@ -636,7 +634,7 @@ __device__ __forceinline__ void step_body(const InstDev& d, int64_t step, int bi
         c0 = 1 + blockIdx.x * strip;
         c1 = min(d.nr - 1, c0 + strip);
     }
-    strip_step<P, R, true, kMov>(d, step, bin, c0, c1, ring, StepShared<P, R>::xbuf(step_smem));
+    strip_step<P, R, true, kMov>(d, step, bin, c0, c1, !rec_apart, ring, StepShared<P, R>::xbuf(step_smem));
 }
 
 template <class P, bool kMov>
@@ -771,7 +769,7 @@ __global__ void __launch_bounds__(kMaxThreads, kMinBlocks) batched_step_kernel(B
         }
         const int c0 = 1 + st * strip;
         const int c1 = min(d.nr - 1, c0 + strip);
-        strip_step<P, R, false, kMov>(d, b.base_step[k] + s, (int)((b.base_bin[k] + s) & 1), c0, c1, ring, xbuf);
+        strip_step<P, R, false, kMov>(d, b.base_step[k] + s, (int)((b.base_bin[k] + s) & 1), c0, c1, true, ring, xbuf);
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0 && !(s == 0 && r == b.skip_release_item))
@@ -869,7 +867,12 @@ void launch_batched_extract(cudaStream_t st, int prec, const BatchDev& b, int ma
 template <class P, bool kMov>
 static void launch_step_m(cudaStream_t st, const InstDev& d, int64_t step, int bin, int strip,
                           const int* part) {
+    // a grid that leaves a block's place free takes its record in a block of its own: on
+    // 800 x 64 (one-column pieces) the block that also took the record was the step's last
+    // (us per step: FP32-Kahan 4.01 -> 3.49, FP32 3.35 -> 3.09); a full wave has no such
+    // place, and the piece that holds the record is cut shorter (refresh_partition)
     int blocks = (d.nr - 2 + strip - 1) / strip;
+    if (blocks < d.resident) ++blocks;
     int threads = d.pitch;
     // programmatic dependent launch (see step_body)
     cudaLaunchAttribute at[1];
