@@ -80,10 +80,22 @@ __device__ __forceinline__ Z<R> gld(const double2* p, size_t o) {
     return {(R)a.x, (R)a.y};
 }
 
-template <typename T, typename R>
-__device__ __forceinline__ R cget(const T* tab, size_t pl, int k, size_t o) {
-    if constexpr (std::is_same<T, DF>::value) return (R)tab[(size_t)k * pl + o].to_double();
-    else return (R)tab[(size_t)k * pl + o];
+// Coefficients as FP64: all of node (i, j), or coefficient k alone
+template <typename T>
+__device__ __forceinline__ double as64(T v) {
+    if constexpr (std::is_same<T, DF>::value) return v.to_double();
+    else return v;
+}
+template <typename T>
+__device__ __forceinline__ void adj_coefs(const void* tab, int pitch, int i, int j, double* c) {
+    T v[kNCoef];
+    load_coefs<T>(tab, pitch, i, j, v);
+#pragma unroll
+    for (int k = 0; k < kNCoef; ++k) c[k] = as64(v[k]);
+}
+template <typename T>
+__device__ __forceinline__ double adj_coef(const void* tab, int pitch, int i, int j, int k) {
+    return as64(((const T*)tab)[coef_index(pitch, i, j, k)]);
 }
 
 // Compensated add of an increment to one co-state node (FP32): value = v - c.
@@ -143,23 +155,17 @@ struct AdjLin {
     }
 };
 
-// g v for g = +-1 (flip: the sign bit if g < 0), without an FP64 operation
-__device__ __forceinline__ double pole_sign(double v, int flip) {
-    return __hiloint2double(__double2hiint(v) ^ flip, __double2loint(v));
-}
-
 // b + Th^T l at row j, Th the angular and zero-order part of one sub-step, ep (F_{j+1} - F_j)
-// - em (F_j - F_{j-1}) + E3 F with the ghost rows of the pole rule (flip: pole_sign of its
-// factor); lm, l, lp: l at the rows j-1, j, j+1.
+// - em (F_j - F_{j-1}) + E3 F with the ghost rows of the pole rule (flip: flip_sign of its
+// factor); c: the node's coefficients; lm, l, lp: l at the rows j-1, j, j+1.
 template <typename T>
-__device__ __forceinline__ Z<double> theta_cot(const AdjLin& A, Z<double> b, const T* tab, size_t pl, size_t o, int j,
-                                               int nth, Z<double> lm, Z<double> l, Z<double> lp, int flip) {
-    const double ep = cget<T, double>(tab, pl, C_EP, o), em = cget<T, double>(tab, pl, C_EM, o);
-    const double e3 = __fma_rn(em, -A.one, __fma_rn(ep, -A.one, cget<T, double>(tab, pl, C_E3R, o)));
-    b = A.cmac(b, e3, cget<T, double>(tab, pl, C_E3I, o), l);
+__device__ __forceinline__ Z<double> theta_cot(const AdjLin& A, Z<double> b, const double* c, const void* tab,
+                                               int pitch, int i, int j, int nth, Z<double> lm, Z<double> l,
+                                               Z<double> lp, int flip) {
+    b = A.cmac(b, __fma_rn(c[C_EM], -A.one, __fma_rn(c[C_EP], -A.one, c[C_E3R])), c[C_E3I], l);
     const bool lo = j >= 1, hi = j + 1 < nth;
-    b = A.mac(b, lo ? cget<T, double>(tab, pl, C_EP, o - 1) : pole_sign(em, flip), lo ? lm : l);
-    return A.mac(b, hi ? cget<T, double>(tab, pl, C_EM, o + 1) : pole_sign(ep, flip), hi ? lp : l);
+    b = A.mac(b, lo ? adj_coef<T>(tab, pitch, i, j - 1, C_EP) : flip_sign(c[C_EM], flip), lo ? lm : l);
+    return A.mac(b, hi ? adj_coef<T>(tab, pitch, i, j + 1, C_EM) : flip_sign(c[C_EP], flip), hi ? lp : l);
 }
 
 // The co-state of one node as stored: FP64 value, or FP32 (v, c) pairs with value v - c.
@@ -256,7 +262,7 @@ __global__ void __launch_bounds__(kSrcGradThreads) adj_src_grad_kernel(InstDev d
     if (t != 0) return;
     const double A = (s.amps != nullptr && n < s.n_amps) ? s.amps[n] : 1.0;
     auto re_mul = [](Z<double> a, double bx, double by) { return a.x * bx - a.y * by; };
-    const double hd = 0.5 * d.dt;
+    const double hd = sizeof(R) == 8 ? d.dt : 0.5 * d.dt;   // (FP64: the window holds mu_Pi / 2)
     gA[k] = hd * re_mul(ph[0], S[0], S[1]) + d.dt * re_mul(ph[1], S[4], S[5]);
     gR[k] = A * (hd * (re_mul(ph[2], S[0], S[1]) + re_mul(ph[0], S[2], S[3])) +
                  d.dt * (re_mul(ph[3], S[4], S[5]) + re_mul(ph[1], S[6], S[7])));
@@ -282,9 +288,9 @@ __device__ __forceinline__ void adj_wait_prev() { asm volatile("griddepcontrol.w
 //   half node h, mu:        cs = mu_Phi + Th^T mu_Pi, cd = -G mu_Phi + conj(E2) mu_Pi,
 //                           csP = (dt/2) mu_Phi + mu_Pi + conj(E1) mu_Pi, cdP = G mu_Pi
 //     lam_Phi += cs +- cd, lam_Pi += csP +- cdP  at the nodes right (+) and left (-) of h
-// 76 FP64 operations a node instead of 190 (4096 x 128: 195 -> 111 us a reverse step, double-float
-// instances 360 -> 204).  mu here is the cotangent of
-// 2 h, so the source window gets 2 mu_Pi.
+// 76 FP64 operations a node instead of 190 (4096 x 128: 195 -> 106 us a reverse step, double-float
+// instances 360 -> 198).  mu here is the cotangent of
+// 2 h (adj_src_grad_kernel doubles it).
 template <typename T, int kMaxT>
 __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin, const double2* gbar,
                                                          CoLevel lout, int strip, void* wh, void* wi) {
@@ -296,11 +302,8 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
     const int j = threadIdx.x, nth = d.nth, nr = d.nr, pitch = d.pitch;
     const bool row_ok = j < nth;
     const int c0 = blockIdx.x * strip, c1 = min(nr, c0 + strip);   // output columns [c0, c1)
-    const T* ci = (const T*)d.coef_i;
-    const T* ch = (const T*)d.coef_h;
-    const size_t pl = plane_elems(d);
-    const double hdt = 0.5 * d.dt, qdt = 0.25 * d.dt, w_e = 1.0 - d.f_e, w_e1 = d.f_e;
-    const int flip = d.ghost < 0.0 ? (int)0x80000000 : 0;
+    const double hdt = d.hdt, qdt = d.qdt;
+    const int flip = pole_flip(d);
     const AdjLin A{d.one};
     const SourceDev& s = d.src;
     const Zd zero = {0, 0};
@@ -321,14 +324,14 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
     auto node_shares = [&](const CoNode<double>& L, int col, Zd& rF, Zd& rP, Zd& lF, Zd& lP) {
         rF = rP = lF = lP = zero;
         if (!row_ok || col < 1 || col > nr - 2) return;
-        const size_t o = node_index(d, col, j);
+        double c[kNCoef];
+        adj_coefs<T>(d.coef_i, pitch, col, j, c);
         Zd lm, lp;
         nb3(LB, col & 1, lm, lp);
-        const double G = cget<T, double>(ci, pl, C_G, o);
-        const Zd cS = theta_cot<T>(A, zero, ci, pl, o, j, nth, lm, L.P, lp, flip);
-        const Zd cD = A.cmac(A.mac(zero, -G, L.F), cget<T, double>(ci, pl, C_E2R, o), cget<T, double>(ci, pl, C_E2I, o), L.P);
-        const Zd cSP = A.cmac(A.mac(zero, qdt, L.F), cget<T, double>(ci, pl, C_E1R, o), cget<T, double>(ci, pl, C_E1I, o), L.P);
-        const Zd cDP = A.mac(zero, G, L.P);
+        const Zd cS = theta_cot<T>(A, zero, c, d.coef_i, pitch, col, j, nth, lm, L.P, lp, flip);
+        const Zd cD = A.cmac(A.mac(zero, -c[C_G], L.F), c[C_E2R], c[C_E2I], L.P);
+        const Zd cSP = A.cmac(A.mac(zero, qdt, L.F), c[C_E1R], c[C_E1I], L.P);
+        const Zd cDP = A.mac(zero, c[C_G], L.P);
         rF = A.add(cS, cD);
         lF = A.sub(cS, cD);
         rP = A.add(cSP, cDP);
@@ -355,24 +358,24 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
                                           // the previous block's)
             const int a = h - s.h_lo, bb = j - s.j_lo;
             if ((unsigned)a < (unsigned)s.nh && (unsigned)bb < (unsigned)s.nj)
-                stv<double>(wh, (size_t)bb * s.nh + a, A.add(muP, muP));
+                stv<double>(wh, (size_t)bb * s.nh + a, muP);
         }
         MB[(size_t)(h & 1) * pitch + j] = muP;
         __syncthreads();
         // the shares of half node h of the nodes h (left) and h+1 (right)
         Zd tF = zero, tP = zero, nF = zero, nP = zero;
         if (half_ok) {
-            const size_t oh = node_index(d, h, j);
+            double c[kNCoef];
+            adj_coefs<T>(d.coef_h, pitch, h, j, c);
             Zd mm, mp;
             nb3(MB, h & 1, mm, mp);
-            const double G = cget<T, double>(ch, pl, C_G, oh);
-            const Zd cs = theta_cot<T>(A, muF, ch, pl, oh, j, nth, mm, muP, mp, flip);
-            const Zd cd = A.cmac(A.mac(zero, -G, muF), cget<T, double>(ch, pl, C_E2R, oh), cget<T, double>(ch, pl, C_E2I, oh), muP);
-            const Zd csP = A.cmac(A.mac(muP, hdt, muF), cget<T, double>(ch, pl, C_E1R, oh), cget<T, double>(ch, pl, C_E1I, oh), muP);
+            const Zd cs = theta_cot<T>(A, muF, c, d.coef_h, pitch, h, j, nth, mm, muP, mp, flip);
+            const Zd cd = A.cmac(A.mac(zero, -c[C_G], muF), c[C_E2R], c[C_E2I], muP);
+            const Zd csP = A.cmac(A.mac(muP, hdt, muF), c[C_E1R], c[C_E1I], muP);
             tF = A.sub(cs, cd);
             nF = A.add(cs, cd);
-            tP = A.mac(csP, -G, muP);
-            nP = A.mac(csP, G, muP);
+            tP = A.mac(csP, -c[C_G], muP);
+            nP = A.mac(csP, c[C_G], muP);
         }
         // lam^n at column h
         if (h >= c0 && row_ok) {
@@ -383,11 +386,7 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
                 aF = A.add(l_cur.F, aF);
                 aP = A.add(l_cur.P, aP);
             }
-            if (gbar) {   // transpose of the linear extraction between i_e and i_e + 1
-                if (h == d.i_e) aF = zadd(aF, zscale(w_e, gld<double>(gbar, j)));
-                if (h == d.i_e + 1) aF = zadd(aF, zscale(w_e1, gld<double>(gbar, j)));
-            }
-            if (TK_IN(d.status, o, pl)) {
+            if (TK_IN(d.status, o, plane_elems(d))) {
                 stv<double>(lout.F, o, aF);
                 stv<double>(lout.P, o, aP);
             }
@@ -402,6 +401,18 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
         muP_part = muP_next;
         aF_part = nF;
         aP_part = nP;
+    }
+    // transpose of the linear extraction between i_e and i_e + 1, added to this row's own
+    // values (in the loop its operations would run, predicated off, at every column)
+    if (gbar && row_ok) {
+        for (int e = 0; e < 2; ++e) {
+            const int col = d.i_e + e;
+            const size_t o = node_index(d, col, j);
+            if (col < c0 || col >= c1 || !TK_IN(d.status, o, plane_elems(d))) continue;
+            const double w = e ? d.f_e : 1.0 - d.f_e;
+            const Zd gb = gld<double>(gbar, j);
+            stv<double>(lout.F, o, zadd(ldv<double>(lout.F, o), zscale(w, gb)));
+        }
     }
 }
 
@@ -445,7 +456,7 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel 
     const bool row_ok = j < nth;
     const int c0 = blockIdx.x * strip, c1 = min(nr, c0 + strip);   // output columns [c0, c1)
     const bool rt_smem = strip + 2 <= kAdjRtCols;   // else the tables are read from global
-    const R g = (R)d.ghost, hdt = (R)(0.5 * d.dt), qdt = (R)(0.5 * d.dt);
+    const R g = d.ghost_f, hdt = d.hdt2.x, qdt = d.hdt2.x;
     const SourceDev& s = d.src;
     // wh, wi: this step's ring slot of the window co-states (null: no source)
     RowTab<PK> rt;

@@ -263,6 +263,12 @@ InstDev dev_of(const teuk_ctx* c, const Instance& I) {
     d.ghost = (std::abs(I.p.m + I.p.s) % 2 == 0) ? 1.0 : -1.0;
     d.ghost_f = (float)d.ghost;
     d.one = 1.0;
+    d.hdt = 0.5 * I.dt;
+    d.qdt = 0.25 * I.dt;
+    const DF h2(d.hdt), q2(d.qdt);
+    d.hdt2 = make_float2(h2.hi, h2.lo);
+    d.qdt2 = make_float2(q2.hi, q2.lo);
+    d.dt_f = (float)I.dt;
     for (int b = 0; b < 2; ++b)
         for (int k = 0; k < 2; ++k) d.buf[b][k] = I.state[b][k];
     d.coef_h = I.coef_h;

@@ -10,9 +10,10 @@
 //                         the represented value being hi - c
 //             FP64_DF     plane 0 = hi {Phi, Pi} (float4), plane 1 = lo {Phi, Pi} (float4),
 //                         the value being hi + lo (double-float)
-//   coef_h  [9][n_rstar][pitch] FP64 (double) and FP64_DF ((hi, lo) float pairs) paths:
-//           predictor coefficients at half nodes (i+1/2, j)
-//   coef_i  [9][n_rstar][pitch] the same at integer nodes (i, j)
+//   coef_h  [n_rstar][pitch / 32][9][32] FP64 (double) and FP64_DF ((hi, lo) float pairs)
+//           paths: predictor coefficients at half nodes (i+1/2, j), a warp's 32 rows of one
+//           column in one tile (coef_index)
+//   coef_i  the same at integer nodes (i, j)
 //   source  FP64 complex profile on a window of nodes around the particle
 //   wave    FP64 ring of waveform records [capacity][n_theta] (double2)
 #pragma once
@@ -34,6 +35,17 @@ constexpr int kPitchAlign = 32;  // elements
 //   6:   em = sd w (1/dth^2 - cot/(2 dth))       (backward theta difference)
 //   7,8: E3 = sd (q - w V)                       (zero-order term)
 enum CoefIdx { C_G = 0, C_E1R, C_E1I, C_E2R, C_E2I, C_EP, C_EM, C_E3R, C_E3I };
+
+// Element of coefficient k of node (i, j) in a coefficient table.  The 32 rows of one warp
+// and column form a tile of 9 x 32 elements: the pairs (E1R, E1I), (E2R, E2I), (EP, EM),
+// (E3R, E3I), one 16-byte pair a row, then G.  A node is then four 16-byte loads and one
+// of 8 bytes at fixed offsets from one address, where nine planes took nine loads at nine
+// addresses (load_coefs).
+__host__ __device__ inline size_t coef_index(int pitch, int i, int j, int k) {
+    const size_t tile = ((size_t)i * (size_t)pitch + (size_t)(j & ~31)) * kNCoef;
+    const int l = j & 31;
+    return k == C_G ? tile + 256 + l : tile + ((k - 1) >> 1) * 64 + 2 * l + ((k - 1) & 1);
+}
 
 struct SourceDev {
     int on;
@@ -89,8 +101,14 @@ struct InstDev {
     float ghost_f;            // +1 even |m + s|, -1 odd |m + s|
     double ghost;
     double one;               // 1.0, as a value the compiler does not know (see Lin)
+    // dt/2 and dt/4 in the arithmetic types, formed on the host: formed in the kernels, the
+    // compiler repeats the FP64 conversions at every column to save a register, 1 (FP32) to
+    // 14 (double-float) instructions a node on the FP64 pipe (see step_hdt)
+    double hdt, qdt;
+    float2 hdt2, qdt2;        // (hi, lo)
+    float dt_f, pad_f;
     void* buf[2][2];          // [ping-pong buffer][plane]
-    const void* coef_h;       // [9][nr][pitch] (double or float)
+    const void* coef_h;       // tiles of double or (hi, lo) float pairs (coef_index)
     const void* coef_i;
     const RTab2* rtab;        // [nr] FP32 paths: radial tables (half node, node) per column
     const ThTab* thtab;       // [nth]

@@ -113,8 +113,9 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
     const int jp = j + 1 < nth ? j + 1 : j, jm = j > 0 ? j - 1 : 0;
     const T g = (T)d.ghost;
     const T gp = top ? g : T(1), gm = bot ? g : T(1);
-    const T hdt = (T)(0.5 * d.dt), fdt = (T)d.dt, qdt = (T)(0.25 * d.dt);
+    const T hdt = step_hdt<T>(d), fdt = (T)d.dt, qdt = step_qdt<T>(d);
     const Lin<T> A(d);
+    const PoleRow pole(d, j);
     const bool has_l = b > 0, has_r = b < r.nb - 1;
 
     using L = ResLayout<P>;
@@ -166,12 +167,9 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
                 mine[q] = cf2[q].x;
                 mine[kNCoef + q] = cf2[q].y;
             }
-        } else if constexpr (P::kind == kDF) {
-            coefs_df(d, true, col, j, (DF*)mine);
-            coefs_df(d, false, col, j, (DF*)(mine + kNCoef));
         } else {
-            coefs64(d, true, col, j, (double*)mine);
-            coefs64(d, false, col, j, (double*)(mine + kNCoef));
+            coefs2d<T>(d, true, col, j, mine);
+            coefs2d<T>(d, false, col, j, mine + kNCoef);
         }
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -297,8 +295,8 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
                     const C sm = A.add(ul.F, ur.F);
                     C s_p = A.add(S.load_phi(sidx(k, jp)).F, S.load_phi(sidx(k + 1, jp)).F);
                     C s_m = A.add(S.load_phi(sidx(k, jm)).F, S.load_phi(sidx(k + 1, jm)).F);
-                    if (top) s_p = g * s_p;
-                    if (bot) s_m = g * s_m;
+                    if (top) s_p = flip_sign(s_p, pole.flip);
+                    if (bot) s_m = flip_sign(s_m, pole.flip);
                     T cf[kNCoef];
 #pragma unroll
                     for (int q = 0; q < kNCoef; ++q) cf[q] = CF[sidx(k, j) * 2 * kNCoef + q];
@@ -318,7 +316,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
                     xpublish(xb, xb + 4 * (j + 1), row, g, row_ok, top, bot);
                 } else {
                     unsigned char* xb = (unsigned char*)(X + (size_t)k * (pitch + 2) * 4);
-                    publish16<T>(xb, j, A.add(HX[sidx(k, j)].F, HX[sidx(k - 1, j)].F), g, row_ok, top, bot);
+                    publish16<T>(xb, j, A.add(HX[sidx(k, j)].F, HX[sidx(k - 1, j)].F), pole, row_ok);
                 }
             }
             __syncthreads();

@@ -109,21 +109,19 @@ __global__ void coef_kernel(double M, double a, int s, int m, double rstar_min, 
     int j = blockIdx.y * blockDim.x + threadIdx.x;   // theta row (fastest in memory)
     int i = blockIdx.x;                              // r* column (grid x: up to 2^31 - 1)
     if (j >= pitch || i >= nr) return;
-    size_t pl = (size_t)nr * pitch;
-    size_t o = (size_t)i * pitch + j;
     double th = (j + 0.5) * dth;
     double c[kNCoef];
     if (j < nth && i < nr - 1) {
         node_coefficients(M, a, s, m, x_half[i], th, dth, dt, drs, 0.5, 1.0, c);
-        for (int k = 0; k < kNCoef; ++k) coef_h[k * pl + o] = (T)c[k];
+        for (int k = 0; k < kNCoef; ++k) coef_h[coef_index(pitch, i, j, k)] = (T)c[k];
     } else {
-        for (int k = 0; k < kNCoef; ++k) coef_h[k * pl + o] = (T)0;
+        for (int k = 0; k < kNCoef; ++k) coef_h[coef_index(pitch, i, j, k)] = (T)0;
     }
     if (j < nth) {
         node_coefficients(M, a, s, m, x_int[i], th, dth, dt, drs, 0.25, 0.5, c);
-        for (int k = 0; k < kNCoef; ++k) coef_i[k * pl + o] = (T)c[k];
+        for (int k = 0; k < kNCoef; ++k) coef_i[coef_index(pitch, i, j, k)] = (T)c[k];
     } else {
-        for (int k = 0; k < kNCoef; ++k) coef_i[k * pl + o] = (T)0;
+        for (int k = 0; k < kNCoef; ++k) coef_i[coef_index(pitch, i, j, k)] = (T)0;
     }
 }
 

@@ -246,8 +246,9 @@ __device__ __forceinline__ void strip_columns_x(const InstDev& d, int64_t step, 
     using C = Cx<T>;
     const Lin<T> A(d);
     const int j = threadIdx.x, nth = d.nth;
-    const bool row_ok = j < nth, bot = j == 0, top = j == nth - 1;
-    const T g = (T)d.ghost, hdt = (T)(0.5 * d.dt), qdt = (T)(0.25 * d.dt);
+    const bool row_ok = j < nth;
+    const PoleRow pole(d, j);
+    const T hdt = step_hdt<T>(d), qdt = step_qdt<T>(d);
     const Planes<P> out = Planes<P>::of(d, 1 - bin);
     // exchange entries: [column parity][S, s][threads + 2] of 16 bytes
     const unsigned xs = 16u * (blockDim.x + 2u);
@@ -263,9 +264,7 @@ __device__ __forceinline__ void strip_columns_x(const InstDev& d, int64_t step, 
         if (threadIdx.x == 0 && col + R <= c1) ring.fill(d, bin, col + R, slot);
     };
     auto coefs = [&](bool half, int col, T* cf) {
-        if (!TK_IN(d.status, col, d.nr)) return;
-        if constexpr (P::kind == kDF) coefs_df(d, half, col, j, (DF*)cf);
-        else coefs64(d, half, col, j, (double*)cf);
+        if (TK_IN(d.status, col, d.nr)) coefs2d<T>(d, half, col, j, cf);
     };
     auto term_h = [&](int h) { return kMov && moving ? msrc_h(h) : src_h(h); };
     auto term_i = [&](int i) { return kMov && moving ? msrc_i(i) : src_i(i); };
@@ -278,8 +277,8 @@ __device__ __forceinline__ void strip_columns_x(const InstDev& d, int64_t step, 
     ring.wait(2);
     NodeV<P> u_next = node(2);
     C s0 = A.add(u_prev.F, u_cur.F), s = A.add(u_cur.F, u_next.F);
-    publish16<T>(xS(c0), j, s0, g, row_ok, top, bot);
-    publish16<T>(xs_(c0), j, s, g, row_ok, top, bot);
+    publish16<T>(xS(c0), j, s0, pole, row_ok);
+    publish16<T>(xs_(c0), j, s, pole, row_ok);
     __syncthreads();
     for (int k = 0; k < 3; ++k) refill(c0 - 1 + k, k);
     HalfX<T> L;
@@ -297,32 +296,41 @@ __device__ __forceinline__ void strip_columns_x(const InstDev& d, int64_t step, 
     auto steady = [&](auto src_kind) {
         constexpr bool kSrc = decltype(src_kind)::value;
         int slot = 3 % R;   // of column c + 1
+        // double-float: coefficients one phase ahead of use, the corrector's loaded before
+        // the predictor, the next half node's after it (16384 x 256: 200 -> 169 us per step).
+        // FP64 has the FP64 pipe to wait for and loads them where they are used (570 us
+        // per step; one phase ahead 577)
+        constexpr bool kAhead = P::kind == kDF;
+        T cf[kNCoef], ci[kNCoef];
+        if constexpr (kAhead) coefs(true, c0, cf);
 #pragma unroll 2
         for (int c = c0 + 1; c <= c1; ++c) {
             // half node c-1/2 = (c-1, c): u_cur holds c-1, u_next column c
             C p, m;
+            if constexpr (kAhead) coefs(false, c - 1, ci);
+            else coefs(true, c - 1, cf);
             nbr(xs_(c - 1), p, m);
-            T cf[kNCoef];
-            coefs(true, c - 1, cf);
             C src = C::zero();
             if constexpr (kSrc) src = term_h(c - 1);
             const HalfX<T> Rh = predict_x<T, kSrc>(A, u_cur.F, u_cur.Pp, u_next.F, u_next.Pp, s, p, m, cf, hdt, src);
+            if constexpr (kAhead) {
+                if (c < c1) coefs(true, c, cf);
+            }
             const C S = A.add(Rh.F, L.F);
-            publish16<T>(xS(c), j, S, g, row_ok, top, bot);
+            publish16<T>(xS(c), j, S, pole, row_ok);
             const NodeV<P> u = u_cur;
             u_cur = u_next;
             if (c < c1) {
                 ring.wait(slot);
                 u_next = node(slot);
                 s = A.add(u_cur.F, u_next.F);
-                publish16<T>(xs_(c), j, s, g, row_ok, top, bot);
+                publish16<T>(xs_(c), j, s, pole, row_ok);
             }
             __syncthreads();
             if (c < c1) refill(c + 1, slot);
             C S_p, S_m;
             nbr(xS(c), S_p, S_m);
-            T ci[kNCoef];
-            coefs(false, c - 1, ci);
+            if constexpr (!kAhead) coefs(false, c - 1, ci);
             C srcc = C::zero();
             if constexpr (kSrc) srcc = term_i(c - 1);
             C dPhi, dPi;
@@ -366,18 +374,9 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
     const int j = threadIdx.x;
     const int nth = d.nth;
     const bool row_ok = j < nth;
-    const bool bot = j == 0, top = j == nth - 1;
-    // theta neighbours in the slot, the pole rows standing in for the ghost rows: row
-    // nth = g * row nth-1 and row -1 = g * row 0 (gp, gm the factors)
-    const int jp = j + 1 < nth ? j + 1 : j, jm = j > 0 ? j - 1 : 0;
-    const T g = (T)d.ghost;
-    const T gp = top ? g : T(1), gm = bot ? g : T(1);
-    const T hdt = (T)(0.5 * d.dt), fdt = (T)d.dt;
     const Planes<P> out = Planes<P>::of(d, 1 - bin);
-    const unsigned xstride = 4u * (blockDim.x + 2u);
     RowTab<P> rt;
     rt.load(d.thtab, j, row_ok);
-    const size_t pitch = (size_t)d.pitch;
 
     // source: this block's columns against the window
     const SourceDev& sw = d.src;
@@ -459,6 +458,15 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
         return source_int<T>(sw, g * sc_fac, i, j);
     };
     if constexpr (kSplit) {
+        const bool bot = j == 0, top = j == nth - 1;
+        // theta neighbours in the slot, the pole rows standing in for the ghost rows: row
+        // nth = g * row nth-1 and row -1 = g * row 0 (gp, gm the factors)
+        const int jp = j + 1 < nth ? j + 1 : j, jm = j > 0 ? j - 1 : 0;
+        const T g = d.ghost_f;
+        const T gp = top ? g : T(1), gm = bot ? g : T(1);
+        const T hdt = step_hdt<T>(d), fdt = d.dt_f;
+        const unsigned xstride = 4u * (blockDim.x + 2u);
+        const size_t pitch = (size_t)d.pitch;
         // own node of the column in slot s (rows past nth read slot padding: their results
         // are never stored or exchanged)
         auto node = [&](int s) { return ring.planes(s).load((size_t)j); };

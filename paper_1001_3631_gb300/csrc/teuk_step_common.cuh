@@ -420,7 +420,9 @@ __host__ __device__ constexpr bool split_angular() { return P::kind == kFP32 || 
 // both), because both increments of the state are formed apart and added once.  16384 x 256,
 // us per step before and after: FP64 947 -> 629, double-float 262 -> 205 (681 -> 506 paired
 // FP32 operations a node, and no register spills: the record of a half node is two complex
-// values instead of eight).
+// values instead of eight); with the time steps formed on the host and the pole factor
+// applied to the sign bits (85 -> 75 FP64 instructions a node, and 14 -> 0 on the
+// double-float path) and double-float coefficients loaded ahead: FP64 570, double-float 148.
 
 // Complex sums and differences.  FP64: as DFMA with a factor one that the compiler cannot
 // see (DADD and DMUL take 19 clocks of the SM's FP64 pipe, DFMA 16; the rounding is the
@@ -505,14 +507,45 @@ __device__ __forceinline__ Cx<T> get16(const void* e) {
         return {T(v.x, v.z), T(v.y, v.w)};
     }
 }
-// Publish this row's value (row j at entry j + 1 of x) and, for the pole rows, the ghost
-// rows' entries 0 and n_theta + 1 (the row times the pole factor g = +-1)
+// +-v, by the sign bits (flip: 0 or the sign bit), without an operation on the FP64 or FMA
+// pipe
+__device__ __forceinline__ float flip_sign(float v, int flip) { return __int_as_float(__float_as_int(v) ^ flip); }
+__device__ __forceinline__ double flip_sign(double v, int flip) {
+    return __hiloint2double(__double2hiint(v) ^ flip, __double2loint(v));
+}
+__device__ __forceinline__ DF flip_sign(DF v, int flip) { return DF(flip_sign(v.hi, flip), flip_sign(v.lo, flip)); }
 template <typename T>
-__device__ __forceinline__ void publish16(unsigned char* x, int j, Cx<T> v, T g, bool row_ok, bool top, bool bot) {
-    unsigned char* mine = x + 16 * (j + 1);
-    if (row_ok) put16(mine, v);
-    if (top) put16(mine + 16, g * v);
-    if (bot) put16(x, g * v);
+__device__ __forceinline__ Cx<T> flip_sign(Cx<T> v, int flip) { return {flip_sign(v.re, flip), flip_sign(v.im, flip)}; }
+// flip of the pole factor
+__device__ __forceinline__ int pole_flip(const InstDev& d) { return d.ghost_f < 0.f ? (int)0x80000000 : 0; }
+
+// The pole rows of a column (0 and n_theta - 1, distinct: n_theta >= 4) and the exchange
+// entry of the ghost row beyond each (0 and n_theta + 1)
+struct PoleRow {
+    bool edge;
+    int entry, flip;
+    __device__ __forceinline__ PoleRow(const InstDev& d, int j)
+        : edge(j == 0 || j == d.nth - 1), entry(j == 0 ? 0 : d.nth + 1), flip(pole_flip(d)) {}
+};
+// Publish this row's value (row j at entry j + 1 of x) and, for a pole row, its ghost row's
+template <typename T>
+__device__ __forceinline__ void publish16(unsigned char* x, int j, Cx<T> v, const PoleRow& pole, bool row_ok) {
+    if (row_ok) put16(x + 16 * (j + 1), v);
+    if (pole.edge) put16(x + 16 * pole.entry, flip_sign(v, pole.flip));
+}
+
+// dt/2 and dt/4 in the arithmetic type
+template <typename T>
+__device__ __forceinline__ T step_hdt(const InstDev& d) {
+    if constexpr (uses_pairs<T>()) return T(d.hdt2.x, d.hdt2.y);
+    else if constexpr (sizeof(T) == 4) return d.hdt2.x;
+    else return d.hdt;
+}
+template <typename T>
+__device__ __forceinline__ T step_qdt(const InstDev& d) {
+    if constexpr (uses_pairs<T>()) return T(d.qdt2.x, d.qdt2.y);
+    else if constexpr (sizeof(T) == 4) return d.qdt2.x;
+    else return d.qdt;
 }
 
 // ---------------------------------------------------------------- split form
@@ -544,11 +577,30 @@ __device__ __forceinline__ CRow<T> combine_lr(const HalfRec<T>& R, const HalfRec
     return c;
 }
 
-// (rows past n_theta read the padding of the tables: in bounds, never used)
+// Coefficients of node (i, j) from a 2D table (rows past n_theta read its padding: in
+// bounds, never used)
 template <typename T>
-__device__ __forceinline__ void load_coefs(const T* tab, size_t pl, size_t o, T* cf) {
+__device__ __forceinline__ void load_coefs(const void* tab, int pitch, int i, int j, T* cf) {
+    const char* p = (const char*)tab + ((size_t)i * (size_t)pitch + (size_t)(j & ~31)) * (kNCoef * 8u);
+    const int l = j & 31;
 #pragma unroll
-    for (int k = 0; k < kNCoef; ++k) cf[k] = __ldg(tab + k * pl + o);
+    for (int q = 0; q < 4; ++q) {
+        if constexpr (uses_pairs<T>()) {
+            const float4 v = __ldg((const float4*)(p + 512 * q) + l);
+            cf[1 + 2 * q] = T(v.x, v.y);
+            cf[2 + 2 * q] = T(v.z, v.w);
+        } else {
+            const double2 v = __ldg((const double2*)(p + 512 * q) + l);
+            cf[1 + 2 * q] = v.x;
+            cf[2 + 2 * q] = v.y;
+        }
+    }
+    if constexpr (uses_pairs<T>()) {
+        const float2 v = __ldg((const float2*)(p + 2048) + l);
+        cf[C_G] = T(v.x, v.y);
+    } else {
+        cf[C_G] = __ldg((const double*)(p + 2048) + l);
+    }
 }
 
 // The theta table of one row as broadcast pairs (x, x), held in registers by its thread
@@ -591,20 +643,11 @@ __device__ __forceinline__ void form_coefs2(const RTab2& t, const ThPair& h, flo
     cf[C_E3I] = __fmul2_rn(t.qi, iS);
 }
 
-// FP64 coefficients of the predictor (half = true, node i+1/2) or the corrector (node i)
-// at row j, from the 2D tables.
-__device__ __forceinline__ void coefs64(const InstDev& d, bool half, int i, int j, double* cf) {
-    load_coefs((const double*)(half ? d.coef_h : d.coef_i), plane_elems(d), node_index(d, i, j), cf);
-}
-// Double-float coefficients (FP64-equivalent path), from its 2D tables of (hi, lo) pairs.
-__device__ __forceinline__ void coefs_df(const InstDev& d, bool half, int i, int j, DF* cf) {
-    const float2* tab = (const float2*)(half ? d.coef_h : d.coef_i);
-    const size_t pl = plane_elems(d), o = node_index(d, i, j);
-#pragma unroll
-    for (int k = 0; k < kNCoef; ++k) {
-        const float2 v = __ldg(tab + k * pl + o);
-        cf[k] = DF(v.x, v.y);
-    }
+// FP64 or double-float coefficients of the predictor (half = true, node i+1/2) or the
+// corrector (node i) at row j, from the 2D tables.
+template <typename T>
+__device__ __forceinline__ void coefs2d(const InstDev& d, bool half, int i, int j, T* cf) {
+    load_coefs<T>(half ? d.coef_h : d.coef_i, d.pitch, i, j, cf);
 }
 
 // Eq. (13) at the own half node, as an increment on the averaged state.  Dp, Dm: its second
