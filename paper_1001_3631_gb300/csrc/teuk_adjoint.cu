@@ -22,6 +22,7 @@
 // condition.  The co-state lam and mu are FP64 for FP64 instances; for FP32 instances
 // they are FP32, lam compensated like the forward state (value hi - c, each step's
 // increment added with Kahan's compensated sum), the gradient sums FP64 either way.
+#include <algorithm>
 #include <type_traits>
 
 #include "teuk_df.cuh"
@@ -288,12 +289,12 @@ __device__ __forceinline__ void adj_wait_prev() { asm volatile("griddepcontrol.w
 //   half node h, mu:        cs = mu_Phi + Th^T mu_Pi, cd = -G mu_Phi + conj(E2) mu_Pi,
 //                           csP = (dt/2) mu_Phi + mu_Pi + conj(E1) mu_Pi, cdP = G mu_Pi
 //     lam_Phi += cs +- cd, lam_Pi += csP +- cdP  at the nodes right (+) and left (-) of h
-// 76 FP64 operations a node instead of 190 (4096 x 128: 195 -> 106 us a reverse step, double-float
-// instances 360 -> 198).  mu here is the cotangent of
+// 76 FP64 operations a node instead of 190 (4096 x 128: 195 -> 89 us a reverse step, double-float
+// instances 360 -> 161).  mu here is the cotangent of
 // 2 h (adj_src_grad_kernel doubles it).
 template <typename T, int kMaxT>
 __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin, const double2* gbar,
-                                                         CoLevel lout, int strip, void* wh, void* wi) {
+                                                         CoLevel lout, int /*strip*/, void* wh, void* wi) {
     using Zd = Z<double>;
     extern __shared__ __align__(16) unsigned char adj_smem[];
     adj_release_next();
@@ -301,7 +302,8 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
     Zd* MB = LB + 2 * (size_t)d.pitch;         // [2][pitch] mu_Pi of a half node
     const int j = threadIdx.x, nth = d.nth, nr = d.nr, pitch = d.pitch;
     const bool row_ok = j < nth;
-    const int c0 = blockIdx.x * strip, c1 = min(nr, c0 + strip);   // output columns [c0, c1)
+    // output columns [c0, c1): one of gridDim.x pieces of equal length to a column
+    const int c0 = (int)((int64_t)blockIdx.x * nr / gridDim.x), c1 = (int)((int64_t)(blockIdx.x + 1) * nr / gridDim.x);
     const double hdt = d.hdt, qdt = d.qdt;
     const int flip = pole_flip(d);
     const AdjLin A{d.one};
@@ -708,17 +710,33 @@ static void adj_dispatch(int prec, int t, F f) {
     }
 }
 
-int adj_step_plan(const InstDev& d, int* strip) {
+// The cut of the reverse step.  FP64 co-state: a whole number of blocks on every SM, two or
+// three of them, each with the same number of columns.  It is bound by the FP64 pipe of
+// the SM that has most blocks, and consecutive steps overlap (programmatic dependent
+// launch), so that any other number piles the next step's blocks on the SMs that happen to
+// be free: 1024 x 64 in 256 strips of 4 columns took 66 us a step, in 304 pieces 20; 2048 x
+// 128 in 512 strips 85, in 304 pieces 49; 4096 x 128 in 820 strips 106, in 456 pieces 88 (304:
+// 102).  More blocks have more columns at their edges computed twice; two an SM hide too
+// little latency once a piece is longer than some six columns.
+// FP32 co-state: one wave of strips of at least four columns.
+AdjCut adj_step_plan(const InstDev& d) {
     int res = 1;
     adj_dispatch(d.prec, d.pitch, [&](auto kernel, size_t sm) {
         // (blocks of more than 256 rows take more than the default 48 KB)
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         res = adj_resident(kernel, d.pitch, sm);
     });
+    if (d.prec == 0 || d.prec == 3) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (sms < 1) sms = 1;
+        const int per = std::min(res / sms, d.nr >= 6 * 3 * sms ? 3 : 2);
+        return {0, std::max(1, std::min(per * sms, d.nr / 2))};
+    }
     int L = (d.nr + res - 1) / res;   // one wave of resident blocks, >= 4 columns each
     if (L < 4) L = 4;
-    *strip = L;
-    return (d.nr + L - 1) / L;
+    return {L, (d.nr + L - 1) / L};
 }
 
 template <class K>
@@ -738,10 +756,9 @@ static void adj_launch(cudaStream_t st, K kernel, int nb, int t, size_t sm, cons
 }
 
 void launch_adj_step(cudaStream_t st, const InstDev& d, const CoLevel& lin, const double2* gbar,
-                     const CoLevel& lout, int strip, void* wh, void* wi) {
-    const int nb = (d.nr + strip - 1) / strip;
+                     const CoLevel& lout, const AdjCut& cut, void* wh, void* wi) {
     adj_dispatch(d.prec, d.pitch, [&](auto kernel, size_t sm) {
-        adj_launch(st, kernel, nb, d.pitch, sm, d, lin, gbar, lout, strip, wh, wi);
+        adj_launch(st, kernel, cut.nb, d.pitch, sm, d, lin, gbar, lout, cut.strip, wh, wi);
     });
 }
 

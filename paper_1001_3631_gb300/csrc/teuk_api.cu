@@ -1,6 +1,7 @@
 // teuk_api.cu -- the C ABI of include/teuk.h: argument validation, device memory
 // (stream-ordered allocation on the caller's stream), kernel launches and copies.
 // No arithmetic of the time step happens on the host.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -21,9 +22,7 @@ constexpr double kPi = 3.141592653589793238462643;
 // The launch configuration a per-step graph captured (compared byte for byte).
 struct StepGraphKey {
     InstDev d;
-    const int* part;
-    int strip;
-    int pad;
+    StepCut cut;
 };
 
 struct Instance {
@@ -62,6 +61,7 @@ struct Instance {
     int* d_part = nullptr;
     std::vector<int> h_part;
     int part_strip = 0;
+    int part_nb = 0, part_cap = 0;   // its pieces, and the cap on blocks an SM (StepCut)
     int fault_col = -1;         // testing aid (teuk_set_fill_fault)
     // slab of a larger grid (teuk_params.slab_ncols > 0): local column k is grid column
     // k + off; local columns 0 and n_rstar - 1 are halos (or the grid's own ends)
@@ -147,6 +147,7 @@ struct teuk_ctx {
     std::string err;
     int strip = 0;           // r* columns per thread block (0 = automatic)
     int steps_per_launch = 1;
+    int sms = 1;             // SMs of the device
     int64_t launches = 0;
     Batch batch;
     int64_t inject_skip_item = -1;   // testing aid: a work item that never releases its flag
@@ -283,7 +284,6 @@ InstDev dev_of(const teuk_ctx* c, const Instance& I) {
     d.wave_cap = I.wave_cap;
     d.status = c->status;
     d.fault_col = I.fault_col;
-    d.resident = I.resident;
     return d;
 }
 
@@ -307,9 +307,42 @@ int eff_strip(const teuk_ctx* c, const Instance& I) {
     return std::max(1, std::min(L, I.p.n_rstar - 2));
 }
 
-// Column partition of the per-step launch: the same number of blocks as uniform strips
-// of the effective length, cut so that the blocks have about equal cost.  A column costs
-// 1, a column of the source window 1 + alpha (its source terms) and the extraction
+// Pieces of the automatic per-step launch (nb) and the cap on blocks an SM (0: none).
+// Consecutive steps overlap (programmatic dependent launch): a step's blocks take the places
+// that the previous step leaves free, so with some places left over they pile up on the SMs
+// that have them, and the SM with most blocks sets the step's time.  The launch therefore
+// takes every place: as many pieces as places, or no more places (the cap) than the pieces
+// need.  us per step, one wave of strips of equal length -> this rule:
+//   FP32, a piece for every place: FP32-Kahan 2048 x 128 6.5 -> 6.0, 5001 x 100 10.5 -> 10.0,
+//     8192 x 128 14.7 -> 14.3
+//   FP64, twelve warps an SM, capped (they fill the FP64 pipe, and fewer pieces compute
+//     fewer half nodes twice): 241 x 32 7.2 -> 6.5, 800 x 64 17.9 -> 13.7, 2048 x 128 51.1 ->
+//     43.7, 5001 x 100 101.8 -> 92.8, 8192 x 128 154.1 -> 149.5
+//   double-float, a piece for every place while it has six columns (5001 x 100 29.7 -> 28.4,
+//     8192 x 128 44.1 -> 43.5; with twelve warps 28.5, 43.8), else as FP64 (800 x 64 6.1 -> 5.4,
+//     2048 x 128 15.0 -> 13.6, 4096 x 64 15.1 -> 13.8; a piece for every place 14.4, 15.8)
+// FP32-Kahan capped on 800 x 64: 3.8 us instead of 3.5 (its next step's start-up is worth
+// more).  Two places an SM were too few for one-warp blocks (241 x 32: 7.1 us, three 6.3).
+// With one block an SM only its longest piece counts: no more pieces than give that length,
+// so that the record has a block of its own (3001 x 300, FP32: 13.0 us, 152 pieces 13.8).
+void auto_cut(const Instance& I, int sms, int* nb, int* cap) {
+    const int cols = I.p.n_rstar - 2;
+    const int places = std::max(1, I.resident / sms), warps = I.pitch / 32;
+    const bool df = I.p.prec == TEUK_FP64_DF;
+    int per = places;
+    if (I.p.prec == TEUK_FP64 || (df && cols < 6 * places * sms)) per = std::min(places, (12 + warps - 1) / warps);
+    *nb = std::min(cols, per * sms);
+    if (places == 1) {
+        const int L = (cols + *nb - 1) / *nb;
+        *nb = (cols + L - 1) / L;
+    }
+    const int held = std::max(kMinCap, (*nb + sms - 1) / sms);
+    *cap = held < places && (df || I.p.prec == TEUK_FP64) ? held : 0;
+}
+
+// Column partition of the per-step launch: the pieces of auto_cut, or as many as uniform
+// strips of a length that was set, cut so that the blocks have about equal cost.  A column
+// costs 1, a column of the source window 1 + alpha (its source terms) and the extraction
 // column 2 more (the FP64 waveform record).  alpha, measured on GB300 (16384 x 256 step
 // time against alpha): FP32 paths 0.25, FP64 0.1, double-float 0.4; for a moving
 // particle, whose source terms also carry the per-step Gaussian factors, FP32 0.8 and
@@ -319,7 +352,8 @@ int eff_strip(const teuk_ctx* c, const Instance& I) {
 teuk_status refresh_partition(teuk_ctx* c, Instance& I) {
     const int strip = eff_strip(c, I);
     const int nr = I.p.n_rstar;
-    const int nb = (nr - 2 + strip - 1) / strip;
+    int nb = (nr - 2 + strip - 1) / strip, cap = 0;
+    if (strip == auto_strip(I)) auto_cut(I, c->sms, &nb, &cap);
     const double alpha = I.p.prec == TEUK_FP64      ? 0.1
                          : I.p.prec == TEUK_FP64_DF ? (I.sd.moving ? 0.6 : 0.4)
                                                     : (I.sd.moving ? 0.8 : 0.25);
@@ -351,6 +385,8 @@ teuk_status refresh_partition(teuk_ctx* c, Instance& I) {
     TK_CUDA(c, cudaMemcpyAsync(I.d_part, I.h_part.data(), sizeof(int) * (nb + 1), cudaMemcpyHostToDevice,
                                c->stream));
     I.part_strip = strip;
+    I.part_nb = nb;
+    I.part_cap = cap;
     return TEUK_OK;
 }
 
@@ -380,8 +416,23 @@ teuk_status coef_tables(teuk_ctx* c, Instance& I) {
     return TEUK_OK;
 }
 
+// The cut of per-step launches with strip length `strip`: the partition built for it, or
+// uniform strips.
+StepCut cut_of(const teuk_ctx* c, const Instance& I, int strip) {
+    StepCut q;
+    q.strip = strip;
+    q.room = I.resident;
+    if (I.part_strip == strip) {
+        q.part = I.d_part;
+        q.nb = I.part_nb;
+        q.cap = I.part_cap;
+        if (q.cap > 0) q.room = std::min(q.room, q.cap * c->sms);
+    }
+    return q;
+}
+
 void do_step(teuk_ctx* c, Instance& I, int strip) {
-    launch_step(c->stream, dev_of(c, I), I.step, I.cur, strip, I.part_strip == strip ? I.d_part : nullptr);
+    launch_step(c->stream, dev_of(c, I), I.step, I.cur, cut_of(c, I, strip));
     c->launches++;
     I.cur = 1 - I.cur;
     I.step++;
@@ -411,8 +462,7 @@ constexpr int64_t kStepGraph = 64;
 // on its stream (any stream, the legacy default one included).  Returns nullptr while
 // the caller is capturing the context's stream, or if capture failed; the steps are
 // then launched directly.
-cudaGraphExec_t step_graph_of(teuk_ctx* c, Instance& I, const InstDev& dv, int p, int strip,
-                              const int* part) {
+cudaGraphExec_t step_graph_of(teuk_ctx* c, Instance& I, const InstDev& dv, int p, const StepCut& cut) {
     if (I.sg_failed) return nullptr;
     cudaStreamCaptureStatus ucs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &ucs) != cudaSuccess || ucs != cudaStreamCaptureStatusNone) {
@@ -430,8 +480,7 @@ cudaGraphExec_t step_graph_of(teuk_ctx* c, Instance& I, const InstDev& dv, int p
     std::memset(&key, 0, sizeof key);
     std::memcpy(&key.d, &dv, sizeof dv);
     key.d.step_base = I.d_step;
-    key.part = part;
-    key.strip = strip;
+    std::memcpy(&key.cut, &cut, sizeof cut);
     if (I.sg_exec[p] && std::memcmp(&key, &I.sg_key[p], sizeof key) == 0) return I.sg_exec[p];
     if (I.sg_exec[p]) cudaGraphExecDestroy(I.sg_exec[p]);
     I.sg_exec[p] = nullptr;
@@ -443,7 +492,7 @@ cudaGraphExec_t step_graph_of(teuk_ctx* c, Instance& I, const InstDev& dv, int p
         return nullptr;
     }
     for (int64_t k = 0; k < kStepGraph; ++k)
-        launch_step(cs, key.d, k, (int)((p + k) & 1), strip, key.part);
+        launch_step(cs, key.d, k, (int)((p + k) & 1), cut);
     launch_advance_step(cs, I.d_step, kStepGraph);
     cudaGraphExec_t e = nullptr;
     if (cudaStreamEndCapture(cs, &g) != cudaSuccess || !g ||
@@ -460,7 +509,7 @@ cudaGraphExec_t step_graph_of(teuk_ctx* c, Instance& I, const InstDev& dv, int p
 }
 
 cudaGraphExec_t step_graph(teuk_ctx* c, Instance& I, int strip) {
-    return step_graph_of(c, I, dev_of(c, I), I.cur, strip, I.part_strip == strip ? I.d_part : nullptr);
+    return step_graph_of(c, I, dev_of(c, I), I.cur, cut_of(c, I, strip));
 }
 
 // Run count steps of the descriptor dv from buffer cur at time level `level` on stream st:
@@ -468,10 +517,10 @@ cudaGraphExec_t step_graph(teuk_ctx* c, Instance& I, int strip) {
 // the rest one launch at a time.  Returns the buffer holding the result.
 int run_steps(teuk_ctx* c, Instance& I, const InstDev& dv, cudaStream_t st, int cur, int64_t level,
               int64_t count, int strip) {
-    const int* part = I.part_strip == strip ? I.d_part : nullptr;
+    const StepCut cut = cut_of(c, I, strip);
     int64_t k = 0;
     cudaGraphExec_t e = (st == c->stream && count >= kStepGraph)
-                            ? step_graph_of(c, I, dv, cur, strip, part) : nullptr;
+                            ? step_graph_of(c, I, dv, cur, cut) : nullptr;
     if (e && I.graph_base != level) {
         I.h_step = level;
         if (cudaMemcpyAsync(I.d_step, &I.h_step, sizeof(int64_t), cudaMemcpyHostToDevice, st) != cudaSuccess) {
@@ -491,7 +540,7 @@ int run_steps(teuk_ctx* c, Instance& I, const InstDev& dv, cudaStream_t st, int 
             I.graph_base += kStepGraph;   // advanced by the graph's last node
         }
     for (; k < count; ++k) {   // (kStepGraph is even: the graphs leave the buffer unchanged)
-        launch_step(st, dv, level + k, cur, strip, part);
+        launch_step(st, dv, level + k, cur, cut);
         c->launches++;
         cur = 1 - cur;
     }
@@ -554,6 +603,8 @@ extern "C" teuk_status teuk_create(const teuk_params* p, int n_instances, void* 
     c->stream = (cudaStream_t)cuda_stream;
     c->prec = p[0].prec;
     c->inst = std::move(inst);
+    cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (c->sms < 1) c->sms = 1;
     auto fail = [&](teuk_status st) {
         g_create_err = c->err;
         teuk_destroy(c);
@@ -1701,12 +1752,14 @@ extern "C" teuk_status teuk_autotune(teuk_ctx* c, int trial_steps, int* chosen) 
                 d.buf[0][q] = scr[0][q];
                 d.buf[1][q] = scr[1][q];
             }
-            const int cand[] = {1, 2, 4, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512};
+            const int cand[] = {auto_strip(I), 1, 2, 4, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512};
             for (int ch : cand) {
-                if (ch > I.p.n_rstar - 2) break;
-                for (int w = 0; w < 2; ++w) launch_step(c->stream, d, I.step + w, w & 1, ch);
+                if (ch > I.p.n_rstar - 2) continue;
+                // (the automatic length times the partition it stands for)
+                const StepCut cut = cut_of(c, I, ch);
+                for (int w = 0; w < 2; ++w) launch_step(c->stream, d, I.step + w, w & 1, cut);
                 cudaEventRecord(e0, c->stream);
-                for (int t = 0; t < trial_steps; ++t) launch_step(c->stream, d, I.step + t, t & 1, ch);
+                for (int t = 0; t < trial_steps; ++t) launch_step(c->stream, d, I.step + t, t & 1, cut);
                 cudaEventRecord(e1, c->stream);
                 cudaEventSynchronize(e1);
                 float ms = 0.f;
@@ -1964,8 +2017,7 @@ extern "C" teuk_status teuk_adjoint_n(teuk_ctx* c, int instance, int64_t step0, 
     }
     // the fused reverse step's strip; with a source, a ring of window co-states that
     // adj_src_grad_kernel turns into gradients every `slots` steps (32 MB at most)
-    int adj_strip = 0;
-    adj_step_plan(dev_of(c, I), &adj_strip);
+    const AdjCut adj_cut = adj_step_plan(dev_of(c, I));
     const bool src_on = I.src_on;
     const size_t wbytes = src_on ? adj_window_bytes(dev_of(c, I)) : 0;
     const int64_t slots = src_on ? std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(n, 256),
@@ -2078,7 +2130,7 @@ extern "C" teuk_status teuk_adjoint_n(teuk_ctx* c, int instance, int64_t step0, 
             }
             const double2* gb = k >= 1 ? gslot(k - 1) : nullptr;
             char* slot = src_on ? wring + (size_t)(k % slots) * wbytes : nullptr;
-            launch_adj_step(s, d, lam[cur], gb, lam[1 - cur], adj_strip, slot, slot ? slot + wh_bytes : nullptr);
+            launch_adj_step(s, d, lam[cur], gb, lam[1 - cur], adj_cut, slot, slot ? slot + wh_bytes : nullptr);
             if (src_on && k % slots == 0) {   // the steps k .. k + slots - 1 are all stored
                 launch_adj_src_grad(s, d, step0, k, std::min<int64_t>(n - 1, k + slots - 1) - k + 1,
                                     (int)slots, wring, gA, gR);

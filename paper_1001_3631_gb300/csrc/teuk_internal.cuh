@@ -120,8 +120,6 @@ struct InstDev {
     unsigned int* status;     // device status word (bit flags)
     int fault_col;            // testing aid: this input column is never filled into the
                               // step kernels' ring (-1: none)
-    int resident;             // blocks of the per-step kernel that the GPU holds at once
-    int pad;
     const int64_t* step_base; // per-step kernels replayed from a graph: their step argument
                               // is an offset from *step_base (null: the argument is the step)
 };
@@ -221,10 +219,16 @@ void launch_trajectory(cudaStream_t st, double M, double a, int m, double rstar_
 // teuk_step.cu
 cudaError_t prepare_step_kernels();
 int step_resident_blocks(int prec, int threads);  // blocks of the step kernel the GPU holds at once
-// part (device, may be null): block b covers the columns [part[b], part[b+1]) of a
-// partition into ceil((n_rstar - 2) / strip) pieces, instead of uniform strips
-void launch_step(cudaStream_t st, const InstDev& d, int64_t step, int bin, int strip,
-                 const int* part = nullptr);
+// How a per-step launch cuts the columns: uniform strips of `strip` columns (part null), or
+// nb pieces, block b covering [part[b], part[b+1]) (part: device); cap > 0: at most cap
+// blocks on an SM at once (by the size of their shared memory); room: blocks the GPU then
+// holds at once.  (Compared byte for byte in the step graphs' keys: no padding.)
+struct StepCut {
+    const int* part = nullptr;
+    int strip = 1, nb = 0, cap = 0, room = 0;
+};
+constexpr int kMinCap = 3;   // the smallest cap
+void launch_step(cudaStream_t st, const InstDev& d, int64_t step, int bin, const StepCut& cut);
 void launch_extract(cudaStream_t st, const InstDev& d, int64_t step, int bin);
 // *base += k (one thread): closes a replayed graph of k per-step launches
 void launch_advance_step(cudaStream_t st, int64_t* base, int64_t k);
@@ -255,13 +259,14 @@ void launch_wave_sum(cudaStream_t st, const double2* wave, int64_t cap, int nth,
 struct CoLevel { void* F; void* P; void* Fc; void* Pc; };
 // lam = E^T gbar: the co-state that starts the reverse sweep
 void launch_adj_init(cudaStream_t st, const InstDev& d, const double2* gbar, const CoLevel& out);
-// the fused reverse step (lam^n from lam^{n+1}): strip length and block count from
-// adj_step_plan; wh, wi (null without a source): the step's ring slot of the window
+// the fused reverse step (lam^n from lam^{n+1}), cut as adj_step_plan says (uniform strips
+// of `strip` columns, or, strip 0, nb pieces of equal length to a column); wh, wi (null without a source): the step's ring slot of the window
 // co-states, mu_Pi at the half-node window ([nj][nh]) and lam'_Pi at the integer-node
 // window ([nj][ni]), complex in the co-state's type
-int adj_step_plan(const InstDev& d, int* strip);
+struct AdjCut { int strip, nb; };
+AdjCut adj_step_plan(const InstDev& d);
 void launch_adj_step(cudaStream_t st, const InstDev& d, const CoLevel& lin, const double2* gbar,
-                     const CoLevel& lout, int strip, void* wh, void* wi);
+                     const CoLevel& lout, const AdjCut& cut, void* wh, void* wi);
 // bytes of one ring slot (the half-node window, then the integer-node window)
 size_t adj_window_bytes(const InstDev& d);
 // source gradients gA[k], gR[k] of the steps k0 .. k0 + count - 1 of a sweep starting at

@@ -609,9 +609,9 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
 // blocks per SM), of up to 512 rows (one block per SM, 128 registers a thread) and of up
 // to 1024 rows.  Dynamic shared memory:
 // StepShared<P, R>::bytes(blockDim.x).
-// part (may be null): the block's columns are [part[b], part[b+1]) instead of the uniform
-// strips; it is written by the host before the launch sequence and never changes while
-// a step runs, so it is read before griddepcontrol.wait.
+// part (may be null): the block's columns are [part[b], part[b+1]), of `strip` pieces, instead
+// of uniform strips of `strip` columns; it is written by the host before the launch sequence
+// and never changes while a step runs, so it is read before griddepcontrol.wait.
 template <class P, int R, bool kMov>
 __device__ __forceinline__ void step_body(const InstDev& d, int64_t step, int bin, int strip,
                                           const int* part) {
@@ -625,7 +625,7 @@ __device__ __forceinline__ void step_body(const InstDev& d, int64_t step, int bi
     // while the graph's steps run
     if (d.step_base) step += *d.step_base;
     // a launch with one block more than pieces takes the record in that block
-    const bool rec_apart = (int64_t)(gridDim.x - 1) * strip >= d.nr - 2;
+    const bool rec_apart = part ? (int)gridDim.x > strip : (int64_t)(gridDim.x - 1) * strip >= d.nr - 2;
     if (rec_apart && blockIdx.x == gridDim.x - 1) {
         griddep_wait();
         if (!(*(volatile unsigned*)d.status & ST_TIMEOUT)) record_level<P>(d, step, bin);
@@ -872,15 +872,26 @@ void launch_batched_extract(cudaStream_t st, int prec, const BatchDev& b, int ma
     else batched_extract_kernel<PK><<<g, 128, 0, st>>>(b);
 }
 
+// Dynamic shared memory (at least `own`) with which an SM holds cap blocks and no more.
+static size_t capped_smem(int cap, size_t own) {
+    int dev = 0, sm = 0, res = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    cudaDeviceGetAttribute(&res, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    const int b = (sm / cap - res - 512) / 128 * 128;   // (512: the kernels' static shared memory)
+    return b > (int)own ? (size_t)b : own;
+}
+
 template <class P, bool kMov>
-static void launch_step_m(cudaStream_t st, const InstDev& d, int64_t step, int bin, int strip,
-                          const int* part) {
+static void launch_step_m(cudaStream_t st, const InstDev& d, int64_t step, int bin, const StepCut& cut) {
+    const int strip = cut.part ? cut.nb : cut.strip;
+    const int* part = cut.part;
     // a grid that leaves a block's place free takes its record in a block of its own: on
     // 800 x 64 (one-column pieces) the block that also took the record was the step's last
     // (us per step: FP32-Kahan 4.01 -> 3.49, FP32 3.35 -> 3.09); a full wave has no such
     // place, and the piece that holds the record is cut shorter (refresh_partition)
-    int blocks = (d.nr - 2 + strip - 1) / strip;
-    if (blocks < d.resident) ++blocks;
+    int blocks = part ? cut.nb : (d.nr - 2 + strip - 1) / strip;
+    if (blocks < cut.room) ++blocks;
     int threads = d.pitch;
     // programmatic dependent launch (see step_body)
     cudaLaunchAttribute at[1];
@@ -894,6 +905,7 @@ static void launch_step_m(cudaStream_t st, const InstDev& d, int64_t step, int b
     cfg.numAttrs = 1;
     if (threads <= 256) {
         cfg.dynamicSmemBytes = StepShared<P, kRingS>::bytes(threads);
+        if (cut.cap > 0) cfg.dynamicSmemBytes = capped_smem(cut.cap, cfg.dynamicSmemBytes);
         cudaLaunchKernelEx(&cfg, step_kernel_s<P, kMov>, d, step, bin, strip, part);
     } else if (threads <= 512) {
         cfg.dynamicSmemBytes = StepShared<P, kRingS>::bytes(threads);
@@ -904,10 +916,9 @@ static void launch_step_m(cudaStream_t st, const InstDev& d, int64_t step, int b
     }
 }
 template <class P>
-static void launch_step_p(cudaStream_t st, const InstDev& d, int64_t step, int bin, int strip,
-                          const int* part) {
-    if (d.src.on && d.src.moving) launch_step_m<P, true>(st, d, step, bin, strip, part);
-    else launch_step_m<P, false>(st, d, step, bin, strip, part);
+static void launch_step_p(cudaStream_t st, const InstDev& d, int64_t step, int bin, const StepCut& cut) {
+    if (d.src.on && d.src.moving) launch_step_m<P, true>(st, d, step, bin, cut);
+    else launch_step_m<P, false>(st, d, step, bin, cut);
 }
 
 template <class P>
@@ -934,19 +945,20 @@ int step_resident_blocks(int prec, int threads) {
     return resident_p<PK>(threads);
 }
 
-void launch_step(cudaStream_t st, const InstDev& d, int64_t step, int bin, int strip,
-                 const int* part) {
-    if (d.prec == 0) launch_step_p<P64>(st, d, step, bin, strip, part);
-    else if (d.prec == 1) launch_step_p<P32>(st, d, step, bin, strip, part);
-    else if (d.prec == 3) launch_step_p<PD>(st, d, step, bin, strip, part);
-    else launch_step_p<PK>(st, d, step, bin, strip, part);
+void launch_step(cudaStream_t st, const InstDev& d, int64_t step, int bin, const StepCut& cut) {
+    if (d.prec == 0) launch_step_p<P64>(st, d, step, bin, cut);
+    else if (d.prec == 1) launch_step_p<P32>(st, d, step, bin, cut);
+    else if (d.prec == 3) launch_step_p<PD>(st, d, step, bin, cut);
+    else launch_step_p<PK>(st, d, step, bin, cut);
 }
 
 // Opt the step kernels in to the dynamic shared memory of their largest blocks (on the
 // current device; called when a context is created).
 template <class P, bool kMov>
 static cudaError_t prepare_m() {
-    const int s = (int)StepShared<P, kRingS>::bytes(256), m = (int)StepShared<P, kRingS>::bytes(512),
+    // (a capped launch, FP64 and double-float, takes more than its blocks need)
+    const unsigned need = StepShared<P, kRingS>::bytes(256);
+    const int s = (int)(split_angular<P>() ? need : capped_smem(kMinCap, need)), m = (int)StepShared<P, kRingS>::bytes(512),
               l = (int)StepShared<P, kRingL>::bytes(1024);
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(step_kernel_s<P, kMov>, a, s);
