@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel 
     const SourceDev& s = d.src;
     // wh, wi: this step's ring slot of the window co-states (null: no source)
     RowTab<PK> rt;
-    rt.load(d.thtab, j, row_ok);
+    rt.load(d.thtab_a, j, row_ok);
     auto lam_at = [&](int col) {
         CoNode<R> z{};
         if (row_ok && col >= 1 && col <= nr - 2) z = co_load<R>(lin, node_index(d, col, j));
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel 
     auto form = [&](int col, CfF& ci, CfF& ch) {
         float2 cf2[kNCoef];
         if (col >= 0 && col <= nr - 1) {
-            form_coefs2(rt_smem ? RT[col - (c0 - 1)] : d.rtab[col], rt.t, cf2);
+            form_coefs2(rt_smem ? RT[col - (c0 - 1)] : d.rtab_a[col], rt.t, cf2);
         } else {
 #pragma unroll
             for (int q = 0; q < kNCoef; ++q) cf2[q] = make_float2(0.f, 0.f);
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel 
         const int ncols = c1 - c0 + 2;
         for (int q = threadIdx.x; q < ncols * 8; q += blockDim.x) {
             const int k = q >> 3, col = c0 - 1 + k;
-            if (col >= 0 && col <= nr - 1) ((float4*)(RT + k))[q & 7] = __ldg((const float4*)(d.rtab + col) + (q & 7));
+            if (col >= 0 && col <= nr - 1) ((float4*)(RT + k))[q & 7] = __ldg((const float4*)(d.rtab_a + col) + (q & 7));
         }
         __syncthreads();
     }

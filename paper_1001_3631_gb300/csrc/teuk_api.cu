@@ -39,6 +39,8 @@ struct Instance {
     double* x_half = nullptr;
     RTab2* rtab = nullptr;      // [nr] (half node, node) per column (FP32 paths)
     ThTab* thtab = nullptr;     // [nth]
+    RTab2* rtab_a = nullptr;    // the same for the adjoint
+    ThTab* thtab_a = nullptr;
     // source
     bool src_on = false;
     teuk_orbit orbit{};
@@ -276,6 +278,8 @@ InstDev dev_of(const teuk_ctx* c, const Instance& I) {
     d.coef_i = I.coef_i;
     d.rtab = I.rtab;
     d.thtab = I.thtab;
+    d.rtab_a = I.rtab_a;
+    d.thtab_a = I.thtab_a;
     d.src = I.sd;
     d.src.on = I.src_on ? 1 : 0;
     d.i_e = I.i_e;
@@ -555,7 +559,7 @@ void free_instance(const teuk_ctx* c, Instance& I) {
     for (int b = 0; b < 2; ++b)
         for (int k = 0; k < 2; ++k)
             if (I.state[b][k]) dfree(c, I.state[b][k], s);
-    void* ptrs[] = {I.coef_h, I.coef_i, I.x_int, I.x_half, I.P_win, I.amps, I.wave, I.rtab, I.thtab,
+    void* ptrs[] = {I.coef_h, I.coef_i, I.x_int, I.x_half, I.P_win, I.amps, I.wave, I.rtab, I.thtab, I.rtab_a, I.thtab_a,
                     I.stage, I.d_part, I.traj_buf, I.res_xg, I.res_flags};
     for (void* q : ptrs)
         if (q) dfree(c, q, s);
@@ -643,11 +647,15 @@ extern "C" teuk_status teuk_create(const teuk_params* p, int n_instances, void* 
             const teuk_status e = coef_tables(c, I);
             if (e != TEUK_OK) return fail(e);
         } else {
-            TK_CCUDA(dmalloc(c, (void**)&I.rtab, sizeof(RTab2) * q.n_rstar, c->stream));
-            TK_CCUDA(dmalloc(c, (void**)&I.thtab, sizeof(ThTab) * q.n_theta, c->stream));
-            launch_tables_1d(c->stream, q.M, q.a, q.s, q.m, I.drs, I.dth, I.dt, q.n_rstar,
-                             q.n_theta, I.x_int, I.x_half, I.rtab, I.thtab);
-            c->launches++;
+            for (int adj = 0; adj < 2; ++adj) {
+                RTab2*& rt = adj ? I.rtab_a : I.rtab;
+                ThTab*& tt = adj ? I.thtab_a : I.thtab;
+                TK_CCUDA(dmalloc(c, (void**)&rt, sizeof(RTab2) * q.n_rstar, c->stream));
+                TK_CCUDA(dmalloc(c, (void**)&tt, sizeof(ThTab) * q.n_theta, c->stream));
+                launch_tables_1d(c->stream, q.M, q.a, q.s, q.m, I.drs, I.dth, I.dt, q.n_rstar, q.n_theta,
+                                 I.x_int, I.x_half, rt, tt, adj == 0);
+                c->launches++;
+            }
         }
         TK_CCUDA(cudaGetLastError());
         I.r_ext = 0;  // filled lazily from x at r*_ext when needed (adjoint loss)

@@ -91,6 +91,9 @@ struct SourceDev {
 //   A, B = Ds iS / dth^2, Ds iS cot / (2 dth)         (Ds = sdt Delta; the split angular
 //                                                       form, ep = A + B, em = A - B)
 //   E3 = ((qr + nDs V) iS, qi iS)                      (qr, qi scaled by sdt; nDs = -Ds)
+// The forward step acts on undivided sums and the negated second difference (split form in
+// teuk_step_common.cuh): its tables hold nsdt, Ds, nDs, qr, qi times 1/2 (half node) and 1/4
+// (node) and i2 = -1/dth^2, all exactly; the adjoint's hold the values above.
 struct RTab2 { float2 R2, naD, Rd, ctr, cti, ctc, pr, pi, nbb, Ds, nDs, qr, qi, nsdt, pad0, pad1; };
 // Per theta row: sin^2, cos, V = (m + s cos)^2/sin^2 - s, i2 = 1/dth^2, i1 = cot/(2 dth)
 struct ThTab { float sin2, cs, V, i2, i1, pad0, pad1, pad2; };
@@ -112,6 +115,8 @@ struct InstDev {
     const void* coef_i;
     const RTab2* rtab;        // [nr] FP32 paths: radial tables (half node, node) per column
     const ThTab* thtab;       // [nth]
+    const RTab2* rtab_a;      // the same for the adjoint (see RTab2)
+    const ThTab* thtab_a;
     SourceDev src;
     int i_e;                  // extraction between i_e and i_e + 1
     double f_e;
@@ -206,7 +211,7 @@ void launch_coefficients(cudaStream_t st, int prec, double M, double a, int s, i
                          void* coef_i);
 void launch_tables_1d(cudaStream_t st, double M, double a, int s, int m, double drs, double dth,
                       double dt, int nr, int nth, const double* x_int, const double* x_half,
-                      RTab2* rtab, ThTab* thtab);
+                      RTab2* rtab, ThTab* thtab, bool forward);
 void launch_profile(cudaStream_t st, double M, double a, double rstar_min, double drs, int off,
                     double dth, double rs0, double sig_r, double sig_t, double drs0_dr0,
                     const double* x_int, const double* x_half, const SourceDev& src, int prec);

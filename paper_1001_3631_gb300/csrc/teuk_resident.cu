@@ -112,8 +112,8 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
     const bool bot = j == 0, top = j == nth - 1;
     const int jp = j + 1 < nth ? j + 1 : j, jm = j > 0 ? j - 1 : 0;
     const T g = (T)d.ghost;
-    const T gp = top ? g : T(1), gm = bot ? g : T(1);
-    const T hdt = step_hdt<T>(d), fdt = (T)d.dt, qdt = step_qdt<T>(d);
+    const T ngp = top ? -g : T(-1), ngm = bot ? -g : T(-1);
+    const T hdt = step_hdt<T>(d), qdt = step_qdt<T>(d);
     const Lin<T> A(d);
     const PoleRow pole(d, j);
     const bool has_l = b > 0, has_r = b < r.nb - 1;
@@ -274,11 +274,11 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
                     C dll, dlml, dlr, dlmr;
                     {
                         const NodeV<P> dn = S.load_phi(sidx(k, jp)), upn = S.load_phi(sidx(k, jm));
-                        ul.theta_split(gp, dn, gm, upn, dll, dlml);
+                        ul.theta_split(ngp, dn, ngm, upn, dll, dlml);
                     }
                     {
                         const NodeV<P> dn = S.load_phi(sidx(k + 1, jp)), upn = S.load_phi(sidx(k + 1, jm));
-                        ur.theta_split(gp, dn, gm, upn, dlr, dlmr);
+                        ur.theta_split(ngp, dn, ngm, upn, dlr, dlmr);
                     }
                     C s_h = C::zero();
                     if (src_blk) s_h = source_half<T>(sw, C{sfac[ip][s][0], sfac[ip][s][1]}, col, j);
@@ -286,9 +286,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
 #pragma unroll
                     for (int q = 0; q < kNCoef; ++q) cf[q] = CF[sidx(k, j) * 2 * kNCoef + q];
                     const Half<T> hp = half_prep<P>(ul, ur);
-                    const C Dp = C::half_sum(dll, dlr);
-                    const C Dm = C::half_sum(dlml, dlmr);
-                    HR[sidx(k, j)] = predictor<T>(hp, Dp, Dm, cf, hdt, s_h);
+                    HR[sidx(k, j)] = predictor<T>(hp, dll + dlr, dlml + dlmr, cf, qdt, s_h);
                 } else {
                     // the sums of the rows above and below, as those rows form them
                     const NodeV<P> ul = S.load(sidx(k, j)), ur = S.load(sidx(k + 1, j));
@@ -335,7 +333,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
 #pragma unroll
                         for (int q = 0; q < kNCoef; ++q) cf[q] = CF[sidx(k, j) * 2 * kNCoef + kNCoef + q];
                         C dPhi, dPi;
-                        corrector_incr<P>(row, Hs_p, Hs_m, cf, fdt, s_i, dPhi, dPi);
+                        corrector_incr<P>(row, Hs_p, Hs_m, cf, qdt, s_i, dPhi, dPi);
                         NodeV<P> u = S.load(sidx(k, j));
                         u.update(dPhi, dPi);
                         S.store(sidx(k, j), u);

@@ -318,13 +318,16 @@ __device__ float2 pair_f(double h, double i) { return make_float2((float)h, (flo
 
 __global__ void tables_1d_kernel(double M, double a, int s, int m, double drs, double dth,
                                  double dt, int nr, int nth, const double* x_int,
-                                 const double* x_half, RTab2* rtab, ThTab* thtab) {
+                                 const double* x_half, RTab2* rtab, ThTab* thtab, double fh, double fi,
+                                 double fi2) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < nr) {
         // the half node nr-1/2 lies outside the grid: zeros
         const RadialVals h = k < nr - 1 ? radial_vals(M, a, s, m, x_half[k], drs, 0.5 * dt) : RadialVals{};
         const RadialVals i = radial_vals(M, a, s, m, x_int[k], drs, dt);
         RTab2 t;
+        // the terms that act on sums, times fh at the half node and fi at the node
+        auto pair_s = [&](double hv, double iv) { return pair_f(fh * hv, fi * iv); };
         t.R2 = pair_f(h.R2, i.R2);
         t.naD = pair_f(h.naD, i.naD);
         t.Rd = pair_f(h.Rd, i.Rd);
@@ -334,11 +337,11 @@ __global__ void tables_1d_kernel(double M, double a, int s, int m, double drs, d
         t.pr = pair_f(h.pr, i.pr);
         t.pi = pair_f(h.pi, i.pi);
         t.nbb = pair_f(h.nbb, i.nbb);
-        t.Ds = pair_f(h.Ds, i.Ds);
-        t.nDs = pair_f(h.nDs, i.nDs);
-        t.qr = pair_f(h.qr, i.qr);
-        t.qi = pair_f(h.qi, i.qi);
-        t.nsdt = pair_f(h.nsdt, i.nsdt);
+        t.Ds = pair_s(h.Ds, i.Ds);
+        t.nDs = pair_s(h.nDs, i.nDs);
+        t.qr = pair_s(h.qr, i.qr);
+        t.qi = pair_s(h.qi, i.qi);
+        t.nsdt = pair_s(h.nsdt, i.nsdt);
         t.pad0 = t.pad1 = make_float2(0.f, 0.f);
         rtab[k] = t;
     }
@@ -350,7 +353,7 @@ __global__ void tables_1d_kernel(double M, double a, int s, int m, double drs, d
         t.sin2 = (float)(sn * sn);
         t.cs = (float)cs;
         t.V = (float)((mv + sv * cs) * (mv + sv * cs) / (sn * sn) - sv);
-        t.i2 = (float)(1.0 / (dth * dth));
+        t.i2 = (float)(fi2 / (dth * dth));
         t.i1 = (float)(cs / sn / (2.0 * dth));
         t.pad0 = t.pad1 = t.pad2 = 0.f;
         thtab[k] = t;
@@ -359,10 +362,13 @@ __global__ void tables_1d_kernel(double M, double a, int s, int m, double drs, d
 
 void launch_tables_1d(cudaStream_t st, double M, double a, int s, int m, double drs, double dth,
                       double dt, int nr, int nth, const double* x_int, const double* x_half,
-                      RTab2* rtab, ThTab* thtab) {
+                      RTab2* rtab, ThTab* thtab, bool forward) {
     int n = nr > nth ? nr : nth;
+    // forward: of the undivided sums of two (half nodes) and four (nodes) values and the
+    // negated second difference (teuk_step_common.cuh)
+    const double fh = forward ? 0.5 : 1.0, fi = forward ? 0.25 : 1.0, fi2 = forward ? -1.0 : 1.0;
     tables_1d_kernel<<<(n + 127) / 128, 128, 0, st>>>(M, a, s, m, drs, dth, dt, nr, nth, x_int,
-                                                      x_half, rtab, thtab);
+                                                      x_half, rtab, thtab, fh, fi, fi2);
 }
 
 void launch_invert_tortoise(cudaStream_t st, double M, double a, double rstar_min, double drs,

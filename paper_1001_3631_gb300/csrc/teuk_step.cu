@@ -460,11 +460,11 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
     if constexpr (kSplit) {
         const bool bot = j == 0, top = j == nth - 1;
         // theta neighbours in the slot, the pole rows standing in for the ghost rows: row
-        // nth = g * row nth-1 and row -1 = g * row 0 (gp, gm the factors)
+        // nth = g * row nth-1 and row -1 = g * row 0 (-ngp, -ngm the factors)
         const int jp = j + 1 < nth ? j + 1 : j, jm = j > 0 ? j - 1 : 0;
         const T g = d.ghost_f;
-        const T gp = top ? g : T(1), gm = bot ? g : T(1);
-        const T hdt = step_hdt<T>(d), fdt = d.dt_f;
+        const T ngp = top ? -g : T(-1), ngm = bot ? -g : T(-1);
+        const T qdt = step_qdt<T>(d);
         const unsigned xstride = 4u * (blockDim.x + 2u);
         const size_t pitch = (size_t)d.pitch;
         // own node of the column in slot s (rows past nth read slot padding: their results
@@ -475,15 +475,13 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
         auto theta_diffs = [&](int s, const NodeV<P>& u, C& dl, C& dlm) {
             const Planes<P> pl = ring.planes(s);
             const NodeV<P> dn = pl.load_phi((size_t)jp), upn = pl.load_phi((size_t)jm);
-            u.theta_split(gp, dn, gm, upn, dl, dlm);
+            u.theta_split(ngp, dn, ngm, upn, dl, dlm);
         };
         // predictor at the half node h between columns h (ul) and h+1 (ur)
         auto predict = [&](const NodeV<P>& ul, const NodeV<P>& ur, C dll, C dlr, C dlml, C dlmr,
                            const T* cf, C src) {
             const Half<T> hp = half_prep<P>(ul, ur);
-            const C Dp = C::half_sum(dll, dlr);     // Fb(j+1) - Fb(j)    (split: Fb(j+1) - 2 Fb(j) + Fb(j-1))
-            const C Dm = C::half_sum(dlml, dlmr);   // Fb(j) - Fb(j-1)    (split: Fb(j+1) - Fb(j-1))
-            return predictor<T>(hp, Dp, Dm, cf, hdt, src);
+            return predictor<T>(hp, dll + dlr, dlml + dlmr, cf, qdt, src);
         };
         // coefficients of column col: the half node col+1/2 into cfh and, on the FP32 paths
         // (formed together in paired instructions), the node col into cfi
@@ -510,7 +508,7 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
             C Hs_p, Hs_m;
             xread(mine, Hs_p, Hs_m);
             C dPhi, dPi;
-            corrector_incr<P>(row, Hs_p, Hs_m, cfi, fdt, srcc, dPhi, dPi);
+            corrector_incr<P>(row, Hs_p, Hs_m, cfi, qdt, srcc, dPhi, dPi);
             if (row_ok && TK_IN(d.status, o, plane_elems(d))) {
                 NodeV<P> u = uc;
                 u.update(dPhi, dPi);

@@ -14,9 +14,6 @@ template <typename T>
 struct Cx {
     T re, im;
     __device__ __forceinline__ static Cx zero() { return {T(0), T(0)}; }
-    __device__ __forceinline__ static Cx half_sum(Cx a, Cx b) {
-        return {T(0.5) * (a.re + b.re), T(0.5) * (a.im + b.im)};
-    }
 };
 template <typename T>
 __device__ __forceinline__ Cx<T> operator+(Cx<T> a, Cx<T> b) { return {a.re + b.re, a.im + b.im}; }
@@ -60,10 +57,6 @@ __device__ __forceinline__ Cx<float> operator-(Cx<float> a, Cx<float> b) {
 __device__ __forceinline__ Cx<float> neg(Cx<float> a) { return up(__fmul2_rn(bc(-1.0f), pk(a))); }
 __device__ __forceinline__ Cx<float> operator*(float s, Cx<float> a) {
     return up(__fmul2_rn(bc(s), pk(a)));
-}
-template <>
-__device__ __forceinline__ Cx<float> Cx<float>::half_sum(Cx<float> a, Cx<float> b) {
-    return up(__fmul2_rn(bc(0.5f), __fadd2_rn(pk(a), pk(b))));
 }
 // Complex double-float values in paired instructions: the high parts (re, im) and the
 // low parts (re, im) each form a register pair, and every step of the scalar
@@ -135,19 +128,6 @@ __device__ __forceinline__ Cx<DF> cmac(Cx<DF> acc, DF cr, DF ci, Cx<DF> z) {
     const DF2 Ci = {make_float2(-ci.hi, ci.hi), make_float2(-ci.lo, ci.lo)};
     return up2(p_tfma(bc2(cr), Z, p_tfma(Ci, Zs, pk2(acc))));
 }
-template <>
-__device__ __forceinline__ Cx<DF> Cx<DF>::half_sum(Cx<DF> a, Cx<DF> b) {
-    const DF2 s = pk2(a + b);
-    return up2({__fmul2_rn(bc(0.5f), s.hi), __fmul2_rn(bc(0.5f), s.lo)});
-}
-// (a + b)/2 + c (the halving is exact, so one fused operation rounds the same)
-template <typename T>
-__device__ __forceinline__ Cx<T> half_sum_add(Cx<T> a, Cx<T> b, Cx<T> c) {
-    return Cx<T>::half_sum(a, b) + c;
-}
-__device__ __forceinline__ Cx<float> half_sum_add(Cx<float> a, Cx<float> b, Cx<float> c) {
-    return up(__ffma2_rn(bc(0.5f), __fadd2_rn(pk(a), pk(b)), pk(c)));
-}
 __device__ __forceinline__ Cx<float> rmac(Cx<float> acc, float s, Cx<float> z) {
     return up(__ffma2_rn(bc(s), pk(z), pk(acc)));
 }
@@ -211,22 +191,22 @@ struct NodeV {
         else return F - o.F;
     }
     // Split theta differences of Phi at this node from the rows above (a, factor ga)
-    // and below (b, factor gb): d2 = ga a - 2 this + gb b and d1 = ga a - gb b.  For
-    // compensated pairs the hi differences (exact for neighbouring values within a
-    // factor of two) and the c differences are combined first, so d2 and d1 round
+    // and below (b, factor gb), given -ga and -gb: nd2 = -(ga a - 2 this + gb b) and d1 =
+    // ga a - gb b.  For compensated pairs the hi differences (exact for neighbouring values
+    // within a factor of two) and the c differences are combined first, so nd2 and d1 round
     // relative to their own size, not to that of the first differences.
-    __device__ __forceinline__ void theta_split(T ga, const NodeV& a, T gb, const NodeV& b,
-                                                Cx<T>& d2, Cx<T>& d1) const {
-        const Cx<T> hp = rmac(neg(F), ga, a.F);   // ga a - this
-        const Cx<T> hm = rmac(F, -gb, b.F);       // this - gb b
+    __device__ __forceinline__ void theta_split(T nga, const NodeV& a, T ngb, const NodeV& b,
+                                                Cx<T>& nd2, Cx<T>& d1) const {
+        const Cx<T> hp = rmac(F, nga, a.F);   // this - ga a
+        const Cx<T> hm = rmac(F, ngb, b.F);   // this - gb b
         if constexpr (P::kahan) {
-            const Cx<T> cp = rmac(neg(Fc), ga, a.Fc);
-            const Cx<T> cm = rmac(Fc, -gb, b.Fc);
-            d2 = (hp - hm) - (cp - cm);
-            d1 = (hp + hm) - (cp + cm);
+            const Cx<T> cp = rmac(Fc, nga, a.Fc);
+            const Cx<T> cm = rmac(Fc, ngb, b.Fc);
+            nd2 = (hp + hm) - (cp + cm);
+            d1 = (hm - hp) - (cm - cp);
         } else {
-            d2 = hp - hm;
-            d1 = hp + hm;
+            nd2 = hp + hm;
+            d1 = hm - hp;
         }
     }
     __device__ __forceinline__ Cx<T> dpi(const NodeV& o) const {
@@ -371,18 +351,18 @@ template <> struct Planes<PD> {
 template <typename T>
 struct Half { Cx<T> Fb, Pb, dF, dP; };
 
-// Averages and radial differences across the half node i+1/2 (own = column i,
-// nb = column i+1).
+// Sums and radial differences across the half node i+1/2 (own = column i, nb = column
+// i+1): Fb = Phi_i + Phi_{i+1}, Pb the same of Pi.
 template <class P>
 __device__ __forceinline__ Half<typename P::T> half_prep(const NodeV<P>& own, const NodeV<P>& nb) {
     using T = typename P::T;
     Half<T> h;
     if constexpr (P::kahan) {
-        h.Fb = T(0.5) * ((own.F + nb.F) - (own.Fc + nb.Fc));
-        h.Pb = T(0.5) * ((own.Pp + nb.Pp) - (own.Pc + nb.Pc));
+        h.Fb = (own.F + nb.F) - (own.Fc + nb.Fc);
+        h.Pb = (own.Pp + nb.Pp) - (own.Pc + nb.Pc);
     } else {
-        h.Fb = Cx<T>::half_sum(own.F, nb.F);
-        h.Pb = Cx<T>::half_sum(own.Pp, nb.Pp);
+        h.Fb = own.F + nb.F;
+        h.Pb = own.Pp + nb.Pp;
     }
     h.dF = nb.dphi(own);
     h.dP = nb.dpi(own);
@@ -549,31 +529,44 @@ __device__ __forceinline__ T step_qdt(const InstDev& d) {
 }
 
 // ---------------------------------------------------------------- split form
-// Predictor output at one half node, plus the inputs the corrector needs from it
-// (Dp = Fb(j+1) - 2 Fb(j) + Fb(j-1), D1 = Fb(j+1) - Fb(j-1)).
+// FP32 and FP32-Kahan step.  Issue and latency bound it (some 250 instructions a node, four
+// warps a scheduler), so the averages over two and four values stay undivided sums, the
+// powers of two folded into the 1D tables (exactly, so that every result keeps its bits), and
+// the second difference is carried with the sign it is formed with.  us per step before and
+// after: FP32-Kahan 16384 x 256 47.0 -> 46.1, 8192 x 128 14.3 -> 13.8; FP32 36.5 -> 34.9, 11.2
+// -> 10.7.  (Real coefficients times complex values as two scalar FMAs, to save the
+// broadcast of the coefficient into a register pair: no faster, FP32 35.2.)
+// s a + b, s a power of two
+__device__ __forceinline__ Cx<float> sadd(float s, Cx<float> a, Cx<float> b) {
+    return up(__ffma2_rn(bc(s), pk(a), pk(b)));
+}
+
+// Predictor output at one half node, plus the inputs the corrector needs from it: Fb, Pb
+// (sums over the two columns), the radial differences, Dp = -(Fb(j+1) - 2 Fb(j) + Fb(j-1)),
+// D1 = Fb(j+1) - Fb(j-1), and the increments hF, hP.
 template <typename T>
 struct HalfRec { Cx<T> Fb, Pb, dF, dP, Dp, D1, hF, hP; };
 
 // Corrector inputs of one row, combined from the half nodes R = i+1/2 and L = i-1/2.
 template <typename T>
 struct CRow {
-    Cx<T> Hs;        // (dh_Phi_R + dh_Phi_L)/2
-    Cx<T> DpS;       // (Dp_R + Dp_L)/2
-    Cx<T> D1S;       // (D1_R + D1_L)/2
-    Cx<T> FC, PC;    // u~ = (h_R + h_L)/2 for Phi and Pi
+    Cx<T> Hs;        // dh_Phi_R + dh_Phi_L
+    Cx<T> DpS;       // Dp_R + Dp_L
+    Cx<T> D1S;       // D1_R + D1_L
+    Cx<T> FC, PC;    // 4 u~, u~ = (h_R + h_L)/2 for Phi and Pi
     Cx<T> dFc, dPc;  // h_R - h_L for Phi and Pi
 };
 
 template <typename T>
 __device__ __forceinline__ CRow<T> combine_lr(const HalfRec<T>& R, const HalfRec<T>& L) {
     CRow<T> c;
-    c.Hs = Cx<T>::half_sum(R.hF, L.hF);
-    c.DpS = Cx<T>::half_sum(R.Dp, L.Dp);
-    c.D1S = Cx<T>::half_sum(R.D1, L.D1);
-    c.FC = half_sum_add(R.Fb, L.Fb, c.Hs);
-    c.PC = half_sum_add(R.Pb, L.Pb, Cx<T>::half_sum(R.hP, L.hP));
-    c.dFc = half_sum_add(R.dF, L.dF, R.hF - L.hF);
-    c.dPc = half_sum_add(R.dP, L.dP, R.hP - L.hP);
+    c.Hs = R.hF + L.hF;
+    c.DpS = R.Dp + L.Dp;
+    c.D1S = R.D1 + L.D1;
+    c.FC = sadd(2.f, c.Hs, R.Fb + L.Fb);
+    c.PC = sadd(2.f, R.hP + L.hP, R.Pb + L.Pb);
+    c.dFc = sadd(0.5f, R.dF + L.dF, R.hF - L.hF);
+    c.dPc = sadd(0.5f, R.dP + L.dP, R.hP - L.hP);
     return c;
 }
 
@@ -637,7 +630,7 @@ __device__ __forceinline__ void form_coefs2(const RTab2& t, const ThPair& h, flo
     cf[C_E2R] = __ffma2_rn(ctre, g, __fmul2_rn(pb, iS));
     cf[C_E2I] = __ffma2_rn(ctim, g, __fmul2_rn(t.pi, iS));
     const float2 ws = __fmul2_rn(t.Ds, iS);
-    cf[C_EP] = __fmul2_rn(ws, h.i2);   // A (split angular form)
+    cf[C_EP] = __fmul2_rn(ws, h.i2);   // A (split angular form; -A from the forward tables)
     cf[C_EM] = __fmul2_rn(ws, h.i1);   // B
     cf[C_E3R] = __fmul2_rn(__ffma2_rn(t.nDs, h.V, t.qr), iS);
     cf[C_E3I] = __fmul2_rn(t.qi, iS);
@@ -650,19 +643,19 @@ __device__ __forceinline__ void coefs2d(const InstDev& d, bool half, int i, int 
     load_coefs<T>(half ? d.coef_h : d.coef_i, d.pitch, i, j, cf);
 }
 
-// Eq. (13) at the own half node, as an increment on the averaged state.  Dp, Dm: its second
-// and two-cell theta differences.
+// Eq. (13) at the own half node, as an increment on the averaged state.  Dp, D1: the second
+// (negated) and two-cell theta differences of Fb; qdt = dt/4.
 template <typename T>
-__device__ __forceinline__ HalfRec<T> predictor(const Half<T>& h, Cx<T> Dp, Cx<T> Dm, const T* cf,
-                                                T hdt, Cx<T> src) {
+__device__ __forceinline__ HalfRec<T> predictor(const Half<T>& h, Cx<T> Dp, Cx<T> D1, const T* cf,
+                                                T qdt, Cx<T> src) {
     HalfRec<T> r;
-    r.Fb = h.Fb; r.Pb = h.Pb; r.dF = h.dF; r.dP = h.dP; r.Dp = Dp; r.D1 = Dm;
-    r.hF = rmac(rmac(Cx<T>::zero(), -cf[C_G], h.dF), hdt, h.Pb);
+    r.Fb = h.Fb; r.Pb = h.Pb; r.dF = h.dF; r.dP = h.dP; r.Dp = Dp; r.D1 = D1;
+    r.hF = rmac(rmac(Cx<T>::zero(), -cf[C_G], h.dF), qdt, h.Pb);
     Cx<T> a = rmac(src, cf[C_G], h.dP);
     a = cmac(a, cf[C_E1R], cf[C_E1I], h.Pb);
     a = cmac(a, cf[C_E2R], cf[C_E2I], h.dF);
     a = rmac(a, cf[C_EP], Dp);
-    a = rmac(a, cf[C_EM], Dm);
+    a = rmac(a, cf[C_EM], D1);
     a = cmac(a, cf[C_E3R], cf[C_E3I], h.Fb);
     r.hP = a;
     return r;
@@ -699,14 +692,14 @@ __device__ __forceinline__ void xread(const float* mine, Cx<float>& Hs_p, Cx<flo
 // the theta neighbours' exchange entries, the node's coefficients cf and source term.
 template <class P>
 __device__ __forceinline__ void corrector_incr(const CRow<typename P::T>& row, Cx<typename P::T> Hs_p,
-                                               Cx<typename P::T> Hs_m, const typename P::T* cf, typename P::T fdt,
+                                               Cx<typename P::T> Hs_m, const typename P::T* cf, typename P::T qdt,
                                                Cx<typename P::T> srcc, Cx<typename P::T>& dPhi,
                                                Cx<typename P::T>& dPi) {
     using C = Cx<typename P::T>;
-    // second and two-cell differences of the corrector's averaged state u~ = (h_R + h_L)/2
-    const C Dplus = row.DpS + ((Hs_p - row.Hs) - (row.Hs - Hs_m));
-    const C Dminus = row.D1S + (Hs_p - Hs_m);
-    dPhi = rmac(rmac(C::zero(), -cf[C_G], row.dFc), fdt, row.PC);
+    // second (negated) and two-cell differences of 4 u~
+    const C Dplus = sadd(-2.f, (Hs_p - row.Hs) - (row.Hs - Hs_m), row.DpS);
+    const C Dminus = sadd(2.f, Hs_p - Hs_m, row.D1S);
+    dPhi = rmac(rmac(C::zero(), -cf[C_G], row.dFc), qdt, row.PC);
     dPi = rmac(srcc, cf[C_G], row.dPc);
     dPi = cmac(dPi, cf[C_E1R], cf[C_E1I], row.PC);
     dPi = cmac(dPi, cf[C_E2R], cf[C_E2I], row.dFc);
