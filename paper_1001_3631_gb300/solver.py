@@ -6,7 +6,10 @@ from __future__ import annotations
 
 import ctypes
 import json
+import mmap
 import os
+import threading
+import weakref
 
 import numpy as np
 
@@ -85,6 +88,51 @@ def _stream_handle(stream):
     return stream.cuda_stream
 
 
+class _HostBuffers:
+    """Result arrays whose memory is used again once the caller has dropped them (every view
+    included).  A fresh array of 134 MB (a 16384 x 256 state) costs 6 to 20 ms of page faults
+    and unmapping a call, on GB300 with its fast host link the copy itself 0.9 ms.  Arrays
+    below 4 MB come from numpy (its heap reuses them); at most KEEP bytes are kept idle, by the solver that made
+    them (any thread may drop an array or ask for one)."""
+    MIN, KEEP = 4 << 20, 1 << 30
+
+    def __init__(self):
+        self._lock = threading.Lock()
+        self._bufs = []   # [mapping, weak reference to the object that its arrays hold], oldest first
+
+    def empty(self, shape, dtype=np.float64):
+        dtype = np.dtype(dtype)
+        count = 1
+        for n in shape:
+            count *= int(n)
+        size = count * dtype.itemsize
+        if size < self.MIN:
+            return np.empty(shape, dtype)
+        with self._lock:
+            idle = [b for b in self._bufs if b[1]() is None]
+            buf = next((b for b in idle if len(b[0]) == size), None)
+            if buf is None:
+                m = mmap.mmap(-1, size, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS)
+                try:   # (as numpy does for its own arrays)
+                    m.madvise(mmap.MADV_HUGEPAGE)
+                except (AttributeError, OSError):
+                    pass
+                buf = [m, None]
+            else:
+                idle.remove(buf)
+                self._bufs.remove(buf)
+            self._bufs.append(buf)
+            kept = sum(len(b[0]) for b in idle)
+            for b in idle:
+                if kept <= self.KEEP:
+                    break
+                self._bufs.remove(b)
+                kept -= len(b[0])
+            raw = (ctypes.c_char * size).from_buffer(buf[0])
+            buf[1] = weakref.ref(raw)   # dead when the last array on the mapping is gone
+        return np.frombuffer(raw, dtype, count).reshape(shape)
+
+
 class TeukSolver:
     """One context of one or more instances (see teuk_create)."""
 
@@ -93,6 +141,7 @@ class TeukSolver:
             params = [params]
         plist = [p if isinstance(p, _lib.teuk_params) else make_params(**p) for p in params]
         self.n = len(plist)
+        self._host = _HostBuffers()
         arr = (_lib.teuk_params * self.n)(*plist)
         self.params = plist
         self._stream = stream
@@ -162,7 +211,7 @@ class TeukSolver:
         check(_lib.load().teuk_set_state(self.ctx, instance, ptr(u), step0), self.ctx)
 
     def get_state(self, instance=0):
-        u = np.empty(self.shape(instance))
+        u = self._host.empty(self.shape(instance))
         check(_lib.load().teuk_get_state(self.ctx, instance, ptr(u)), self.ctx)
         return u
 
@@ -175,7 +224,7 @@ class TeukSolver:
         step, _ = self.time(instance)
         if cap is None:
             cap = step + 1
-        out = np.empty((cap, p.n_theta, 2))
+        out = self._host.empty((cap, p.n_theta, 2))
         sc = np.empty((cap, 2)) if scalar else None
         nw, first = ctypes.c_int64(0), ctypes.c_int64(0)
         check(_lib.load().teuk_extract(self.ctx, instance, ptr(out), ptr(sc), cap,
@@ -191,10 +240,10 @@ class TeukSolver:
         azimuths phi: complex array [n_records][n_theta][len(phi)]."""
         ph = np.ascontiguousarray(np.atleast_1d(phi), dtype=np.float64)
         nth = self.params[0].n_theta
-        out = np.empty((n_records, nth, ph.size, 2))
+        out = self._host.empty((n_records, nth, ph.size), np.complex128)   # (re, im) pairs
         check(_lib.load().teuk_mode_sum(self.ctx, ptr(ph), ph.size, int(first), int(n_records),
                                         ptr(out)), self.ctx)
-        return out[..., 0] + 1j * out[..., 1]
+        return out
 
     def radiated_flux(self, first, n_records):
         """Energy, linear momentum and Jz carried off by the field of the instances (distinct
