@@ -224,8 +224,9 @@ teuk_status teuk_extract(teuk_ctx* ctx, int instance, double* out, double* out_s
  *   phi~_l = phi[l] + a/(r_+ - r_-) ln((r_ext - r_+)/(r_ext - r_-))      (Eq. 3)
  * for the time levels first .. first + n_records - 1 (each held by every instance,
  * see teuk_extract) and the azimuths phi[0 .. n_phi-1] (host), instances added in
- * index order, in one kernel.  out: host [n_records][n_theta][n_phi][2] (re, im).
- * Allocates and frees 16 n_records n_theta n_phi bytes of device memory; synchronizes.
+ * index order, in kernels (the phases of the modes and azimuths, then the sum).  out: host
+ * [n_records][n_theta][n_phi][2] (re, im).  Allocates and frees 16 (n_records n_theta +
+ * n_instances) n_phi bytes of device memory and some; synchronizes.
  * TEUK_EINVAL if the instances are not modes of one problem, a record is not held,
  * or n_phi < 1. */
 teuk_status teuk_mode_sum(teuk_ctx* ctx, const double* phi, int n_phi, int64_t first,

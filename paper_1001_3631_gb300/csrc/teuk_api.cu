@@ -1386,7 +1386,7 @@ static teuk_status modes_of_problem(teuk_ctx* c, int64_t first, int64_t n_record
             TK_FAIL(c, TEUK_EINVAL, "instance %d holds records [%lld, %lld), not [%lld, %lld)", (int)i,
                     (long long)I.wave_lo, (long long)I.wave_hi, (long long)first,
                     (long long)(first + n_records));
-        modes[i] = ModeRing{I.wave, I.wave_cap, I.p.m, 0};
+        modes[i] = ModeRing{I.wave, I.wave_cap, first % I.wave_cap, I.p.m, 0};
     }
     return TEUK_OK;
 }
@@ -1410,15 +1410,16 @@ extern "C" teuk_status teuk_mode_sum(teuk_ctx* c, const double* phi, int n_phi, 
     char* buf = nullptr;
     const size_t b_modes = (sizeof(ModeRing) * modes.size() + 255) / 256 * 256;
     const size_t b_phi = (sizeof(double) * n_phi + 255) / 256 * 256;
-    TK_CUDA(c, dmalloc(c, (void**)&buf, b_modes + b_phi + sizeof(double2) * n_out, c->stream));
+    const size_t b_phase = (sizeof(double2) * modes.size() * n_phi + 255) / 256 * 256;
+    TK_CUDA(c, dmalloc(c, (void**)&buf, b_modes + b_phi + b_phase + sizeof(double2) * n_out, c->stream));
     ModeRing* d_modes = (ModeRing*)buf;
     double* d_phi = (double*)(buf + b_modes);
-    double2* d_out = (double2*)(buf + b_modes + b_phi);
+    double2* d_phase = (double2*)(buf + b_modes + b_phi);
+    double2* d_out = (double2*)(buf + b_modes + b_phi + b_phase);
     cudaMemcpyAsync(d_modes, modes.data(), sizeof(ModeRing) * modes.size(), cudaMemcpyHostToDevice, c->stream);
     cudaMemcpyAsync(d_phi, phi, sizeof(double) * n_phi, cudaMemcpyHostToDevice, c->stream);
-    launch_mode_sum(c->stream, d_modes, (int)modes.size(), nth, d_phi, n_phi, first, n_records,
-                    r_ext * r_ext * r_ext, shift, d_out);
-    c->launches++;
+    c->launches += launch_mode_sum(c->stream, d_modes, (int)modes.size(), nth, d_phi, n_phi, n_records,
+                                   r_ext * r_ext * r_ext, shift, d_phase, d_out);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(out, d_out, sizeof(double2) * n_out, cudaMemcpyDeviceToHost, c->stream);
@@ -1487,7 +1488,7 @@ extern "C" teuk_status teuk_radiated_flux(teuk_ctx* c, int64_t first, int64_t n_
     fs.out = (double*)take(b_out);
     cudaMemcpyAsync(d_modes, modes.data(), sizeof(ModeRing) * K, cudaMemcpyHostToDevice, c->stream);
     cudaMemcpyAsync(d_part, partner.data(), sizeof(int) * K, cudaMemcpyHostToDevice, c->stream);
-    const FluxDev f{d_modes, K, nth, first, n_records, (int)Lc, (int)n_chunks, RB, n_rg,
+    const FluxDev f{d_modes, K, nth, n_records, (int)Lc, (int)n_chunks, RB, n_rg,
                     I0.dt, r_ext, I0.p.a, shift};
     c->launches += launch_radiated_flux(c->stream, f, fs);
     cudaError_t e = cudaGetLastError();

@@ -1,6 +1,8 @@
 // teuk_aux.cu -- small kernels around the time step: conversion between the host
 // u-layout and the internal planes, the finiteness scan, the sin(theta)-weighted
 // theta sum of the waveform records, and the sum of the records over modes.
+#include <algorithm>
+
 #include "teuk_aux.cuh"
 #include "teuk_internal.cuh"
 #include "teuk_step_common.cuh"
@@ -117,40 +119,53 @@ void launch_wave_sum(cudaStream_t st, const double2* wave, int64_t cap, int nth,
                                                                      k_count, out);
 }
 
-// Thread per (record k, row j, azimuth l), grid-stride; the modes are added in order.
-__global__ void mode_sum_kernel(const ModeRing* modes, int n_modes, int nth, const double* phi,
-                                int n_phi, int64_t first, int64_t n_rec, double r3, double shift,
-                                double2* out) {
-    const int64_t total = n_rec * nth * n_phi;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int l = (int)(idx % n_phi);
-        const int64_t t = idx / n_phi;
-        const int j = (int)(t % nth);
-        const int64_t k = t / nth;
-        const double ph = phi[l] + shift;
-        double re = 0.0, im = 0.0;
-        for (int i = 0; i < n_modes; ++i) {
-            const ModeRing q = modes[i];
-            const double2 w = q.wave[(size_t)((first + k) % q.cap) * nth + j];
-            double sn, cs;
-            sincos((double)q.m * ph, &sn, &cs);
-            re += cs * w.x - sn * w.y;
-            im += cs * w.y + sn * w.x;
-        }
-        out[idx] = make_double2(r3 * re, r3 * im);
+// phase[i][l] = e^{i m_i (phi[l] + shift)}
+__global__ void mode_phase_kernel(const ModeRing* modes, int n_modes, const double* phi, int n_phi, double shift,
+                                  double2* phase) {
+    const int64_t total = (int64_t)n_modes * n_phi;
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
+        double sn, cs;
+        sincos((double)modes[q / n_phi].m * (phi[q % n_phi] + shift), &sn, &cs);
+        phase[q] = make_double2(cs, sn);
     }
 }
 
-void launch_mode_sum(cudaStream_t st, const ModeRing* modes, int n_modes, int nth,
-                     const double* phi, int n_phi, int64_t first, int64_t n_rec, double r3,
-                     double shift, double2* out) {
-    const int64_t total = n_rec * nth * n_phi;
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    if (blocks < 1) blocks = 1;
-    mode_sum_kernel<<<(unsigned)blocks, 256, 0, st>>>(modes, n_modes, nth, phi, n_phi, first,
-                                                      n_rec, r3, shift, out);
+// Block column x: record k; the threads of block row y take (row j, azimuth l), l fastest;
+// the modes are added in order.  Bound by the FP64 pipe (4 operations a mode and output):
+// the phases come from a table (a sincos an output and mode, some 100 operations, had taken
+// ten times the sum; 6 modes, 250 records x 128 rows x 16 azimuths: 280 -> 125 us a call, host copy included).  U: the type of
+// the index within a record (32 bits when it fits: its division is the other large cost).
+template <typename U>
+__global__ void mode_sum_kernel(const ModeRing* modes, int n_modes, int nth, U n_phi, const double2* phase, double r3,
+                                double2* out) {
+    const int64_t k = blockIdx.x;
+    const U total = (U)nth * n_phi;
+    double2* o = out + (size_t)k * total;
+    for (U q = (U)blockIdx.y * blockDim.x + threadIdx.x; q < total; q += (U)gridDim.y * blockDim.x) {
+        const U j = q / n_phi, l = q - j * n_phi;
+        double re = 0.0, im = 0.0;
+        for (int i = 0; i < n_modes; ++i) {
+            const double2 w = modes[i].record(k, nth)[j], e = phase[(size_t)i * n_phi + l];
+            re += e.x * w.x - e.y * w.y;
+            im += e.x * w.y + e.y * w.x;
+        }
+        o[q] = make_double2(r3 * re, r3 * im);
+    }
+}
+
+int launch_mode_sum(cudaStream_t st, const ModeRing* modes, int n_modes, int nth,
+                    const double* phi, int n_phi, int64_t n_rec, double r3, double shift,
+                    double2* phase, double2* out) {
+    const int64_t np = (int64_t)n_modes * n_phi, total = (int64_t)nth * n_phi;
+    mode_phase_kernel<<<(unsigned)std::min<int64_t>((np + 63) / 64, 1024), 64, 0, st>>>(modes, n_modes, phi, n_phi,
+                                                                                      shift, phase);
+    const unsigned gy = (unsigned)std::min<int64_t>((total + 255) / 256, 65535);
+    const dim3 g((unsigned)n_rec, gy);
+    if (total <= ((int64_t)1 << 31))   // (the stride past the end stays within 32 bits)
+        mode_sum_kernel<uint32_t><<<g, 256, 0, st>>>(modes, n_modes, nth, (uint32_t)n_phi, phase, r3, out);
+    else
+        mode_sum_kernel<uint64_t><<<g, 256, 0, st>>>(modes, n_modes, nth, (uint64_t)n_phi, phase, r3, out);
+    return 2;
 }
 
 // (checked builds) the bounds check of an index one past the end of the state plane; the

@@ -55,7 +55,7 @@ __device__ double2 entry_factor(const FluxDev& f, int i, double cth) {
 }
 
 __device__ __forceinline__ double2 record(const FluxDev& f, const ModeRing& q, int j, int64_t k) {
-    return q.wave[(size_t)((f.first + k) % q.cap) * f.nth + j];
+    return q.record(k, f.nth)[j];
 }
 
 // chunk c advances the records s_c -> e_c (s_0 = 0, s_c = c Lc - 1, e_c = min((c+1) Lc, R) - 1)
