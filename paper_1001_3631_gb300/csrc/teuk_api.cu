@@ -90,7 +90,7 @@ struct Instance {
 
 // Device side of the batched persistent launch of one context: one persistent kernel
 // per block-size class (instances whose theta pitch is the same), run one after the
-// other (classes are independent).
+// other or side by side (plan_branches; classes are independent).
 struct BatchClass {
     int pitch = 0;                  // threads per block
     std::vector<int> members;       // instance indices
@@ -99,7 +99,10 @@ struct BatchClass {
     int* d_flags = nullptr;
     int64_t flags_cap = 0;
     int64_t items = -1;
-    int grid = 0;
+    int grid = 0;                   // blocks the GPU holds at once
+    int share = 0;                  // blocks of a concurrent launch beside the other classes
+    cudaStream_t side = nullptr;    // its branch of the captured graph (classes but the first)
+    cudaEvent_t done = nullptr;
     int max_nth = 0;
     bool moving = false;            // a member has a moving particle
     BatchDev bd{};
@@ -114,6 +117,8 @@ struct Batch {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     bool graph_failed = false;
+    bool branches = false;          // the classes run side by side
+    cudaEvent_t fork = nullptr;
 };
 
 }  // namespace
@@ -988,15 +993,106 @@ void invalidate_graph(teuk_ctx* c) {
     B.graph = nullptr;
 }
 
+void enqueue_class(teuk_ctx* c, BatchClass& K, cudaStream_t st, int grid) {
+    cudaMemsetAsync(K.d_counter, 0, sizeof(unsigned long long), st);
+    cudaMemsetAsync(K.d_flags, 0, sizeof(int) * K.items, st);
+    launch_batched_step(st, c->prec, K.bd, grid, K.pitch, K.moving);
+    launch_batched_extract(st, c->prec, K.bd, K.max_nth);
+}
+
+// One class after the other, each on the whole GPU.
 void enqueue_batched(teuk_ctx* c, cudaStream_t st) {
     Batch& B = c->batch;
     cudaMemsetAsync(B.d_abort, 0, sizeof(int), st);
-    for (BatchClass& K : B.cls) {
-        cudaMemsetAsync(K.d_counter, 0, sizeof(unsigned long long), st);
-        cudaMemsetAsync(K.d_flags, 0, sizeof(int) * K.items, st);
+    for (BatchClass& K : B.cls) enqueue_class(c, K, st, K.grid);
+}
+
+// The classes side by side (capture only): each a branch of its own with its share of the
+// GPU's places, so that the waits of one class for its neighbours' strips are filled with
+// another's work.
+void enqueue_batched_branches(teuk_ctx* c, cudaStream_t st) {
+    Batch& B = c->batch;
+    cudaMemsetAsync(B.d_abort, 0, sizeof(int), st);
+    cudaEventRecord(B.fork, st);
+    for (size_t k = 1; k < B.cls.size(); ++k) {
+        BatchClass& K = B.cls[k];
+        cudaStreamWaitEvent(K.side, B.fork, 0);
+        enqueue_class(c, K, K.side, K.share);
+        cudaEventRecord(K.done, K.side);
     }
-    for (BatchClass& K : B.cls) launch_batched_step(st, c->prec, K.bd, K.grid, K.pitch, K.moving);
-    for (BatchClass& K : B.cls) launch_batched_extract(st, c->prec, K.bd, K.max_nth);
+    enqueue_class(c, B.cls[0], st, B.cls[0].share);
+    for (size_t k = 1; k < B.cls.size(); ++k) cudaStreamWaitEvent(st, B.cls[k].done, 0);
+}
+
+// Whether the classes run side by side, and their shares: a whole number of blocks of every
+// class on each SM (512 threads at the kernels' 128 registers), so that the launches find
+// their places whatever their order; blocks are added where a block has most columns.
+// us per step, one class after the other -> side by side: 6 modes of 1024..4100 columns and 64,
+// 128, 192 rows, FP32-Kahan 46.2 -> 37.0, double-float 118.8 -> 96.1; two of them 19.6 -> 13.1.
+// Not so with few columns (6 modes of 20..60 rows, 4.4 columns a place: 20.0 -> 22.0) or many
+// (128 instances, 2000 columns a place: 1727 -> 1900, an eighth of the threads left over).
+void plan_branches(teuk_ctx* c, Batch& B) {
+    constexpr int kThreads = 512;
+    std::vector<double> work(B.cls.size(), 0.0);
+    std::vector<int> n(B.cls.size(), 1);
+    double total = 0.0;
+    int used = 0;
+    for (size_t k = 0; k < B.cls.size(); ++k) {
+        BatchClass& K = B.cls[k];
+        if (!K.grid) K.grid = batched_grid(c->prec, K.pitch);
+        for (int q : K.members) work[k] += (double)c->inst[q].p.n_rstar * K.pitch;
+        total += work[k];
+        used += K.pitch;
+    }
+    auto load = [&](size_t k) { return work[k] / ((double)n[k] * B.cls[k].pitch); };
+    B.branches = B.cls.size() > 1 && used <= kThreads;
+    if (!B.branches) return;
+    for (;;) {
+        size_t best = B.cls.size();
+        for (size_t k = 0; k < B.cls.size(); ++k)
+            if (used + B.cls[k].pitch <= kThreads && (n[k] + 1) * c->sms <= B.cls[k].grid &&
+                (best == B.cls.size() || load(k) > load(best)))
+                best = k;
+        if (best == B.cls.size()) break;
+        used += B.cls[best].pitch;
+        ++n[best];
+    }
+    double longest = 0.0;
+    for (size_t k = 0; k < B.cls.size(); ++k) {
+        longest = std::max(longest, load(k));
+        B.cls[k].share = n[k] * c->sms;
+    }
+    // well balanced, and of a size that waiting matters in: columns a place, all classes
+    const double columns = total / kThreads / c->sms;
+    B.branches = longest <= 1.3 * total / kThreads && columns >= 5.0 && columns <= 100.0;
+}
+
+// The side streams and events of the branches; false if they cannot be had (the classes then
+// run one after the other).
+bool batch_branches(Batch& B) {
+    if (B.cls.size() < 2) return false;
+    bool ok = B.fork || cudaEventCreateWithFlags(&B.fork, cudaEventDisableTiming) == cudaSuccess;
+    for (size_t k = 1; ok && k < B.cls.size(); ++k) {
+        BatchClass& K = B.cls[k];
+        if (!K.side) ok = cudaStreamCreateWithFlags(&K.side, cudaStreamNonBlocking) == cudaSuccess;
+        if (ok && !K.done) ok = cudaEventCreateWithFlags(&K.done, cudaEventDisableTiming) == cudaSuccess;
+    }
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
+// Strip length of instance I in a launch of its class on `grid` blocks: its own, the
+// context's, or the length that gives the blocks one and a half strips of the class a step
+// each: with one, every block waits for its neighbours' previous step; more cost columns
+// computed twice (us per step of the 6 modes above with 1, 1.5, 2, 3 strips: 44.5, 37.0, 39.5,
+// 45.8; one wave of each instance by itself, as a single instance takes: 51.5; the 128
+// instances 1817, 1727, 1730, 1743; 2415).
+int batch_strip(const teuk_ctx* c, const Instance& I, const BatchClass& K, int grid) {
+    if (I.strip > 0 || c->strip > 0) return eff_strip(c, I);
+    int64_t cols = 0;
+    for (int q : K.members) cols += c->inst[q].p.n_rstar - 2;
+    const int64_t L = (2 * cols + 3 * (int64_t)grid - 1) / (3 * (int64_t)grid);
+    return (int)std::max<int64_t>(1, std::min<int64_t>({L, 512, I.p.n_rstar - 2}));
 }
 
 // All instances advance n steps: one persistent launch per block-size class, captured
@@ -1018,6 +1114,7 @@ teuk_status batched_step(teuk_ctx* c, int64_t n) {
             K->members.push_back(k);
         }
     }
+    plan_branches(c, B);
     // per-class descriptor blocks:
     // InstDev[m] | item_base[m+1] | base_step[m] | n_steps | strip[m] | nstrip[m] | base_bin[m]
     std::vector<char> blob;
@@ -1038,7 +1135,7 @@ teuk_status batched_step(teuk_ctx* c, int64_t n) {
         bool moving = false;
         for (int q = 0; q < m; ++q) {
             Instance& I = c->inst[K.members[q]];
-            strip[q] = eff_strip(c, I);
+            strip[q] = batch_strip(c, I, K, B.branches ? K.share : K.grid);
             nstrip[q] = (I.p.n_rstar - 2 + strip[q] - 1) / strip[q];
             ib[q + 1] = ib[q] + nstrip[q];
             bs[q] = I.step;
@@ -1080,7 +1177,6 @@ teuk_status batched_step(teuk_ctx* c, int64_t n) {
         B.blob_bytes = blob.size();
         for (BatchClass& K : B.cls) {
             TK_CUDA(c, dmalloc(c, (void**)&K.d_counter, sizeof(unsigned long long), c->stream));
-            K.grid = batched_grid(c->prec, K.pitch);
         }
         B.alloc = true;
         changed = true;
@@ -1116,7 +1212,8 @@ teuk_status batched_step(teuk_ctx* c, int64_t n) {
     if (!B.exec && !B.graph_failed && cs) {
         cudaGraph_t g = nullptr;
         if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-            enqueue_batched(c, cs);
+            if (B.branches && batch_branches(B)) enqueue_batched_branches(c, cs);
+            else enqueue_batched(c, cs);
             if (cudaStreamEndCapture(cs, &g) == cudaSuccess && g &&
                 cudaGraphInstantiate(&B.exec, g, 0) == cudaSuccess) {
                 B.graph = g;
@@ -1869,7 +1966,10 @@ extern "C" void teuk_destroy(teuk_ctx* c) {
         void* ptrs[] = {B.d_blob, B.d_abort};
         for (void* q : ptrs)
             if (q) dfree(c, q, c->stream);
+        if (B.fork) cudaEventDestroy(B.fork);
         for (BatchClass& K : B.cls) {
+            if (K.side) cudaStreamDestroy(K.side);
+            if (K.done) cudaEventDestroy(K.done);
             if (K.d_counter) dfree(c, K.d_counter, c->stream);
             if (K.d_flags) dfree(c, K.d_flags, c->stream);
         }
