@@ -349,8 +349,8 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
                         C dPhi, dPi;
                         correct_x<T, true>(A, Rh, Lh, A.add(Rh.F, Lh.F), S_p, S_m, cf, qdt, s_i, dPhi, dPi);
                         NodeV<P> u = S.load(sidx(k, j));
-                        u.F = A.add(u.F, dPhi);
-                        u.Pp = A.add(u.Pp, dPi);
+                        u.F = A.update(u.F, dPhi);
+                        u.Pp = A.update(u.Pp, dPi);
                         S.store(sidx(k, j), u);
                     }
                 }

@@ -337,8 +337,8 @@ __device__ __forceinline__ void strip_columns_x(const InstDev& d, int64_t step, 
             correct_x<T, kSrc>(A, Rh, L, S, S_p, S_m, ci, qdt, srcc, dPhi, dPi);
             if (row_ok && TK_IN(d.status, o, plane_elems(d))) {
                 NodeV<P> v = u;
-                v.F = A.add(v.F, dPhi);
-                v.Pp = A.add(v.Pp, dPi);
+                v.F = A.update(v.F, dPhi);
+                v.Pp = A.update(v.Pp, dPi);
                 out.store(o, v);
             }
             L = Rh;

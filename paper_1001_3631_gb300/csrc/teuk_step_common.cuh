@@ -69,7 +69,7 @@ __device__ __forceinline__ DF2 pk2(Cx<DF> a) {
 __device__ __forceinline__ Cx<DF> up2(DF2 v) { return {DF(v.hi.x, v.lo.x), DF(v.hi.y, v.lo.y)}; }
 __device__ __forceinline__ float2 p_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 p_sub(float2 a, float2 b) { return __ffma2_rn(bc(-1.0f), b, a); }   // exact product
-__device__ __forceinline__ float2 p_neg(float2 a) { return __fmul2_rn(bc(-1.0f), a); }
+__device__ __forceinline__ float2 p_neg(float2 a) { return make_float2(-a.x, -a.y); }
 // s + e = a + b exactly (per component)
 __device__ __forceinline__ DF2 p_two_sum(float2 a, float2 b) {
     const float2 s = p_add(a, b);
@@ -100,14 +100,16 @@ __device__ __forceinline__ Cx<DF> neg(Cx<DF> a) {
     const DF2 A = pk2(a);
     return up2({p_neg(A.hi), p_neg(A.lo)});
 }
-// a * b + c per component, a given as pairs (hi, lo): the double-float tfma
+// a * b + c per component, a given as pairs (hi, lo): the double-float tfma without its last
+// normalisation, so that lo may reach a few units in the last place of hi (one per link of a
+// chain of such sums)
 __device__ __forceinline__ DF2 p_tfma(DF2 A, DF2 B, DF2 C) {
     const float2 p = __fmul2_rn(A.hi, B.hi);
     float2 e = __ffma2_rn(A.hi, B.hi, p_neg(p));
     e = __ffma2_rn(A.hi, B.lo, e);
     e = __ffma2_rn(A.lo, B.hi, e);
     const DF2 S = p_two_sum(p, C.hi);
-    return p_fast_two_sum(S.hi, p_add(S.lo, p_add(e, C.lo)));
+    return {S.hi, p_add(S.lo, p_add(e, C.lo))};
 }
 __device__ __forceinline__ DF2 bc2(DF s) { return {bc(s.hi), bc(s.lo)}; }
 __device__ __forceinline__ Cx<DF> operator*(DF s, Cx<DF> a) {
@@ -415,17 +417,39 @@ template <> struct Lin<double> {
     __device__ __forceinline__ C add(C a, C b) const {
         return {__fma_rn(a.re, one, b.re), __fma_rn(a.im, one, b.im)};
     }
+    __device__ __forceinline__ C update(C a, C b) const { return add(a, b); }
     __device__ __forceinline__ C sub(C a, C b) const {
         return {__fma_rn(b.re, -one, a.re), __fma_rn(b.im, -one, a.im)};
     }
     __device__ __forceinline__ C mul(double s, C a) const { return {__fma_rn(s, a.re, 0.0), __fma_rn(s, a.im, 0.0)}; }
 };
+// Double-float: the sums, differences and products of a step's chain stay unnormalised (three
+// operations saved in each; as in Ogita, Rump and Oishi's compensated dot product, the
+// residues are summed apart), only the state that is stored is normalised (update).  The
+// error against 64 bits is the same (8192 x 128, 300 steps: 1.83e-14 both; 3001 x 300: 1.60e-14
+// both).  us per step: 16384 x 256 148 -> 136 (the tables and the state alone take 129 at the
+// measured copy rate), 8192 x 128 43.5 -> 37.9, 800 x 64 5.4 -> 4.8.
 template <> struct Lin<DF> {
     using C = Cx<DF>;
     __device__ __forceinline__ explicit Lin(const InstDev&) {}
-    __device__ __forceinline__ C add(C a, C b) const { return a + b; }
-    __device__ __forceinline__ C sub(C a, C b) const { return a - b; }
-    __device__ __forceinline__ C mul(DF s, C a) const { return s * a; }
+    __device__ __forceinline__ C update(C a, C b) const { return a + b; }
+    __device__ __forceinline__ C add(C x, C y) const {
+        const DF2 X = pk2(x), Y = pk2(y);
+        const DF2 S = p_two_sum(X.hi, Y.hi);
+        return up2({S.hi, p_add(S.lo, p_add(X.lo, Y.lo))});
+    }
+    __device__ __forceinline__ C sub(C x, C y) const {
+        const DF2 X = pk2(x), Y = pk2(y);
+        const DF2 S = p_two_diff(X.hi, Y.hi);
+        return up2({S.hi, p_add(S.lo, p_sub(X.lo, Y.lo))});
+    }
+    __device__ __forceinline__ C mul(DF s, C a) const {
+        const DF2 S = bc2(s), A = pk2(a);
+        const float2 p = __fmul2_rn(S.hi, A.hi);
+        float2 e = __ffma2_rn(S.hi, A.hi, p_neg(p));
+        e = __ffma2_rn(S.hi, A.lo, e);
+        return up2({p, __ffma2_rn(S.lo, A.hi, e)});
+    }
 };
 
 template <> struct Lin<float> {   // (the FP32 paths take the split form)
