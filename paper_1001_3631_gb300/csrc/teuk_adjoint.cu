@@ -294,7 +294,7 @@ __device__ __forceinline__ void adj_wait_prev() { asm volatile("griddepcontrol.w
 // 2 h (adj_src_grad_kernel doubles it).
 template <typename T, int kMaxT>
 __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin, const double2* gbar,
-                                                         CoLevel lout, int /*strip*/, void* wh, void* wi) {
+                                                         CoLevel lout, void* wh, void* wi) {
     using Zd = Z<double>;
     extern __shared__ __align__(16) unsigned char adj_smem[];
     adj_release_next();
@@ -440,13 +440,13 @@ __device__ __forceinline__ Z<float> theta_cot_v(const CfF& c, float ep_m, float 
     return r;
 }
 
-// columns of radial tables the FP32 reverse step stages in shared memory (strips of up
-// to kAdjRtCols - 2 columns; longer strips read the tables from global memory)
+// columns of radial tables the FP32 reverse step stages in shared memory (pieces of up
+// to kAdjRtCols - 2 columns; longer ones read the tables from global memory)
 constexpr int kAdjRtCols = 64;
 
 template <int kMaxT>
 __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel lin, const double2* gbar,
-                                                             CoLevel lout, int strip, void* wh, void* wi) {
+                                                             CoLevel lout, void* wh, void* wi) {
     using R = float;
     extern __shared__ __align__(16) unsigned char adj_smem[];
     adj_release_next();
@@ -456,8 +456,9 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel 
     float4* EB = (float4*)(MB + 2 * (size_t)pitch);   // [3][pitch] {ep, em} of node, half node
     RTab2* RT = (RTab2*)(EB + 3 * (size_t)pitch);      // radial tables of columns c0-1 .. c1
     const bool row_ok = j < nth;
-    const int c0 = blockIdx.x * strip, c1 = min(nr, c0 + strip);   // output columns [c0, c1)
-    const bool rt_smem = strip + 2 <= kAdjRtCols;   // else the tables are read from global
+    // output columns [c0, c1): one of gridDim.x pieces of equal length to a column
+    const int c0 = (int)((int64_t)blockIdx.x * nr / gridDim.x), c1 = (int)((int64_t)(blockIdx.x + 1) * nr / gridDim.x);
+    const bool rt_smem = c1 - c0 + 2 <= kAdjRtCols;   // else the tables are read from global
     const R g = d.ghost_f, hdt = d.hdt2.x, qdt = d.hdt2.x;
     const SourceDev& s = d.src;
     // wh, wi: this step's ring slot of the window co-states (null: no source)
@@ -718,30 +719,33 @@ static void adj_dispatch(int prec, int t, F f) {
 // 128 in 512 strips 85, in 304 pieces 49; 4096 x 128 in 820 strips 106, in 456 pieces 88 (304:
 // 102).  More blocks have more columns at their edges computed twice; two an SM hide too
 // little latency once a piece is longer than some six columns.
-// FP32 co-state: one wave of strips of at least four columns.
+// FP32 co-state: a piece for every place the GPU has, or, while a piece would have less than
+// three columns, half as many places (down to four an SM), capped.  us per step, one wave of
+// strips of at least four columns -> this: 512 x 32 6.1 -> 3.7, 1024 x 64 9.4 -> 5.2, 2048 x 128
+// 10.0 -> 9.7, 4096 x 64 9.8 -> 9.4, 4096 x 128 14.0.
 AdjCut adj_step_plan(const InstDev& d) {
-    int res = 1;
+    int res = 1, dev = 0, sms = 0;
     adj_dispatch(d.prec, d.pitch, [&](auto kernel, size_t sm) {
-        // (blocks of more than 256 rows take more than the default 48 KB)
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        // (blocks of more than 256 rows, and capped ones, take more than the default 48 KB)
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)capped_smem(4, sm));
         res = adj_resident(kernel, d.pitch, sm);
     });
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (sms < 1) sms = 1;
+    const int places = std::max(1, res / sms);
     if (d.prec == 0 || d.prec == 3) {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms < 1) sms = 1;
-        const int per = std::min(res / sms, d.nr >= 6 * 3 * sms ? 3 : 2);
-        return {0, std::max(1, std::min(per * sms, d.nr / 2))};
+        const int per = std::min(places, d.nr >= 6 * 3 * sms ? 3 : 2);
+        return {std::max(1, std::min(per * sms, d.nr / 2)), 0};
     }
-    int L = (d.nr + res - 1) / res;   // one wave of resident blocks, >= 4 columns each
-    if (L < 4) L = 4;
-    return {L, (d.nr + L - 1) / L};
+    int per = places;
+    while (per > 4 && d.nr < 3 * per * sms) per = std::max(4, per / 2);
+    return {std::min(per * sms, d.nr), per < places ? per : 0};
 }
 
 template <class K>
 static void adj_launch(cudaStream_t st, K kernel, int nb, int t, size_t sm, const InstDev& d, const CoLevel& lin,
-                       const double2* gbar, const CoLevel& lout, int strip, void* wh, void* wi) {
+                       const double2* gbar, const CoLevel& lout, void* wh, void* wi) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -752,13 +756,14 @@ static void adj_launch(cudaStream_t st, K kernel, int nb, int t, size_t sm, cons
     cfg.stream = st;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, d, lin, gbar, lout, strip, wh, wi);
+    cudaLaunchKernelEx(&cfg, kernel, d, lin, gbar, lout, wh, wi);
 }
 
 void launch_adj_step(cudaStream_t st, const InstDev& d, const CoLevel& lin, const double2* gbar,
                      const CoLevel& lout, const AdjCut& cut, void* wh, void* wi) {
     adj_dispatch(d.prec, d.pitch, [&](auto kernel, size_t sm) {
-        adj_launch(st, kernel, cut.nb, d.pitch, sm, d, lin, gbar, lout, cut.strip, wh, wi);
+        if (cut.cap > 0) sm = capped_smem(cut.cap, sm);
+        adj_launch(st, kernel, cut.nb, d.pitch, sm, d, lin, gbar, lout, wh, wi);
     });
 }
 

@@ -425,6 +425,22 @@ teuk_status coef_tables(teuk_ctx* c, Instance& I) {
     return TEUK_OK;
 }
 
+// The 1D tables of an FP32 instance: the forward step's (at creation) or the adjoint's (on
+// its first call).
+teuk_status tables_1d(teuk_ctx* c, Instance& I, bool forward) {
+    RTab2*& rt = forward ? I.rtab : I.rtab_a;
+    ThTab*& tt = forward ? I.thtab : I.thtab_a;
+    if (rt && tt) return TEUK_OK;
+    const teuk_params& q = I.p;
+    if (!rt) TK_CUDA(c, dmalloc(c, (void**)&rt, sizeof(RTab2) * q.n_rstar, c->stream));
+    if (!tt) TK_CUDA(c, dmalloc(c, (void**)&tt, sizeof(ThTab) * q.n_theta, c->stream));
+    launch_tables_1d(c->stream, q.M, q.a, q.s, q.m, I.drs, I.dth, I.dt, q.n_rstar, q.n_theta, I.x_int, I.x_half, rt,
+                     tt, forward);
+    c->launches++;
+    TK_CUDA(c, cudaGetLastError());
+    return TEUK_OK;
+}
+
 // The cut of per-step launches with strip length `strip`: the partition built for it, or
 // uniform strips.
 StepCut cut_of(const teuk_ctx* c, const Instance& I, int strip) {
@@ -652,15 +668,8 @@ extern "C" teuk_status teuk_create(const teuk_params* p, int n_instances, void* 
             const teuk_status e = coef_tables(c, I);
             if (e != TEUK_OK) return fail(e);
         } else {
-            for (int adj = 0; adj < 2; ++adj) {
-                RTab2*& rt = adj ? I.rtab_a : I.rtab;
-                ThTab*& tt = adj ? I.thtab_a : I.thtab;
-                TK_CCUDA(dmalloc(c, (void**)&rt, sizeof(RTab2) * q.n_rstar, c->stream));
-                TK_CCUDA(dmalloc(c, (void**)&tt, sizeof(ThTab) * q.n_theta, c->stream));
-                launch_tables_1d(c->stream, q.M, q.a, q.s, q.m, I.drs, I.dth, I.dt, q.n_rstar, q.n_theta,
-                                 I.x_int, I.x_half, rt, tt, adj == 0);
-                c->launches++;
-            }
+            const teuk_status e = tables_1d(c, I, true);
+            if (e != TEUK_OK) return fail(e);
         }
         TK_CCUDA(cudaGetLastError());
         I.r_ext = 0;  // filled lazily from x at r*_ext when needed (adjoint loss)
@@ -2106,10 +2115,9 @@ extern "C" teuk_status teuk_adjoint_n(teuk_ctx* c, int instance, int64_t step0, 
                 (long long)I.step, (long long)step0);
     cudaStream_t s = c->stream;
     const int nth = I.p.n_theta;
-    if (I.p.prec == TEUK_FP64 || I.p.prec == TEUK_FP64_DF) {   // (FP32 instances form theirs)
-        st = coef_tables(c, I);
-        if (st) return st;
-    }
+    // (FP32 instances form their coefficients from the 1D tables)
+    st = I.p.prec == TEUK_FP64 || I.p.prec == TEUK_FP64_DF ? coef_tables(c, I) : tables_1d(c, I, false);
+    if (st) return st;
     // co-state planes ([nr][pitch] complex): FP64 for FP64 instances, else FP32 with
     // compensation planes for lam
     const bool co32 = I.p.prec == TEUK_FP32 || I.p.prec == TEUK_FP32_KAHAN;

@@ -233,6 +233,8 @@ struct StepCut {
     int strip = 1, nb = 0, cap = 0, room = 0;
 };
 constexpr int kMinCap = 3;   // the smallest cap
+// Dynamic shared memory (at least `own`) with which an SM holds cap blocks and no more
+size_t capped_smem(int cap, size_t own);
 void launch_step(cudaStream_t st, const InstDev& d, int64_t step, int bin, const StepCut& cut);
 void launch_extract(cudaStream_t st, const InstDev& d, int64_t step, int bin);
 // *base += k (one thread): closes a replayed graph of k per-step launches
@@ -264,11 +266,11 @@ void launch_wave_sum(cudaStream_t st, const double2* wave, int64_t cap, int nth,
 struct CoLevel { void* F; void* P; void* Fc; void* Pc; };
 // lam = E^T gbar: the co-state that starts the reverse sweep
 void launch_adj_init(cudaStream_t st, const InstDev& d, const double2* gbar, const CoLevel& out);
-// the fused reverse step (lam^n from lam^{n+1}), cut as adj_step_plan says (uniform strips
-// of `strip` columns, or, strip 0, nb pieces of equal length to a column); wh, wi (null without a source): the step's ring slot of the window
+// the fused reverse step (lam^n from lam^{n+1}), cut as adj_step_plan says: nb pieces of
+// equal length to a column, at most cap blocks on an SM (0: no cap); wh, wi (null without a source): the step's ring slot of the window
 // co-states, mu_Pi at the half-node window ([nj][nh]) and lam'_Pi at the integer-node
 // window ([nj][ni]), complex in the co-state's type
-struct AdjCut { int strip, nb; };
+struct AdjCut { int nb, cap; };
 AdjCut adj_step_plan(const InstDev& d);
 void launch_adj_step(cudaStream_t st, const InstDev& d, const CoLevel& lin, const double2* gbar,
                      const CoLevel& lout, const AdjCut& cut, void* wh, void* wi);

@@ -136,11 +136,14 @@ struct ColumnRing {
     __device__ __forceinline__ Planes<P> planes(int s) const { return Planes<P>::at(slot(s), stride); }
     // One thread: copy column col of buffer bin (and its radial tables) into slot s, and
     // prefetch the column's slices of the source profile into L2 (read once per step,
-    // they would otherwise come from DRAM, evicted by the state streaming through L2).
+    // they would otherwise come from DRAM, evicted by the state streaming through L2); kSrc
+    // false: the block meets no source (this thread's instructions are on every column's path:
+    // FP32-Kahan 8192 x 128 13.8 -> 13.6 us per step).
+    template <bool kSrc = true>
     __device__ __forceinline__ void fill(const InstDev& d, int bin, int col, int s) const {
         if (col == d.fault_col) return;   // testing aid: the slot's phase never completes
         if (!TK_IN(d.status, col, d.nr)) return;   // (checked builds; the waiters time out)
-        if (d.src.on) {
+        if (kSrc && d.src.on) {
             const SourceDev& w = d.src;
             const unsigned cb = (unsigned)w.q_stride * (unsigned)sizeof(typename V2T<typename P::T>::V);
             const int a = col - w.i_lo, h = col - w.h_lo;
@@ -569,7 +572,7 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
                 coefs(sp, c - 1, cfh, cfi);
                 const HalfRec<T> Rh = predict(u_prev, u_cur, dl_prev, dl, dlm_prev, dlm, cfh, s_h);
                 correct(Rh, L, u_prev, cfi, c - 1, xbuf + (c & 1) * xstride, o, s_i);
-                if (threadIdx.x == 0 && c - 2 + R <= c1) ring.fill(d, bin, c - 2 + R, sf);
+                if (threadIdx.x == 0 && c - 2 + R <= c1) ring.template fill<kSrc != 0>(d, bin, c - 2 + R, sf);
                 L = Rh;
                 u_prev = u_cur;
                 dl_prev = dl;
@@ -603,9 +606,9 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
     return true;
 }
 
-// Three register budgets: columns of up to 256 rows (the common case, P::blocks256
-// blocks per SM), of up to 512 rows (one block per SM, 128 registers a thread) and of up
-// to 1024 rows.  Dynamic shared memory:
+// Four register budgets: columns of up to 256 rows (the common case, P::blocks256
+// blocks per SM), of up to 320 rows (FP32 paths, two blocks per SM, 96 registers), of
+// up to 512 rows (one block per SM, 128 registers a thread) and of up to 1024 rows.  Dynamic shared memory:
 // StepShared<P, R>::bytes(blockDim.x).
 // part (may be null): the block's columns are [part[b], part[b+1]), of `strip` pieces, instead
 // of uniform strips of `strip` columns; it is written by the host before the launch sequence
@@ -647,6 +650,19 @@ template <class P, bool kMov>
 __global__ void __launch_bounds__(256, P::blocks256) step_kernel_s(InstDev d, int64_t step, int bin, int strip,
                                                                   const int* part) {
     step_body<P, kRingS, kMov>(d, step, bin, strip, part);
+}
+
+// FP32 paths, columns of 257 to 320 rows: with 96 registers a thread
+// two blocks per SM, 20 warps, where the 512-row build holds one, 10 warps.
+// us per step, 3001 x 300: FP32 12.6 -> 10.6, FP32-Kahan 15.6 -> 13.2; 8192 x 288: 30.5 -> 23.9, 38.7 ->
+// 30.8.  (FP64 3001 x 300 147.8 -> 145.3 but 1000 x 270 53.9 -> 55.5; double-float spills.)
+constexpr int kWideRows = 320;
+template <class P>
+__host__ __device__ constexpr bool has_wide() { return split_angular<P>(); }
+template <class P, bool kMov>
+__global__ void __launch_bounds__(kWideRows, 2) step_kernel_w(InstDev d, int64_t step, int bin, int strip,
+                                                             const int* part) {
+    if constexpr (has_wide<P>()) step_body<P, kRingS, kMov>(d, step, bin, strip, part);
 }
 
 template <class P, bool kMov>
@@ -870,8 +886,7 @@ void launch_batched_extract(cudaStream_t st, int prec, const BatchDev& b, int ma
     else batched_extract_kernel<PK><<<g, 128, 0, st>>>(b);
 }
 
-// Dynamic shared memory (at least `own`) with which an SM holds cap blocks and no more.
-static size_t capped_smem(int cap, size_t own) {
+size_t capped_smem(int cap, size_t own) {
     int dev = 0, sm = 0, res = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
@@ -905,6 +920,9 @@ static void launch_step_m(cudaStream_t st, const InstDev& d, int64_t step, int b
         cfg.dynamicSmemBytes = StepShared<P, kRingS>::bytes(threads);
         if (cut.cap > 0) cfg.dynamicSmemBytes = capped_smem(cut.cap, cfg.dynamicSmemBytes);
         cudaLaunchKernelEx(&cfg, step_kernel_s<P, kMov>, d, step, bin, strip, part);
+    } else if (threads <= kWideRows && has_wide<P>()) {
+        cfg.dynamicSmemBytes = StepShared<P, kRingS>::bytes(threads);
+        cudaLaunchKernelEx(&cfg, step_kernel_w<P, kMov>, d, step, bin, strip, part);
     } else if (threads <= 512) {
         cfg.dynamicSmemBytes = StepShared<P, kRingS>::bytes(threads);
         cudaLaunchKernelEx(&cfg, step_kernel_m<P, kMov>, d, step, bin, strip, part);
@@ -926,6 +944,9 @@ static int resident_p(int threads) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (threads <= 256)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel_s<P, false>, threads,
+                                                      StepShared<P, kRingS>::bytes(threads));
+    else if (threads <= kWideRows && has_wide<P>())
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel_w<P, false>, threads,
                                                       StepShared<P, kRingS>::bytes(threads));
     else if (threads <= 512)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel_m<P, false>, threads,
@@ -960,6 +981,8 @@ static cudaError_t prepare_m() {
               l = (int)StepShared<P, kRingL>::bytes(1024);
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(step_kernel_s<P, kMov>, a, s);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(step_kernel_w<P, kMov>, a, (int)StepShared<P, kRingS>::bytes(kWideRows));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(step_kernel_m<P, kMov>, a, m);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(step_kernel_l<P, kMov>, a, l);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(batched_step_kernel<P, 256, P::blocks256, kRingS, kMov>, a, s);
