@@ -47,25 +47,6 @@ template <typename R> struct R2T;
 template <> struct R2T<double> { using V = double2; };
 template <> struct R2T<float> { using V = float2; };
 
-// One co-state plane (complex, [nr][pitch]) and, for FP32, its compensation plane.
-template <typename R>
-struct CoPlane {
-    typename R2T<R>::V* v;
-    float2* c;   // FP32 only: value = v - c
-    __device__ __forceinline__ Z<R> ld(size_t o) const {
-        const typename R2T<R>::V a = v[o];
-        if constexpr (sizeof(R) == 4) {
-            const float2 b = c[o];
-            return {a.x - b.x, a.y - b.y};
-        } else {
-            return {a.x, a.y};
-        }
-    }
-};
-template <typename R>
-__device__ __forceinline__ CoPlane<R> coplane(const CoLevel& L, int k) {
-    return {(typename R2T<R>::V*)(k == 0 ? L.F : L.P), (float2*)(k == 0 ? L.Fc : L.Pc)};
-}
 template <typename R>
 __device__ __forceinline__ Z<R> ldv(const void* p, size_t o) {
     const typename R2T<R>::V a = ((const typename R2T<R>::V*)p)[o];
@@ -99,16 +80,6 @@ __device__ __forceinline__ double adj_coef(const void* tab, int pitch, int i, in
     return as64(((const T*)tab)[coef_index(pitch, i, j, k)]);
 }
 
-// Compensated add of an increment to one co-state node (FP32): value = v - c.
-__device__ __forceinline__ void kahan_node(float2& v, float2& c, Z<float> dlt) {
-    float yx = __fsub_rn(dlt.x, c.x), yy = __fsub_rn(dlt.y, c.y);
-    float tx = __fadd_rn(v.x, yx), ty = __fadd_rn(v.y, yy);
-    c.x = __fsub_rn(__fsub_rn(tx, v.x), yx);
-    c.y = __fsub_rn(__fsub_rn(ty, v.y), yy);
-    v.x = tx;
-    v.y = ty;
-}
-
 // lam = E^T gbar (the start of the reverse sweep).
 template <typename R>
 __global__ void adj_init_kernel(InstDev d, const double2* gbar, CoLevel out) {
@@ -119,11 +90,12 @@ __global__ void adj_init_kernel(InstDev d, const double2* gbar, CoLevel out) {
     Z<double> a = {0, 0};
     if (gbar && i == d.i_e) a = zscale(1.0 - d.f_e, gld<double>(gbar, j));
     if (gbar && i == d.i_e + 1) a = zscale(d.f_e, gld<double>(gbar, j));
-    stv<R>(out.F, o, Z<R>{(R)a.x, (R)a.y});
-    stv<R>(out.P, o, Z<R>{0, 0});
     if constexpr (sizeof(R) == 4) {
-        ((float2*)out.Fc)[o] = make_float2(0.f, 0.f);
-        ((float2*)out.Pc)[o] = make_float2(0.f, 0.f);
+        ((float4*)out.F)[o] = make_float4((float)a.x, (float)a.y, 0.f, 0.f);
+        ((float4*)out.Fc)[o] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+        stv<R>(out.F, o, Z<R>{(R)a.x, (R)a.y});
+        stv<R>(out.P, o, Z<R>{0, 0});
     }
 }
 
@@ -169,28 +141,8 @@ __device__ __forceinline__ Z<double> theta_cot(const AdjLin& A, Z<double> b, con
     return A.mac(b, hi ? adj_coef<T>(tab, pitch, i, j + 1, C_EM) : flip_sign(c[C_EP], flip), hi ? lp : l);
 }
 
-// The co-state of one node as stored: FP64 value, or FP32 (v, c) pairs with value v - c.
-template <typename R>
-struct CoNode {
-    Z<R> F, P;          // values
-    float2 vF, cF, vP, cP;   // FP32: the stored pairs
-};
-template <typename R>
-__device__ __forceinline__ CoNode<R> co_load(const CoLevel& L, size_t o) {
-    CoNode<R> n{};
-    if constexpr (sizeof(R) == 4) {
-        n.vF = ((const float2*)L.F)[o];
-        n.cF = ((const float2*)L.Fc)[o];
-        n.vP = ((const float2*)L.P)[o];
-        n.cP = ((const float2*)L.Pc)[o];
-        n.F = {n.vF.x - n.cF.x, n.vF.y - n.cF.y};
-        n.P = {n.vP.x - n.cP.x, n.vP.y - n.cP.y};
-    } else {
-        n.F = ldv<R>(L.F, o);
-        n.P = ldv<R>(L.P, o);
-    }
-    return n;
-}
+// The FP64 co-state of one node.
+struct CoNode { Z<double> F, P; };
 
 // Source gradients of step n.  With e = e^{-i phi} the phase of a sub-step and
 // de = d e / d r0,
@@ -263,7 +215,7 @@ __global__ void __launch_bounds__(kSrcGradThreads) adj_src_grad_kernel(InstDev d
     if (t != 0) return;
     const double A = (s.amps != nullptr && n < s.n_amps) ? s.amps[n] : 1.0;
     auto re_mul = [](Z<double> a, double bx, double by) { return a.x * bx - a.y * by; };
-    const double hd = sizeof(R) == 8 ? d.dt : 0.5 * d.dt;   // (FP64: the window holds mu_Pi / 2)
+    const double hd = d.dt;   // (the window holds the cotangent of 2 h_Pi)
     gA[k] = hd * re_mul(ph[0], S[0], S[1]) + d.dt * re_mul(ph[1], S[4], S[5]);
     gR[k] = A * (hd * (re_mul(ph[2], S[0], S[1]) + re_mul(ph[0], S[2], S[3])) +
                  d.dt * (re_mul(ph[3], S[4], S[5]) + re_mul(ph[1], S[6], S[7])));
@@ -291,7 +243,7 @@ __device__ __forceinline__ void adj_wait_prev() { asm volatile("griddepcontrol.w
 //     lam_Phi += cs +- cd, lam_Pi += csP +- cdP  at the nodes right (+) and left (-) of h
 // 76 FP64 operations a node instead of 190 (4096 x 128: 195 -> 89 us a reverse step, double-float
 // instances 360 -> 161).  mu here is the cotangent of
-// 2 h (adj_src_grad_kernel doubles it).
+// 2 h (adj_src_grad_kernel has the factor).
 template <typename T, int kMaxT>
 __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin, const double2* gbar,
                                                          CoLevel lout, void* wh, void* wi) {
@@ -312,8 +264,11 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
     // wh, wi: this step's ring slot of the window co-states (null: no source)
     // lam' = P lam^{n+1} at column col (zero at the boundary columns and outside)
     auto lam_at = [&](int col) {
-        CoNode<double> z{};
-        if (row_ok && col >= 1 && col <= nr - 2) z = co_load<double>(lin, node_index(d, col, j));
+        CoNode z{};
+        if (row_ok && col >= 1 && col <= nr - 2) {
+            const size_t o = node_index(d, col, j);
+            z = CoNode{ldv<double>(lin.F, o), ldv<double>(lin.P, o)};
+        }
         return z;
     };
     auto nb3 = [&](const Zd* buf, int sl, Zd& lm, Zd& lp) {
@@ -323,7 +278,7 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
     };
     // shares of node col (co-state L, its Pi part exchanged) of the half nodes to its right
     // (rF, rP) and left (lF, lP)
-    auto node_shares = [&](const CoNode<double>& L, int col, Zd& rF, Zd& rP, Zd& lF, Zd& lP) {
+    auto node_shares = [&](const CoNode& L, int col, Zd& rF, Zd& rP, Zd& lF, Zd& lP) {
         rF = rP = lF = lP = zero;
         if (!row_ok || col < 1 || col > nr - 2) return;
         double c[kNCoef];
@@ -341,7 +296,7 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
     };
     adj_wait_prev();
     // prologue: column c0 - 1
-    CoNode<double> l_cur = lam_at(c0 - 1), l_next;
+    CoNode l_cur = lam_at(c0 - 1), l_next;
     LB[(size_t)((c0 - 1) & 1) * pitch + j] = l_cur.P;
     __syncthreads();
     Zd muF_part, muP_part, aF_part = zero, aP_part = zero, x, y;
@@ -418,137 +373,98 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
     }
 }
 
-// The FP32 co-state (FP32 and FP32-Kahan instances): the same reverse step with the
-// coefficients formed in registers from the 1D tables (form_coefs2, the split angular
-// form turned back into ep = A + B, em = A - B), i.e. the coefficients the forward FP32
-// kernels compute, instead of 2D tables: the reverse step is then the transpose of the
-// forward operator as it is evaluated, and it reads no coefficient tables.  Each column's
-// coefficients are formed once per step and used at once for both nodes they enter: the
-// corrector coefficients of column c enter mu(c-1) (as its right node) and mu(c) (as its
-// left node), those of half node c enter lam(c) and lam(c+1); the partial sums are
-// carried to the next column, so every sum is formed in the order of the gather form
-// (left neighbour first).
+// The FP32 co-state (FP32 and FP32-Kahan instances): the same shares as in the FP64 kernel,
+// with the coefficients formed in registers from 1D tables (form_coefs2; the adjoint's own
+// tables carry the powers of two, ep = A + B and em = A - B turn the split angular form back),
+// i.e. the coefficients that the forward FP32 kernels compute, and the co-state compensated
+// like the forward state (value v - c, two planes of {Phi, Pi}).  Bound by instruction issue:
+// each column's coefficients are formed once and each node's and half node's shares once, the
+// rows exchange the products ep l and em l instead of l and their coefficients, and complex
+// sums run in paired instructions.  4096 x 128: 13.7 -> 10.0 us a reverse step; 400 instructions a
+// node instead of 588.
 struct CfF { float g, e1r, e1i, e2r, e2i, ep, em, e3r, e3i; };
-
-__device__ __forceinline__ Z<float> theta_cot_v(const CfF& c, float ep_m, float em_p, Z<float> lm,
-                                                Z<float> l0, Z<float> lp, int j, int nth, float g) {
-    Z<float> r = zconjmul(c.e3r - c.ep - c.em, c.e3i, l0);
-    if (j >= 1) r = zadd(r, zscale(ep_m, lm));
-    else r = zadd(r, zscale(g * c.em, l0));
-    if (j + 1 < nth) r = zadd(r, zscale(em_p, lp));
-    else r = zadd(r, zscale(g * c.ep, l0));
-    return r;
-}
 
 // columns of radial tables the FP32 reverse step stages in shared memory (pieces of up
 // to kAdjRtCols - 2 columns; longer ones read the tables from global memory)
 constexpr int kAdjRtCols = 64;
 
+__device__ __forceinline__ Cx<float> conj_mac(Cx<float> b, float cr, float ci, Cx<float> a) {
+    return {__fmaf_rn(cr, a.re, __fmaf_rn(ci, a.im, b.re)), __fmaf_rn(cr, a.im, __fmaf_rn(-ci, a.re, b.im))};
+}
+
 template <int kMaxT>
 __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel lin, const double2* gbar,
                                                              CoLevel lout, void* wh, void* wi) {
-    using R = float;
+    using C = Cx<float>;
     extern __shared__ __align__(16) unsigned char adj_smem[];
     adj_release_next();
     const int j = threadIdx.x, nth = d.nth, nr = d.nr, pitch = d.pitch;
-    Z<R>* LB = (Z<R>*)adj_smem;                   // [2][pitch] lam'_Pi of a column
-    Z<R>* MB = LB + 2 * (size_t)pitch;            // [2][pitch] mu_Pi of a half node
-    float4* EB = (float4*)(MB + 2 * (size_t)pitch);   // [3][pitch] {ep, em} of node, half node
-    RTab2* RT = (RTab2*)(EB + 3 * (size_t)pitch);      // radial tables of columns c0-1 .. c1
-    const bool row_ok = j < nth;
+    float4* LB = (float4*)adj_smem;                 // [2][pitch] {ep l, em l} of a column, l = lam'_Pi
+    float4* MB = LB + 2 * (size_t)pitch;            // [2][pitch] the same of a half node, l = mu_Pi
+    RTab2* RT = (RTab2*)(MB + 2 * (size_t)pitch);   // radial tables of columns c0-1 .. c1
+    const bool row_ok = j < nth, lo_ok = j >= 1, hi_ok = j + 1 < nth;
     // output columns [c0, c1): one of gridDim.x pieces of equal length to a column
     const int c0 = (int)((int64_t)blockIdx.x * nr / gridDim.x), c1 = (int)((int64_t)(blockIdx.x + 1) * nr / gridDim.x);
-    const bool rt_smem = c1 - c0 + 2 <= kAdjRtCols;   // else the tables are read from global
-    const R g = d.ghost_f, hdt = d.hdt2.x, qdt = d.hdt2.x;
+    const bool rt_smem = c1 - c0 + 2 <= kAdjRtCols;
+    const float hdt = d.hdt2.x, qdt = d.qdt2.x;
+    const int flip = pole_flip(d);
     const SourceDev& s = d.src;
+    const C zero = C::zero();
     // wh, wi: this step's ring slot of the window co-states (null: no source)
     RowTab<PK> rt;
     rt.load(d.thtab_a, j, row_ok);
-    auto lam_at = [&](int col) {
-        CoNode<R> z{};
-        if (row_ok && col >= 1 && col <= nr - 2) z = co_load<R>(lin, node_index(d, col, j));
-        return z;
-    };
-    // the stored pairs of a column, loaded one column ahead of use (zero outside the
-    // interior columns, as lam_at); as_node forms the values when the column is used
-    struct CoRaw { float2 vF, cF, vP, cP; };
-    auto raw_at = [&](int col) {
-        CoRaw z{};
+    // a column as stored, loaded one column ahead of use (zero off the interior columns)
+    struct Node { C vF, vP, cF, cP; };
+    auto load = [&](int col) {
+        Node n{zero, zero, zero, zero};
         if (row_ok && col >= 1 && col <= nr - 2) {
             const size_t o = node_index(d, col, j);
-            z.vF = __ldg((const float2*)lin.F + o);
-            z.cF = __ldg((const float2*)lin.Fc + o);
-            z.vP = __ldg((const float2*)lin.P + o);
-            z.cP = __ldg((const float2*)lin.Pc + o);
+            const float4 v = __ldg((const float4*)lin.F + o), c = __ldg((const float4*)lin.Fc + o);
+            n = Node{{v.x, v.y}, {v.z, v.w}, {c.x, c.y}, {c.z, c.w}};
         }
-        return z;
-    };
-    auto as_node = [](const CoRaw& r) {
-        CoNode<R> n;
-        n.vF = r.vF;
-        n.cF = r.cF;
-        n.vP = r.vP;
-        n.cP = r.cP;
-        n.F = {r.vF.x - r.cF.x, r.vF.y - r.cF.y};
-        n.P = {r.vP.x - r.cP.x, r.vP.y - r.cP.y};
         return n;
     };
     // coefficients of column col: node col (ci) and half node col+1/2 (ch)
     auto form = [&](int col, CfF& ci, CfF& ch) {
-        float2 cf2[kNCoef];
+        float2 cf[kNCoef];
         if (col >= 0 && col <= nr - 1) {
-            form_coefs2(rt_smem ? RT[col - (c0 - 1)] : d.rtab_a[col], rt.t, cf2);
+            form_coefs2(rt_smem ? RT[col - (c0 - 1)] : d.rtab_a[col], rt.t, cf);
         } else {
 #pragma unroll
-            for (int q = 0; q < kNCoef; ++q) cf2[q] = make_float2(0.f, 0.f);
+            for (int q = 0; q < kNCoef; ++q) cf[q] = make_float2(0.f, 0.f);
         }
-        auto pick = [&](bool half) {
-            auto v = [&](int q) { return half ? cf2[q].x : cf2[q].y; };
-            return CfF{v(C_G), v(C_E1R), v(C_E1I), v(C_E2R), v(C_E2I), __fadd_rn(v(C_EP), v(C_EM)),
-                       __fsub_rn(v(C_EP), v(C_EM)), v(C_E3R), v(C_E3I)};
-        };
-        ci = pick(false);
-        ch = pick(true);
+        const float2 ep = __fadd2_rn(cf[C_EP], cf[C_EM]), em = p_sub(cf[C_EP], cf[C_EM]);
+        ch = CfF{cf[C_G].x, cf[C_E1R].x, cf[C_E1I].x, cf[C_E2R].x, cf[C_E2I].x, ep.x, em.x, cf[C_E3R].x, cf[C_E3I].x};
+        ci = CfF{cf[C_G].y, cf[C_E1R].y, cf[C_E1I].y, cf[C_E2R].y, cf[C_E2I].y, ep.y, em.y, cf[C_E3R].y, cf[C_E3I].y};
     };
-    auto nb3 = [&](const Z<R>* buf, int sl, Z<R>& lm, Z<R>& lp) {
-        const Z<R>* b = buf + (size_t)sl * pitch;
-        lm = j >= 1 ? b[j - 1] : Z<R>{0, 0};
-        lp = j + 1 < nth ? b[j + 1] : Z<R>{0, 0};
+    // this row's products ep l and em l, published for the rows above and below
+    auto publish = [&](float4* x, const CfF& c, C l) {
+        const float4 p = make_float4(c.ep * l.re, c.ep * l.im, c.em * l.re, c.em * l.im);
+        x[j] = p;
+        return p;
     };
-    // corrector contribution of node col (coefficients c, co-state L) to a half node on
-    // its right (sR = +1) or left (sR = -1)
-    auto e3 = [](int col) { return (col + 3) % 3; };   // EB slot of column col >= -1
-    auto corr = [&](const CfF& c, const CoNode<R>& L, int col, R sR, Z<R>& muF, Z<R>& muP) {
-        const int sl = col & 1;
-        Z<R> lm, lp;
-        nb3(LB, sl, lm, lp);
-        const float4 em = EB[(size_t)e3(col) * pitch + (j >= 1 ? j - 1 : j)];   // row j-1
-        const float4 ep = EB[(size_t)e3(col) * pitch + (j + 1 < nth ? j + 1 : j)];   // row j+1
-        const Z<R> tc = theta_cot_v(c, em.x, ep.y, lm, L.P, lp, j, nth, g);
-        muF = zadd(muF, zscale(-sR * c.g, L.F));
-        muF = zadd(muF, zscale(sR, zconjmul(c.e2r, c.e2i, L.P)));
-        muF = zadd(muF, zscale(R(0.5), tc));
-        muP = zadd(muP, zscale(hdt, L.F));
-        muP = zadd(muP, zscale(sR * c.g, L.P));
-        muP = zadd(muP, zscale(R(0.5), zconjmul(c.e1r, c.e1i, L.P)));
+    // b + Th^T l from this row's products p and the neighbours' in x, as differences: a product
+    // enters its own row and its neighbour's with opposite signs and the same rounding
+    auto theta = [&](C b, const CfF& c, const float4* x, float4 p, C l) {
+        const C ep = {p.x, p.y}, em = {p.z, p.w};
+        C lo = flip_sign(em, flip), hi = flip_sign(ep, flip);
+        if (lo_ok) lo = up(*(const float2*)(x + j - 1));
+        if (hi_ok) hi = up(*((const float2*)(x + j + 1) + 1));
+        return conj_mac(b, c.e3r, c.e3i, l) + ((lo - ep) + (hi - em));
     };
-    // predictor contribution of half node hh (coefficients c, cotangent MF, MP) to the node
-    // on its right (sR = +1) or left (sR = -1)
-    auto pred = [&](const CfF& c, Z<R> MF, Z<R> MP, int hh, R sR, Z<R>& aF, Z<R>& aP) {
-        const int sl = hh & 1;
-        Z<R> mm, mp;
-        nb3(MB, sl, mm, mp);
-        const float4 em = EB[(size_t)e3(hh) * pitch + (j >= 1 ? j - 1 : j)];   // row j-1
-        const float4 ep = EB[(size_t)e3(hh) * pitch + (j + 1 < nth ? j + 1 : j)];   // row j+1
-        const Z<R> tc = theta_cot_v(c, em.z, ep.w, mm, MP, mp, j, nth, g);
-        aF = zadd(aF, zscale(R(0.5) - sR * c.g, MF));
-        aF = zadd(aF, zscale(sR, zconjmul(c.e2r, c.e2i, MP)));
-        aF = zadd(aF, zscale(R(0.5), tc));
-        aP = zadd(aP, zscale(R(0.5) * qdt, MF));
-        aP = zadd(aP, zscale(R(0.5) + sR * c.g, MP));
-        aP = zadd(aP, zscale(R(0.5), zconjmul(c.e1r, c.e1i, MP)));
+    // shares of node col (co-state lF, lP) of the half nodes to its right (rF, rP) and left (xF, xP)
+    auto node_shares = [&](const CfF& c, const float4* x, float4 p, C lF, C lP, int col, C& rF, C& rP, C& xF, C& xP) {
+        rF = rP = xF = xP = zero;
+        if (!row_ok || col < 1 || col > nr - 2) return;
+        const C cS = theta(zero, c, x, p, lP);
+        const C cD = conj_mac(rmac(zero, -c.g, lF), c.e2r, c.e2i, lP);
+        const C cSP = conj_mac(rmac(zero, qdt, lF), c.e1r, c.e1i, lP);
+        rF = cS + cD;
+        xF = cS - cD;
+        rP = rmac(cSP, c.g, lP);
+        xP = rmac(cSP, -c.g, lP);
     };
-    // the strip's radial tables into shared memory (one broadcast read per column later)
+    // the piece's radial tables into shared memory (one broadcast read per column later)
     if (rt_smem) {
         const int ncols = c1 - c0 + 2;
         for (int q = threadIdx.x; q < ncols * 8; q += blockDim.x) {
@@ -558,82 +474,84 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel 
         __syncthreads();
     }
     adj_wait_prev();
+    // the record's cotangent and the extraction weights, once (column -2: no record)
+    const int ie = gbar ? d.i_e : -2;
+    float we = 0.f, we1 = 0.f;
+    C gb = zero;
+    if (gbar && row_ok && c0 <= ie + 1 && ie < c1) {
+        const Z<float> g = gld<float>(gbar, j);
+        gb = {g.x, g.y};
+        we = (float)(1.0 - d.f_e);
+        we1 = (float)d.f_e;
+    }
     // prologue: column c0 - 1
-    CoNode<R> l_cur = lam_at(c0 - 1);
-    CfF ci_cur, ch_cur;
-    form(c0 - 1, ci_cur, ch_cur);
-    LB[(size_t)((c0 - 1) & 1) * pitch + j] = l_cur.P;
-    EB[(size_t)e3(c0 - 1) * pitch + j] = make_float4(ci_cur.ep, ci_cur.em, ch_cur.ep, ch_cur.em);
+    Node cur = load(c0 - 1), next = load(c0);
+    C lF = cur.vF - cur.cF, lP = cur.vP - cur.cP;
+    CfF ci, ch_cur, ch_n;
+    form(c0 - 1, ci, ch_cur);
+    float4 p = publish(LB + (size_t)((c0 - 1) & 1) * pitch, ci, lP);
     __syncthreads();
-    Z<R> muF_part = {0, 0}, muP_part = {0, 0};      // mu(h): the left node's share
-    if (row_ok && c0 - 1 >= 1 && c0 - 1 <= nr - 2) corr(ci_cur, l_cur, c0 - 1, R(1), muF_part, muP_part);
-    Z<R> aF_part = {0, 0}, aP_part = {0, 0};        // lam(h): the left half node's share
-    CoRaw r_next = raw_at(c0);
+    C muF_part, muP_part, aF_part = zero, aP_part = zero, xF, xP;
+    node_shares(ci, LB + (size_t)((c0 - 1) & 1) * pitch, p, lF, lP, c0 - 1, muF_part, muP_part, xF, xP);
     for (int h = c0 - 1; h <= c1 - 1; ++h) {
-        // A: column h+1: its co-state (loaded one column ahead) and coefficients
-        const CoNode<R> l_next = as_node(r_next);
-        r_next = raw_at(h + 2);
-        CfF ci_n, ch_n;
-        form(h + 1, ci_n, ch_n);
-        LB[(size_t)((h + 1) & 1) * pitch + j] = l_next.P;
-        EB[(size_t)e3(h + 1) * pitch + j] = make_float4(ci_n.ep, ci_n.em, ch_n.ep, ch_n.em);
+        // column h+1: lam' and its shares; mu at half node h
+        const Node nx = next;
+        next = load(h + 2);
+        lF = nx.vF - nx.cF;
+        const C lP_n = nx.vP - nx.cP;
+        float4* lb = LB + (size_t)((h + 1) & 1) * pitch;
+        form(h + 1, ci, ch_n);
+        p = publish(lb, ci, lP_n);
         __syncthreads();
-        // C: mu(h) = its left node's share + the right node h+1; the left share of mu(h+1)
-        Z<R> muF = muF_part, muP = muP_part, mfn = {0, 0}, mpn = {0, 0};
-        const bool half_ok = h >= 0 && h <= nr - 2;
-        if (row_ok && h + 1 >= 1 && h + 1 <= nr - 2) {
-            if (half_ok) corr(ci_n, l_next, h + 1, R(-1), muF, muP);
-            if (h + 1 <= nr - 2) corr(ci_n, l_next, h + 1, R(1), mfn, mpn);
-        }
-        if (!half_ok || !row_ok) muF = muP = Z<R>{0, 0};
-        if (wh && half_ok && row_ok && h >= c0) {
+        C muF_next, muP_next;
+        node_shares(ci, lb, p, lF, lP_n, h + 1, muF_next, muP_next, xF, xP);
+        const bool half_ok = row_ok && h >= 0 && h <= nr - 2;
+        const C muF = half_ok ? muF_part + xF : zero, muP = half_ok ? muP_part + xP : zero;
+        if (wh && half_ok && h >= c0) {   // half-node window (half node c0 - 1 is the previous block's)
             const int a = h - s.h_lo, bb = j - s.j_lo;
             if ((unsigned)a < (unsigned)s.nh && (unsigned)bb < (unsigned)s.nj)
-                stv<R>(wh, (size_t)bb * s.nh + a, muP);
+                ((float2*)wh)[(size_t)bb * s.nh + a] = pk(muP);
         }
-        MB[(size_t)(h & 1) * pitch + j] = muP;
+        float4* mb = MB + (size_t)(h & 1) * pitch;
+        p = publish(mb, ch_cur, muP);
         __syncthreads();
-        // F: half node h's shares of lam(h) (completing it) and lam(h+1)
-        Z<R> aF = aF_part, aP = aP_part, afn = {0, 0}, apn = {0, 0};
-        if (row_ok && half_ok) {
-            pred(ch_cur, muF, muP, h, R(-1), aF, aP);
-            pred(ch_cur, muF, muP, h, R(1), afn, apn);
+        // the shares of half node h of the nodes h (left) and h+1 (right)
+        C tF = zero, tP = zero, nF = zero, nP = zero;
+        if (half_ok) {
+            const C cs = theta(muF, ch_cur, mb, p, muP);
+            const C cd = conj_mac(rmac(zero, -ch_cur.g, muF), ch_cur.e2r, ch_cur.e2i, muP);
+            const C csP = conj_mac(rmac(muP, hdt, muF), ch_cur.e1r, ch_cur.e1i, muP);
+            tF = cs - cd;
+            nF = cs + cd;
+            tP = rmac(csP, -ch_cur.g, muP);
+            nP = rmac(csP, ch_cur.g, muP);
         }
+        // lam^n at column h
         if (h >= c0 && row_ok) {
-            const int i = h;
-            const size_t o = node_index(d, i, j);
-            const bool interior = i >= 1 && i <= nr - 2;
-            if (gbar) {
-                if (i == d.i_e) aF = zadd(aF, zscale((R)(1.0 - d.f_e), gld<R>(gbar, j)));
-                if (i == d.i_e + 1) aF = zadd(aF, zscale((R)d.f_e, gld<R>(gbar, j)));
-            }
-            float2 vF = {0.f, 0.f}, cF = {0.f, 0.f}, vP = {0.f, 0.f}, cP = {0.f, 0.f};
-            if (interior) {
-                vF = l_cur.vF;
-                cF = l_cur.cF;
-                vP = l_cur.vP;
-                cP = l_cur.cP;
-            }
-            kahan_node(vF, cF, aF);
-            kahan_node(vP, cP, aP);
+            const size_t o = node_index(d, h, j);
+            C aF = aF_part + tF;
+            const C aP = aP_part + tP;
+            if (h == ie) aF = rmac(aF, we, gb);
+            if (h == ie + 1) aF = rmac(aF, we1, gb);
+            const C lam = cur.vP - cur.cP;   // (lam'_Pi, for the window)
+            kahan_add(cur.vF, cur.cF, aF);   // (a column off the interior was loaded as zero)
+            kahan_add(cur.vP, cur.cP, aP);
             if (TK_IN(d.status, o, plane_elems(d))) {
-                ((float2*)lout.F)[o] = vF;
-                ((float2*)lout.Fc)[o] = cF;
-                ((float2*)lout.P)[o] = vP;
-                ((float2*)lout.Pc)[o] = cP;
+                ((float4*)lout.F)[o] = make_float4(cur.vF.re, cur.vF.im, cur.vP.re, cur.vP.im);
+                ((float4*)lout.Fc)[o] = make_float4(cur.cF.re, cur.cF.im, cur.cP.re, cur.cP.im);
             }
-            if (wi) {
-                const int a = i - s.i_lo, bb = j - s.j_lo;
+            if (wi) {   // integer-node window: lam'_Pi (zero off the interior columns)
+                const int a = h - s.i_lo, bb = j - s.j_lo;
                 if ((unsigned)a < (unsigned)s.ni && (unsigned)bb < (unsigned)s.nj)
-                    stv<R>(wi, (size_t)bb * s.ni + a, interior ? l_cur.P : Z<R>{0, 0});
+                    ((float2*)wi)[(size_t)bb * s.ni + a] = pk(lam);
             }
         }
-        l_cur = l_next;
+        cur = nx;
         ch_cur = ch_n;
-        muF_part = mfn;
-        muP_part = mpn;
-        aF_part = afn;
-        aP_part = apn;
+        muF_part = muF_next;
+        muP_part = muP_next;
+        aF_part = nF;
+        aP_part = nP;
     }
 }
 
@@ -675,8 +593,7 @@ void launch_adj_init(cudaStream_t st, const InstDev& d, const double2* gbar, con
 // dynamic shared memory of the reverse-step kernels for blocks of `threads` rows
 template <typename R>
 static size_t adj_smem(int threads, bool f32) {
-    return 4 * (size_t)threads * sizeof(Z<R>) +
-           (f32 ? 3 * (size_t)threads * sizeof(float4) + kAdjRtCols * sizeof(RTab2) : 0);
+    return 4 * (size_t)threads * (f32 ? sizeof(float4) : sizeof(Z<R>)) + (f32 ? kAdjRtCols * sizeof(RTab2) : 0);
 }
 
 template <class K>
@@ -722,7 +639,7 @@ static void adj_dispatch(int prec, int t, F f) {
 // FP32 co-state: a piece for every place the GPU has, or, while a piece would have less than
 // three columns, half as many places (down to four an SM), capped.  us per step, one wave of
 // strips of at least four columns -> this: 512 x 32 6.1 -> 3.7, 1024 x 64 9.4 -> 5.2, 2048 x 128
-// 10.0 -> 9.7, 4096 x 64 9.8 -> 9.4, 4096 x 128 14.0.
+// 10.0 -> 9.7, 4096 x 64 9.8 -> 9.4, 4096 x 128 14.0 both (with the step then at 588 instructions a node).
 AdjCut adj_step_plan(const InstDev& d) {
     int res = 1, dev = 0, sms = 0;
     adj_dispatch(d.prec, d.pitch, [&](auto kernel, size_t sm) {

@@ -2121,16 +2121,12 @@ extern "C" teuk_status teuk_adjoint_n(teuk_ctx* c, int instance, int64_t step0, 
     // co-state planes ([nr][pitch] complex): FP64 for FP64 instances, else FP32 with
     // compensation planes for lam
     const bool co32 = I.p.prec == TEUK_FP32 || I.p.prec == TEUK_FP32_KAHAN;
-    const size_t plane = (size_t)I.p.n_rstar * I.pitch * (co32 ? sizeof(float2) : sizeof(double2));
+    const size_t plane = (size_t)I.p.n_rstar * I.pitch * 16;
     AdjBuffers B(c, s);
     CoLevel lam[2] = {};
     for (int b = 0; b < 2; ++b) {
         TK_CUDA(c, B.get(&lam[b].F, plane));
-        TK_CUDA(c, B.get(&lam[b].P, plane));
-        if (co32) {
-            TK_CUDA(c, B.get(&lam[b].Fc, plane));
-            TK_CUDA(c, B.get(&lam[b].Pc, plane));
-        }
+        TK_CUDA(c, B.get(co32 ? &lam[b].Fc : &lam[b].P, plane));
     }
     // the fused reverse step's strip; with a source, a ring of window co-states that
     // adj_src_grad_kernel turns into gradients every `slots` steps (32 MB at most)

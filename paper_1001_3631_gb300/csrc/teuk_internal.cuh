@@ -93,7 +93,9 @@ struct SourceDev {
 //   E3 = ((qr + nDs V) iS, qi iS)                      (qr, qi scaled by sdt; nDs = -Ds)
 // The forward step acts on undivided sums and the negated second difference (split form in
 // teuk_step_common.cuh): its tables hold nsdt, Ds, nDs, qr, qi times 1/2 (half node) and 1/4
-// (node) and i2 = -1/dth^2, all exactly; the adjoint's hold the values above.
+// (node) and i2 = -1/dth^2, all exactly.  The reverse step is the transpose of the step in
+// undivided half-node sums 2 h (predict_x): the adjoint's tables hold the same five times 1
+// and 1/4, the terms of radial differences (Rd, pr, pi, nbb) times 2 and 1/2, and i2 as above.
 struct RTab2 { float2 R2, naD, Rd, ctr, cti, ctc, pr, pi, nbb, Ds, nDs, qr, qi, nsdt, pad0, pad1; };
 // Per theta row: sin^2, cos, V = (m + s cos)^2/sin^2 - s, i2 = 1/dth^2, i1 = cot/(2 dth)
 struct ThTab { float sin2, cs, V, i2, i1, pad0, pad1, pad2; };
@@ -260,10 +262,10 @@ void launch_scan_finite(cudaStream_t st, const InstDev& d, int bin);
 void launch_wave_sum(cudaStream_t st, const double2* wave, int64_t cap, int nth, double dth,
                      int64_t level0, int64_t k_count, double2* out);
 // teuk_adjoint.cu
-// Co-state of one time level (teuk_adjoint.cu): F and P planes ([nr][pitch] complex,
-// double2 for FP64 instances, float2 otherwise) and, for FP32, their compensation
-// planes (float2; the value is v - c).
-struct CoLevel { void* F; void* P; void* Fc; void* Pc; };
+// Co-state of one time level (teuk_adjoint.cu), planes [nr][pitch]: FP64, F and P (double2,
+// Phi and Pi); FP32, F the values {Phi, Pi} (float4) and Fc their compensations (float4; the
+// co-state is the value minus the compensation).
+struct CoLevel { void* F; void* P; void* Fc; };
 // lam = E^T gbar: the co-state that starts the reverse sweep
 void launch_adj_init(cudaStream_t st, const InstDev& d, const double2* gbar, const CoLevel& out);
 // the fused reverse step (lam^n from lam^{n+1}), cut as adj_step_plan says: nb pieces of

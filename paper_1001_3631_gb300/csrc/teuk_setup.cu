@@ -318,25 +318,25 @@ __device__ float2 pair_f(double h, double i) { return make_float2((float)h, (flo
 
 __global__ void tables_1d_kernel(double M, double a, int s, int m, double drs, double dth,
                                  double dt, int nr, int nth, const double* x_int,
-                                 const double* x_half, RTab2* rtab, ThTab* thtab, double fh, double fi,
-                                 double fi2) {
+                                 const double* x_half, RTab2* rtab, ThTab* thtab, double fs, double fd, double fi2) {
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < nr) {
         // the half node nr-1/2 lies outside the grid: zeros
         const RadialVals h = k < nr - 1 ? radial_vals(M, a, s, m, x_half[k], drs, 0.5 * dt) : RadialVals{};
         const RadialVals i = radial_vals(M, a, s, m, x_int[k], drs, dt);
         RTab2 t;
-        // the terms that act on sums, times fh at the half node and fi at the node
-        auto pair_s = [&](double hv, double iv) { return pair_f(fh * hv, fi * iv); };
+        // the terms that act on sums and those on radial differences
+        auto pair_s = [&](double hv, double iv) { return pair_f(fs * hv, 0.25 * iv); };
+        auto pair_d = [&](double hv, double iv) { return pair_f(fd * hv, iv / fd); };
         t.R2 = pair_f(h.R2, i.R2);
         t.naD = pair_f(h.naD, i.naD);
-        t.Rd = pair_f(h.Rd, i.Rd);
+        t.Rd = pair_d(h.Rd, i.Rd);
         t.ctr = pair_f(h.ctr, i.ctr);
         t.cti = pair_f(h.cti, i.cti);
         t.ctc = pair_f(h.ctc, i.ctc);
-        t.pr = pair_f(h.pr, i.pr);
-        t.pi = pair_f(h.pi, i.pi);
-        t.nbb = pair_f(h.nbb, i.nbb);
+        t.pr = pair_d(h.pr, i.pr);
+        t.pi = pair_d(h.pi, i.pi);
+        t.nbb = pair_d(h.nbb, i.nbb);
         t.Ds = pair_s(h.Ds, i.Ds);
         t.nDs = pair_s(h.nDs, i.nDs);
         t.qr = pair_s(h.qr, i.qr);
@@ -364,11 +364,11 @@ void launch_tables_1d(cudaStream_t st, double M, double a, int s, int m, double 
                       double dt, int nr, int nth, const double* x_int, const double* x_half,
                       RTab2* rtab, ThTab* thtab, bool forward) {
     int n = nr > nth ? nr : nth;
-    // forward: of the undivided sums of two (half nodes) and four (nodes) values and the
-    // negated second difference (teuk_step_common.cuh)
-    const double fh = forward ? 0.5 : 1.0, fi = forward ? 0.25 : 1.0, fi2 = forward ? -1.0 : 1.0;
+    // powers of two of the undivided sums, and the forward step's negated second difference
+    // (see RTab2)
+    const double fs = forward ? 0.5 : 1.0, fd = forward ? 1.0 : 2.0, fi2 = forward ? -1.0 : 1.0;
     tables_1d_kernel<<<(n + 127) / 128, 128, 0, st>>>(M, a, s, m, drs, dth, dt, nr, nth, x_int,
-                                                      x_half, rtab, thtab, fh, fi, fi2);
+                                                      x_half, rtab, thtab, fs, fd, fi2);
 }
 
 void launch_invert_tortoise(cudaStream_t st, double M, double a, double rstar_min, double drs,
