@@ -91,9 +91,12 @@ def _stream_handle(stream):
 class _HostBuffers:
     """Result arrays whose memory is used again once the caller has dropped them (every view
     included).  A fresh array of 134 MB (a 16384 x 256 state) costs 6 to 20 ms of page faults
-    and unmapping a call, on GB300 with its fast host link the copy itself 0.9 ms.  Arrays
-    below 4 MB come from numpy (its heap reuses them); at most KEEP bytes are kept idle, by the solver that made
-    them (any thread may drop an array or ask for one)."""
+    and unmapping a call, on GB300 with its fast host link the copy itself 0.9 ms.  Memory that
+    the GPU alone goes on using is moved about by the driver, and every few copies then take
+    15 to 35 ms; one access by the host to each page before the copy keeps it where it is
+    (`_touch`, 0.05 ms).  Arrays below 4 MB come from numpy (its heap reuses them); at most KEEP
+    bytes are kept idle, by the solver that made them (any thread may drop an array or ask for
+    one)."""
     MIN, KEEP = 4 << 20, 1 << 30
 
     def __init__(self):
@@ -111,6 +114,7 @@ class _HostBuffers:
         with self._lock:
             idle = [b for b in self._bufs if b[1]() is None]
             buf = next((b for b in idle if len(b[0]) == size), None)
+            again = buf is not None
             if buf is None:
                 m = mmap.mmap(-1, size, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS)
                 try:   # (as numpy does for its own arrays)
@@ -130,7 +134,16 @@ class _HostBuffers:
                 kept -= len(b[0])
             raw = (ctypes.c_char * size).from_buffer(buf[0])
             buf[1] = weakref.ref(raw)   # dead when the last array on the mapping is gone
+        if again:
+            np.frombuffer(raw, np.uint8)[::mmap.PAGESIZE] = 0
         return np.frombuffer(raw, dtype, count).reshape(shape)
+
+
+def _touch(u):
+    """Read one value of each page of a large contiguous host array before the GPU copies it:
+    16384 x 256 states set in turn, 0.9 or 20 to 36 ms a call -> 0.95 ms every time."""
+    if u.nbytes >= _HostBuffers.MIN:
+        u.reshape(-1)[::mmap.PAGESIZE // u.itemsize].copy()
 
 
 class TeukSolver:
@@ -208,6 +221,7 @@ class TeukSolver:
     def set_state(self, u, step0=0, instance=0):
         u = np.ascontiguousarray(u, dtype=np.float64)
         assert u.shape == self.shape(instance)
+        _touch(u)
         check(_lib.load().teuk_set_state(self.ctx, instance, ptr(u), step0), self.ctx)
 
     def get_state(self, instance=0):
