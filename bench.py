@@ -33,7 +33,7 @@ WORKLOAD = "paper-scale single mode 16384x256 (s=-2, m=2, a=0.9, r*=[-200,800], 
 KAHAN_BYTES_PER_UPDATE = 64   # read + write of (hi, c) for Phi and Pi, FP32
 FP64_BYTES_PER_UPDATE = 64    # read + write of Phi and Pi, FP64 (and double-float)
 FP32_BYTES_PER_UPDATE = 32    # read + write of Phi and Pi, plain FP32
-FP64_FLOPS_PER_UPDATE = 156   # FP64 flops of one point update in the kernel's formulation (FMA = 2)
+FP64_FLOPS_PER_UPDATE = 112   # FP64 flops of one point update in the kernel's formulation (FMA = 2)
 FP64_PEAK_TFLOPS = 1.25       # GB300 FP64 (non-tensor) nominal: 152 SMs x 2 DFMA/clk x 2 x 2.07 GHz
 
 
@@ -352,7 +352,7 @@ def single_mode_leg(steps=2000):
     double-float path, FP32-Kahan and FP32.  hbm_frac is the algorithmic bytes per update
     against the measured HBM copy bandwidth (the grid is L2-resident, so this is the
     fraction of the HBM roofline, not a DRAM measurement); native FP64 is also stated
-    against its ALU ceiling (156 flops per update at the nominal FP64 rate)."""
+    against its ALU ceiling (112 flops per update at the nominal FP64 rate)."""
     import torch
 
     from paper_1001_3631_gb300 import TeukSolver, inputs
