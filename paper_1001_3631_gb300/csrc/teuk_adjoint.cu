@@ -413,13 +413,15 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel 
     // wh, wi: this step's ring slot of the window co-states (null: no source)
     RowTab<PK> rt;
     rt.load(d.thtab_a, j, row_ok);
-    // a column as stored, loaded one column ahead of use (zero off the interior columns)
+    // a column as stored, loaded one column ahead of use (zero off the interior columns); plain
+    // loads: the previous reverse step may still write these planes while this block is set up,
+    // so they are not read-only for the kernel's life and must stay behind adj_wait_prev
     struct Node { C vF, vP, cF, cP; };
     auto load = [&](int col) {
         Node n{zero, zero, zero, zero};
         if (row_ok && col >= 1 && col <= nr - 2) {
             const size_t o = node_index(d, col, j);
-            const float4 v = __ldg((const float4*)lin.F + o), c = __ldg((const float4*)lin.Fc + o);
+            const float4 v = ((const float4*)lin.F)[o], c = ((const float4*)lin.Fc)[o];
             n = Node{{v.x, v.y}, {v.z, v.w}, {c.x, c.y}, {c.z, c.w}};
         }
         return n;
