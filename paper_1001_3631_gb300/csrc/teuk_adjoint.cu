@@ -56,9 +56,11 @@ template <typename R>
 __device__ __forceinline__ void stv(void* p, size_t o, Z<R> z) {
     ((typename R2T<R>::V*)p)[o] = {z.x, z.y};
 }
+// Row j of a record's cotangent (n_theta values: the padding rows of a column have none)
 template <typename R>
-__device__ __forceinline__ Z<R> gld(const double2* p, size_t o) {
-    const double2 a = p[o];
+__device__ __forceinline__ Z<R> gld(const InstDev& d, const double2* gbar, int j) {
+    if (!TK_IN(d.status, j, d.nth)) return {0, 0};
+    const double2 a = gbar[j];
     return {(R)a.x, (R)a.y};
 }
 
@@ -88,8 +90,8 @@ __global__ void adj_init_kernel(InstDev d, const double2* gbar, CoLevel out) {
     if (j >= d.pitch || i >= d.nr) return;
     size_t o = node_index(d, i, j);
     Z<double> a = {0, 0};
-    if (gbar && i == d.i_e) a = zscale(1.0 - d.f_e, gld<double>(gbar, j));
-    if (gbar && i == d.i_e + 1) a = zscale(d.f_e, gld<double>(gbar, j));
+    if (gbar && j < d.nth && i == d.i_e) a = zscale(1.0 - d.f_e, gld<double>(d, gbar, j));
+    if (gbar && j < d.nth && i == d.i_e + 1) a = zscale(d.f_e, gld<double>(d, gbar, j));
     if constexpr (sizeof(R) == 4) {
         ((float4*)out.F)[o] = make_float4((float)a.x, (float)a.y, 0.f, 0.f);
         ((float4*)out.Fc)[o] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -367,7 +369,7 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel(InstDev d, CoLevel lin,
             const size_t o = node_index(d, col, j);
             if (col < c0 || col >= c1 || !TK_IN(d.status, o, plane_elems(d))) continue;
             const double w = e ? d.f_e : 1.0 - d.f_e;
-            const Zd gb = gld<double>(gbar, j);
+            const Zd gb = gld<double>(d, gbar, j);
             stv<double>(lout.F, o, zadd(ldv<double>(lout.F, o), zscale(w, gb)));
         }
     }
@@ -481,7 +483,7 @@ __global__ void __launch_bounds__(kMaxT) adj_step_kernel_f32(InstDev d, CoLevel 
     float we = 0.f, we1 = 0.f;
     C gb = zero;
     if (gbar && row_ok && c0 <= ie + 1 && ie < c1) {
-        const Z<float> g = gld<float>(gbar, j);
+        const Z<float> g = gld<float>(d, gbar, j);
         gb = {g.x, g.y};
         we = (float)(1.0 - d.f_e);
         we1 = (float)d.f_e;
