@@ -595,9 +595,9 @@ void launch_adj_init(cudaStream_t st, const InstDev& d, const double2* gbar, con
 }
 
 // dynamic shared memory of the reverse-step kernels for blocks of `threads` rows
-template <typename R>
-static size_t adj_smem(int threads, bool f32) {
-    return 4 * (size_t)threads * (f32 ? sizeof(float4) : sizeof(Z<R>)) + (f32 ? kAdjRtCols * sizeof(RTab2) : 0);
+static size_t adj_smem_bytes(int prec, int threads) {
+    const bool f32 = prec != 0 && prec != 3;
+    return 4 * (size_t)threads * 16 + (f32 ? kAdjRtCols * sizeof(RTab2) : 0);
 }
 
 template <class K>
@@ -609,26 +609,24 @@ static int adj_resident(K kernel, int threads, size_t smem) {
     return (per > 0 ? per : 1) * (sms > 0 ? sms : 1);
 }
 
-// f(kernel, dynamic shared memory) with the reverse-step kernel built for blocks of t rows
-// (up to 256, 512 or 1024)
+// f(kernel, dynamic shared memory, rows) with the reverse-step kernel built for blocks of t
+// rows (up to 256, 512 or 1024: rows is the build's limit)
 template <class F>
 static void adj_dispatch(int prec, int t, F f) {
-    if (prec == 0 || prec == 3) {
-        const size_t sm = adj_smem<double>(t, false);
-        if (prec == 0) {
-            if (t <= 256) f(adj_step_kernel<double, 256>, sm);
-            else if (t <= 512) f(adj_step_kernel<double, 512>, sm);
-            else f(adj_step_kernel<double, 1024>, sm);
-        } else {
-            if (t <= 256) f(adj_step_kernel<DF, 256>, sm);
-            else if (t <= 512) f(adj_step_kernel<DF, 512>, sm);
-            else f(adj_step_kernel<DF, 1024>, sm);
-        }
+    const int rows = t <= 256 ? 256 : t <= 512 ? 512 : 1024;
+    const size_t sm = adj_smem_bytes(prec, t);
+    if (prec == 0) {
+        if (rows == 256) f(adj_step_kernel<double, 256>, sm, rows);
+        else if (rows == 512) f(adj_step_kernel<double, 512>, sm, rows);
+        else f(adj_step_kernel<double, 1024>, sm, rows);
+    } else if (prec == 3) {
+        if (rows == 256) f(adj_step_kernel<DF, 256>, sm, rows);
+        else if (rows == 512) f(adj_step_kernel<DF, 512>, sm, rows);
+        else f(adj_step_kernel<DF, 1024>, sm, rows);
     } else {
-        const size_t sm = adj_smem<float>(t, true);
-        if (t <= 256) f(adj_step_kernel_f32<256>, sm);
-        else if (t <= 512) f(adj_step_kernel_f32<512>, sm);
-        else f(adj_step_kernel_f32<1024>, sm);
+        if (rows == 256) f(adj_step_kernel_f32<256>, sm, rows);
+        else if (rows == 512) f(adj_step_kernel_f32<512>, sm, rows);
+        else f(adj_step_kernel_f32<1024>, sm, rows);
     }
 }
 
@@ -646,9 +644,12 @@ static void adj_dispatch(int prec, int t, F f) {
 // 10.0 -> 9.7, 4096 x 64 9.8 -> 9.4, 4096 x 128 14.0 both (with the step then at 588 instructions a node).
 AdjCut adj_step_plan(const InstDev& d) {
     int res = 1, dev = 0, sms = 0;
-    adj_dispatch(d.prec, d.pitch, [&](auto kernel, size_t sm) {
-        // (blocks of more than 256 rows, and capped ones, take more than the default 48 KB)
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)capped_smem(4, sm));
+    adj_dispatch(d.prec, d.pitch, [&](auto kernel, size_t sm, int rows) {
+        // Tall blocks, and capped ones, take more than the default 48 KB.  The limit belongs to the
+        // kernel, not to this context: it is set to what the build's tallest block and its smallest
+        // cap take, the same whoever calls, so that no call lowers it under another context's sweep
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)capped_smem(4, adj_smem_bytes(d.prec, rows)));
         res = adj_resident(kernel, d.pitch, sm);
     });
     cudaGetDevice(&dev);
@@ -682,7 +683,7 @@ static void adj_launch(cudaStream_t st, K kernel, int nb, int t, size_t sm, cons
 
 void launch_adj_step(cudaStream_t st, const InstDev& d, const CoLevel& lin, const double2* gbar,
                      const CoLevel& lout, const AdjCut& cut, void* wh, void* wi) {
-    adj_dispatch(d.prec, d.pitch, [&](auto kernel, size_t sm) {
+    adj_dispatch(d.prec, d.pitch, [&](auto kernel, size_t sm, int) {
         if (cut.cap > 0) sm = capped_smem(cut.cap, sm);
         adj_launch(st, kernel, cut.nb, d.pitch, sm, d, lin, gbar, lout, wh, wi);
     });
