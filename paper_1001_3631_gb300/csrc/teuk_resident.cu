@@ -405,10 +405,21 @@ __global__ void __launch_bounds__(kResMaxThreads, 1) resident_kernel(ResidentArg
 
 // ---------------------------------------------------------------- host side
 
+// The kernel's limit of dynamic shared memory is set to all that a block can have, not to one
+// plan's need: it belongs to the kernel, and a plan for a smaller grid must not lower it
+// under a context that launches a larger one.
 template <class P>
 static cudaError_t res_occupancy(int threads, size_t smem, int* per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(resident_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, resident_kernel<P>);
+    if (e != cudaSuccess) return e;
+    const int limit = optin - (int)fa.sharedSizeBytes;
+    if ((int64_t)smem > limit) return cudaErrorInvalidValue;
+    if (fa.maxDynamicSharedSizeBytes < limit)
+        e = cudaFuncSetAttribute(resident_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, resident_kernel<P>, threads, smem);
 }

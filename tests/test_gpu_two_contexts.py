@@ -44,3 +44,25 @@ def test_a_shorter_reverse_sweep_beside_a_tall_one(prec):
     assert not errors
     for ga, gr, _ in beside:
         assert np.array_equal(ga, alone[0]) and gr == alone[1]
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp64_df", "fp32_kahan", "fp32"])
+def test_a_small_resident_grid_planned_beside_a_large_one(prec):
+    # the plan of 241 x 32 takes less shared memory than that of 800 x 64
+    u0 = inputs.smooth_state(64, 800, seed=4)
+
+    def states(between):
+        with TeukSolver(params_of(800, 64, prec)) as s:
+            s.set_resident(1)
+            s.set_source(8.0)
+            s.set_state(u0)
+            s.step(7)
+            if between:
+                with TeukSolver(params_of(241, 32, prec)) as small:
+                    small.set_resident(1)
+                    small.step(3)
+                    small.sync()
+            s.step(7)
+            return s.get_state()
+
+    assert np.array_equal(states(False), states(True))
