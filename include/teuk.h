@@ -319,6 +319,12 @@ teuk_status teuk_get_geometry(const teuk_ctx* ctx, int instance, double* out);
  * (the per-point arithmetic is fixed). */
 teuk_status teuk_set_tiling(teuk_ctx* ctx, int strip, int steps_per_launch);
 
+/* The cut of one instance's columns in effect: shape[0..3] = {1 if automatic, 0 if a strip
+ * length is set; r* columns of its longest piece; pieces a step; 1 if the block-size classes
+ * of a context of several instances run side by side, else 0}.  (Resident and blocked
+ * launches have cuts of their own.) */
+teuk_status teuk_get_tiling(teuk_ctx* ctx, int instance, int* shape);
+
 /* Resident launches for a single-instance context whose grid fits the GPU's shared
  * memory (a not-in-the-paper launch form for small grids, such as 800 x 64): each
  * teuk_step_n becomes one cooperative launch in which every block keeps a run of r*

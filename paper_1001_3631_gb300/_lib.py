@@ -64,6 +64,7 @@ _PROTOS = {
     "teuk_check_selftest": (_I, [_P]),
     "teuk_get_time": (_I, [_P, _I, ctypes.POINTER(_L), ctypes.POINTER(_D)]),
     "teuk_set_tiling": (_I, [_P, _I, _I]),
+    "teuk_get_tiling": (_I, [_P, _I, _P]),
     "teuk_set_resident": (_I, [_P, _I]),
     "teuk_set_resident_shape": (_I, [_P, _I, _I]),
     "teuk_set_blocked": (_I, [_P, _I, _I]),

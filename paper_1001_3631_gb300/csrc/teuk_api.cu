@@ -296,12 +296,14 @@ InstDev dev_of(const teuk_ctx* c, const Instance& I) {
     return d;
 }
 
-// Strip length so that the grid holds about 16 warps per SM on 152 SMs, at least
-// 8 columns (a strip reads 2 columns beyond its outputs).
-// Strip length that gives one wave of resident blocks (at most 512 columns).  Grids too
-// small to fill the GPU get one column per block: the step time is then the ring's
-// start-up plus the strip, so the shortest strip is fastest (800 x 64 on GB300: 4.2 us
-// per step at one column, 8.2 us at eight).
+// Whether no strip length is set for the instance: per-step launches then take the cut of
+// auto_cut, batched ones the length of batch_strip.  (Not told by the length: a length that is
+// set may equal auto_strip.)
+bool auto_tiled(const teuk_ctx* c, const Instance& I) { return I.strip == 0 && c->strip == 0; }
+
+// Strip length that gives one wave of resident blocks (at most 512 columns; grids too small to
+// fill the GPU get one column per block).  It names an automatic launch (eff_strip) but does
+// not cut it.
 int auto_strip(const Instance& I) {
     int64_t blocks = I.resident > 0 ? I.resident : 1;
     int64_t cols = I.p.n_rstar - 2;
@@ -362,7 +364,7 @@ teuk_status refresh_partition(teuk_ctx* c, Instance& I) {
     const int strip = eff_strip(c, I);
     const int nr = I.p.n_rstar;
     int nb = (nr - 2 + strip - 1) / strip, cap = 0;
-    if (strip == auto_strip(I)) auto_cut(I, c->sms, &nb, &cap);
+    if (auto_tiled(c, I)) auto_cut(I, c->sms, &nb, &cap);
     const double alpha = I.p.prec == TEUK_FP64      ? 0.1
                          : I.p.prec == TEUK_FP64_DF ? (I.sd.moving ? 0.6 : 0.4)
                                                     : (I.sd.moving ? 0.8 : 0.25);
@@ -1033,6 +1035,23 @@ void enqueue_batched_branches(teuk_ctx* c, cudaStream_t st) {
     for (size_t k = 1; k < B.cls.size(); ++k) cudaStreamWaitEvent(st, B.cls[k].done, 0);
 }
 
+// The block-size classes: the instances of one theta pitch each.
+void form_classes(const teuk_ctx* c, Batch& B) {
+    if (!B.cls.empty()) return;
+    for (int k = 0; k < (int)c->inst.size(); ++k) {
+        const int pitch = c->inst[k].pitch;
+        BatchClass* K = nullptr;
+        for (BatchClass& q : B.cls)
+            if (q.pitch == pitch) K = &q;
+        if (!K) {
+            B.cls.emplace_back();
+            K = &B.cls.back();
+            K->pitch = pitch;
+        }
+        K->members.push_back(k);
+    }
+}
+
 // Whether the classes run side by side, and their shares: a whole number of blocks of every
 // class on each SM (512 threads at the kernels' 128 registers), so that the launches find
 // their places whatever their order; blocks are added where a block has most columns.
@@ -1108,21 +1127,7 @@ int batch_strip(const teuk_ctx* c, const Instance& I, const BatchClass& K, int g
 // once in a CUDA graph and replayed (the per-call descriptors are uploaded first).
 teuk_status batched_step(teuk_ctx* c, int64_t n) {
     Batch& B = c->batch;
-    const int ni = (int)c->inst.size();
-    if (B.cls.empty()) {
-        for (int k = 0; k < ni; ++k) {
-            int pitch = c->inst[k].pitch;
-            BatchClass* K = nullptr;
-            for (BatchClass& q : B.cls)
-                if (q.pitch == pitch) K = &q;
-            if (!K) {
-                B.cls.emplace_back();
-                K = &B.cls.back();
-                K->pitch = pitch;
-            }
-            K->members.push_back(k);
-        }
-    }
+    form_classes(c, B);
     plan_branches(c, B);
     // per-class descriptor blocks:
     // InstDev[m] | item_base[m+1] | base_step[m] | n_steps | strip[m] | nstrip[m] | base_bin[m]
@@ -1657,6 +1662,29 @@ extern "C" teuk_status teuk_set_tiling(teuk_ctx* c, int strip, int steps_per_lau
     c->steps_per_launch = steps_per_launch;
     invalidate_graph(c);
     return refresh_partitions(c);
+}
+
+extern "C" teuk_status teuk_get_tiling(teuk_ctx* c, int instance, int* shape) {
+    teuk_status st = check_instance(c, instance);
+    if (st) return st;
+    if (!shape) TK_FAIL(c, TEUK_EINVAL, "null output");
+    const Instance& I = c->inst[instance];
+    shape[0] = auto_tiled(c, I) ? 1 : 0;
+    shape[3] = 0;
+    if (c->inst.size() > 1 || c->steps_per_launch == 0) {
+        Batch& B = c->batch;
+        form_classes(c, B);
+        plan_branches(c, B);
+        for (const BatchClass& K : B.cls)
+            if (K.pitch == I.pitch) shape[1] = batch_strip(c, I, K, B.branches ? K.share : K.grid);
+        shape[2] = (I.p.n_rstar - 2 + shape[1] - 1) / shape[1];
+        shape[3] = B.branches ? 1 : 0;
+    } else {
+        shape[1] = 0;
+        for (int b = 0; b < I.part_nb; ++b) shape[1] = std::max(shape[1], I.h_part[b + 1] - I.h_part[b]);
+        shape[2] = I.part_nb;
+    }
+    return TEUK_OK;
 }
 
 extern "C" teuk_status teuk_set_fault_injection(teuk_ctx* c, int64_t skip_release_item,

@@ -314,6 +314,13 @@ class TeukSolver:
         check(_lib.load().teuk_set_tiling(self.ctx, strip, steps_per_launch), self.ctx)
         self._steps_per_launch = steps_per_launch
 
+    def tiling(self, instance=0):
+        """The cut of an instance's columns in effect: dict(automatic, columns (of the longest
+        piece), pieces, side_by_side (the block-size classes of a batch))."""
+        out = (ctypes.c_int * 4)()
+        check(_lib.load().teuk_get_tiling(self.ctx, instance, out), self.ctx)
+        return dict(automatic=bool(out[0]), columns=out[1], pieces=out[2], side_by_side=bool(out[3]))
+
     def set_resident(self, halo=1, blocks_per_sm=1):
         """Resident launches (one cooperative launch per step() call, the grid held in
         shared memory, boundary columns exchanged every ``halo`` steps, the column runs cut
