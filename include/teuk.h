@@ -360,16 +360,18 @@ teuk_status teuk_set_blocked(teuk_ctx* ctx, int steps, int blocks_per_sm);
 teuk_status teuk_set_instance_tiling(teuk_ctx* ctx, int instance, int strip);
 
 /* Autotuner of the strip length (r* columns per block), written to every instance
- * (chosen, may be NULL, receives them).  A single instance stepped one launch per step:
- * trial_steps steps of each candidate (1 .. 512 columns) and of resident launches with
- * halo 1 .. 4 and 1 .. 3 blocks per SM (teuk_set_resident_shape, where the grid fits) on
- * a scratch copy of the instance; the fastest is applied, and chosen[k] < 0 reports
- * resident launches with halo (-chosen[k]) % 16 and (-chosen[k]) / 16 + 1 blocks per SM.  Contexts that run the persistent kernels (several instances, or one with
- * steps_per_launch = 0): trial_steps steps of the whole context per candidate (16 .. 512),
- * one length for all instances first, then block-size class by class, on the live state,
- * which is restored afterwards from a snapshot (device memory for one copy of every
- * instance's state and waveform ring while the call runs).  The state, the time levels
- * and the waveform records are unchanged on return.  Synchronizes. */
+ * (chosen, may be NULL, receives them; 0: no length of its own is fastest, that is the
+ * automatic cut unless teuk_set_tiling set a length).  A single instance stepped one launch
+ * per step: trial_steps steps of that cut, of each candidate (1 .. 512 columns) and of
+ * resident launches with halo 1 .. 4 and 1 .. 3 blocks per SM (teuk_set_resident_shape,
+ * where the grid fits) on a scratch copy of the instance; the fastest is applied, and
+ * chosen[k] < 0 reports resident launches with halo (-chosen[k]) % 16 and
+ * (-chosen[k]) / 16 + 1 blocks per SM.  Contexts that run the persistent kernels (several
+ * instances, or one with steps_per_launch = 0): trial_steps steps of the whole context per
+ * candidate (0, 16 .. 512), one choice for all instances first, then block-size class by
+ * class, on the live state, which is restored afterwards from a snapshot (device memory for
+ * one copy of every instance's state and waveform ring while the call runs).  The state, the
+ * time levels and the waveform records are unchanged on return.  Synchronizes. */
 teuk_status teuk_autotune(teuk_ctx* ctx, int trial_steps, int* chosen);
 
 /* Testing aid for the bounded device waits of the batched kernel: work item

@@ -1777,7 +1777,7 @@ static teuk_status autotune_batched(teuk_ctx* c, int trial_steps, int* chosen) {
         return TEUK_OK;
     };
     auto set_strip = [&](const std::vector<int>& members, int L) {
-        for (int k : members) c->inst[k].strip = std::max(1, std::min(L, c->inst[k].p.n_rstar - 2));
+        for (int k : members) c->inst[k].strip = std::min(L, c->inst[k].p.n_rstar - 2);
     };
     // block-size classes, as batched_step forms them (instances with the same pitch)
     std::vector<std::vector<int>> cls;
@@ -1792,20 +1792,21 @@ static teuk_status autotune_batched(teuk_ctx* c, int trial_steps, int* chosen) {
         }
         cls[q].push_back(k);
     }
-    // strips of 16 to 512 columns; shorter ones as well when 16-column strips would leave
+    // no length of its own (0: the length of batch_strip, unless the context has one), strips of
+    // 16 to 512 columns; shorter ones as well when 16-column strips would leave
     // fewer than four work items per step for each SM (a grid too small to fill the GPU,
     // where one-column strips are fastest)
-    std::vector<int> cand = {16, 32, 64, 128, 256, 512};
+    std::vector<int> cand = {0, 16, 32, 64, 128, 256, 512};
     {
         int64_t items16 = 0;
         for (int k = 0; k < ni; ++k) items16 += (c->inst[k].p.n_rstar - 2 + 15) / 16;
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (items16 < 4 * (int64_t)(sms > 0 ? sms : 1)) cand.insert(cand.begin(), {1, 2, 4, 8});
+        if (items16 < 4 * (int64_t)(sms > 0 ? sms : 1)) cand.insert(cand.begin() + 1, {1, 2, 4, 8});
     }
     float best_ms = 1e30f;
-    int best_all = 128;
+    int best_all = 0;
     teuk_status st = TEUK_OK;
     for (int L : cand) {
         set_strip(all, L);
@@ -1858,8 +1859,9 @@ static teuk_status autotune_batched(teuk_ctx* c, int trial_steps, int* chosen) {
     return refresh_partitions(c);
 }
 
-// Single instance stepped one launch per step: time each candidate strip length on a
-// scratch copy of the instance and keep the fastest.  Otherwise see autotune_batched.
+// Single instance stepped one launch per step: time the cut without a length of its own (the
+// automatic one, unless the context has a length), then each candidate strip length, on a
+// scratch copy of the instance, and keep the fastest.  Otherwise see autotune_batched.
 extern "C" teuk_status teuk_autotune(teuk_ctx* c, int trial_steps, int* chosen) {
     if (!c) return TEUK_EINVAL;
     if (trial_steps < 1) TK_FAIL(c, TEUK_EINVAL, "trial_steps must be >= 1");
@@ -1884,7 +1886,11 @@ extern "C" teuk_status teuk_autotune(teuk_ctx* c, int trial_steps, int* chosen) 
                                     c->stream) != cudaSuccess)
             err = TEUK_ENOMEM;
         float best_ms = 1e30f;
-        int best_strip = auto_strip(I);
+        int best_strip = 0;
+        if (!err) {
+            I.strip = 0;
+            err = refresh_partition(c, I);
+        }
         if (!err) {
             InstDev d = dev_of(c, I);
             d.wave = scr_wave;           // trial records must not touch the live ring
@@ -1895,11 +1901,13 @@ extern "C" teuk_status teuk_autotune(teuk_ctx* c, int trial_steps, int* chosen) 
                 d.buf[0][q] = scr[0][q];
                 d.buf[1][q] = scr[1][q];
             }
-            const int cand[] = {auto_strip(I), 1, 2, 4, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512};
-            for (int ch : cand) {
+            // (0 first and last: the first launches meet a GPU that may be idle)
+            for (int ch : {0, 1, 2, 4, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512, 0}) {
                 if (ch > I.p.n_rstar - 2) continue;
-                // (the automatic length times the partition it stands for)
-                const StepCut cut = cut_of(c, I, ch);
+                StepCut cut;   // (a candidate length: uniform strips)
+                cut.strip = ch;
+                cut.room = I.resident;
+                if (ch == 0) cut = cut_of(c, I, I.part_strip);
                 for (int w = 0; w < 2; ++w) launch_step(c->stream, d, I.step + w, w & 1, cut);
                 cudaEventRecord(e0, c->stream);
                 for (int t = 0; t < trial_steps; ++t) launch_step(c->stream, d, I.step + t, t & 1, cut);

@@ -88,6 +88,10 @@ def _stream_handle(stream):
     return stream.cuda_stream
 
 
+# of the rules that cut the columns automatically: tables tuned against other rules are not used
+_CUT_VERSION = 2
+
+
 class _HostBuffers:
     """Result arrays whose memory is used again once the caller has dropped them (every view
     included).  A fresh array of 134 MB (a 16384 x 256 state) costs 6 to 20 ms of page faults
@@ -347,11 +351,14 @@ class TeukSolver:
 
     def autotune(self, trial_steps=10, cache_path=None):
         """Strip length per instance from a cached table keyed by (GPU, launch mode, n_theta,
-        precision, n_rstar bucket); entries missing from the table are timed by
-        teuk_autotune.  A negative entry -v (single instance stepped per call) selects
-        resident launches with halo v % 16 and v // 16 + 1 blocks per SM.  The launch mode is "step" for one instance stepped one launch per
-        step, and for contexts that run the persistent kernels a signature of the whole
-        set of instances (their best strips depend on one another)."""
+        precision, n_rstar bucket, version of the kernels' automatic cut); entries missing
+        from the table are timed by teuk_autotune.  An entry 0 stands for no length of its own
+        (the automatic cut: on another grid of the bucket, that grid's).  A negative entry -v
+        (single instance stepped per call) selects resident launches with halo v % 16 and
+        v // 16 + 1 blocks per SM.  The launch mode is "step" for one instance stepped one
+        launch per step, and for contexts that run the persistent kernels a signature of the
+        whole set of instances (their best strips depend on one another).  Returns the lengths
+        in effect (of the longest piece for an automatic cut), or the negative entries."""
         import hashlib
 
         import torch
@@ -363,8 +370,8 @@ class TeukSolver:
         else:
             shapes = sorted((p.n_rstar, p.n_theta, p.prec) for p in self.params)
             mode = "batch:" + hashlib.sha1(repr(shapes).encode()).hexdigest()[:12]
-        keys = ["%s|%s|%d|%d|%d" % (gpu, mode, p.n_theta, p.prec, int(np.ceil(np.log2(p.n_rstar))))
-                for p in self.params]
+        keys = ["%s|%s|%d|%d|%d|cut%d" % (gpu, mode, p.n_theta, p.prec, int(np.ceil(np.log2(p.n_rstar))),
+                                          _CUT_VERSION) for p in self.params]
         table = {}
         if os.path.exists(path):
             try:
@@ -381,7 +388,7 @@ class TeukSolver:
                     self.set_instance_tiling(i, v)
                     if self.n == 1 and self._steps_per_launch != 0:
                         self.set_resident(0)
-            return [int(table[k]) for k in keys]
+            return self._in_effect([int(table[k]) for k in keys])
         chosen = np.zeros(self.n, dtype=np.int32)
         check(_lib.load().teuk_autotune(self.ctx, trial_steps, chosen.ctypes.data_as(ctypes.c_void_p)),
               self.ctx)
@@ -395,4 +402,7 @@ class TeukSolver:
             os.replace(tmp, path)
         except OSError:
             pass
-        return [int(c) for c in chosen]
+        return self._in_effect([int(c) for c in chosen])
+
+    def _in_effect(self, chosen):
+        return [c or self.tiling(i)["columns"] for i, c in enumerate(chosen)]

@@ -1,5 +1,7 @@
 """The cut of the columns that is in effect (teuk_get_tiling): a strip length that is set is
-kept whatever its value."""
+kept whatever its value, and the autotuner knows the automatic cut."""
+import json
+
 import pytest
 
 from paper_1001_3631_gb300 import TeukSolver
@@ -27,3 +29,44 @@ def test_a_strip_that_is_set_is_kept(nr, nth, prec):
                 assert (t["automatic"], t["pieces"]) == (False, pieces), (strip, t)
                 put(0)
                 assert s.tiling() == auto
+
+
+def test_the_tuner_keeps_an_automatic_cut_that_is_fastest(tmp_path):
+    # FP64 2048 x 128 (too large for resident launches): 43.7 us a step, uniform strips 51
+    with TeukSolver(params_of(2048, 128, "fp64")) as s:
+        s.set_instance_tiling(0, 5)
+        chosen = s.autotune(trial_steps=30, cache_path=str(tmp_path / "t.json"))
+        t = s.tiling()
+        assert t["automatic"] and chosen == [t["columns"]]
+    table = json.loads((tmp_path / "t.json").read_text())
+    assert list(table.values()) == [0]
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_a_cached_automatic_cut_is_each_grids_own(tmp_path, batch):
+    # one entry serves every grid of its bucket (a batch: every context of the same shapes)
+    cache = tmp_path / "t.json"
+    grids = [8000, 8000] if batch else [8000, 5001]
+    for k, nr in enumerate(grids):
+        ps = [params_of(nr, 128, "fp32_kahan")] * (2 if batch else 1)
+        with TeukSolver(ps) as s:
+            auto = s.tiling()
+            if k == 0:
+                s.autotune(trial_steps=2, cache_path=str(cache))
+                cache.write_text(json.dumps({key: 0 for key in json.loads(cache.read_text())}))
+                continue
+            s.set_instance_tiling(0, 7)
+            launches = s.kernel_launches()
+            assert s.autotune(cache_path=str(cache)) == [auto["columns"]] * len(ps)
+            assert s.kernel_launches() == launches and s.tiling() == auto
+
+
+def test_tables_of_other_cuts_are_not_used(tmp_path):
+    cache = tmp_path / "t.json"
+    with TeukSolver(params_of(8000, 128, "fp32_kahan")) as s:
+        s.autotune(trial_steps=2, cache_path=str(cache))
+        (key,) = json.loads(cache.read_text())
+        old = key.rsplit("|", 1)[0]   # as written before the cut had a version
+        cache.write_text(json.dumps({old: 3}))
+        s.autotune(trial_steps=2, cache_path=str(cache))
+        assert json.loads(cache.read_text()).keys() == {old, key}
