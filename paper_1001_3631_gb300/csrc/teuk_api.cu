@@ -1053,12 +1053,15 @@ void form_classes(const teuk_ctx* c, Batch& B) {
 }
 
 // Whether the classes run side by side, and their shares: a whole number of blocks of every
-// class on each SM (512 threads at the kernels' 128 registers), so that the launches find
-// their places whatever their order; blocks are added where a block has most columns.
-// us per step, one class after the other -> side by side: 6 modes of 1024..4100 columns and 64,
-// 128, 192 rows, FP32-Kahan 46.2 -> 37.0, double-float 118.8 -> 96.1; two of them 19.6 -> 13.1.
-// Not so with few columns (6 modes of 20..60 rows, 4.4 columns a place: 20.0 -> 22.0) or many
-// (128 instances, 2000 columns a place: 1727 -> 1900, an eighth of the threads left over).
+// class on each SM (512 threads at the kernels' 128 registers, within the shared memory that
+// the kernels ask for, kBatchCarveout), so that the launches find their places whatever their
+// order; blocks are added where a block has most columns.  Measured on 54 batches of two to
+// four classes of 1 to 10 warps, in each precision: one class after the other / side by side.
+//   longest share up to 1.3 of the even one and up to 70 columns a place: 0.99 to 2.5 (FP32-Kahan
+//     6 modes of 1024..4100 columns and 64, 128, 192 rows, 47 columns: 46.2 -> 37.0 us; 20, 50,
+//     70 rows, 0.3 columns: 24.9 -> 10.3; FP64 3000 columns of 32 and 64 rows, 4.9: 63.2 -> 55.8)
+//   86 columns a place: 0.83 to 0.89, 104: 0.99 to 1.05; 2000 (128 instances): 0.94
+//   longest share 1.35 to 1.5: 0.99 to 3.1; 1.6 to 1.9 with 24 columns and more: 0.75 to 1.05
 void plan_branches(teuk_ctx* c, Batch& B) {
     constexpr int kThreads = 512;
     std::vector<double> work(B.cls.size(), 0.0);
@@ -1090,9 +1093,9 @@ void plan_branches(teuk_ctx* c, Batch& B) {
         longest = std::max(longest, load(k));
         B.cls[k].share = n[k] * c->sms;
     }
-    // well balanced, and of a size that waiting matters in: columns a place, all classes
+    // well balanced, and not of a size that waiting no longer matters in (columns a place)
     const double columns = total / kThreads / c->sms;
-    B.branches = longest <= 1.3 * total / kThreads && columns >= 5.0 && columns <= 100.0;
+    B.branches = longest <= 1.3 * total / kThreads && columns <= 70.0;
 }
 
 // The side streams and events of the branches; false if they cannot be had (the classes then

@@ -971,6 +971,17 @@ void launch_step(cudaStream_t st, const InstDev& d, int64_t step, int bin, const
     else launch_step_p<PK>(st, d, step, bin, cut);
 }
 
+// Shared memory that the batched kernels of up to 512 rows ask an SM to set aside, per cent of
+// its 228 KB: 164 KB, room for the 512 threads of a plan of several classes side by side
+// (plan_branches: at most 256 bytes a thread and 1.7 KB a block, of 16 blocks 155 KB).
+// Left to the launches, an SM set aside what the class that came first needs; the blocks of
+// the other class found no room there and joined only when it had finished.  us per step,
+// FP32-Kahan 32 + 64 rows, 12000 columns each: 46.4 -> 30.4, one class after the other 33.4;
+// FP64 128 + 160 rows: 210 -> 121, 128.  What the L1 loses costs nothing (one class after the
+// other 1.00 in 54 batches); 100 per cent costs double-float 3 to 10 % (its tables come
+// through the L1), 70 per cent leaves 132 KB, too little.
+constexpr int kBatchCarveout = 72;
+
 // Opt the step kernels in to the dynamic shared memory of their largest blocks (on the
 // current device; called when a context is created).
 template <class P, bool kMov>
@@ -988,6 +999,9 @@ static cudaError_t prepare_m() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(batched_step_kernel<P, 256, P::blocks256, kRingS, kMov>, a, s);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(batched_step_kernel<P, 512, 1, kRingS, kMov>, a, m);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(batched_step_kernel<P, 1024, 1, kRingL, kMov>, a, l);
+    const cudaFuncAttribute cv = cudaFuncAttributePreferredSharedMemoryCarveout;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(batched_step_kernel<P, 256, P::blocks256, kRingS, kMov>, cv, kBatchCarveout);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(batched_step_kernel<P, 512, 1, kRingS, kMov>, cv, kBatchCarveout);
     return e;
 }
 template <class P>
