@@ -120,7 +120,10 @@ class _HostBuffers:
             buf = next((b for b in idle if len(b[0]) == size), None)
             again = buf is not None
             if buf is None:
-                m = mmap.mmap(-1, size, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS)
+                try:
+                    m = mmap.mmap(-1, size, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS)
+                except (OSError, OverflowError, ValueError):   # not to be had: numpy's own answer
+                    return np.empty(shape, dtype)
                 try:   # (as numpy does for its own arrays)
                     m.madvise(mmap.MADV_HUGEPAGE)
                 except (AttributeError, OSError):
