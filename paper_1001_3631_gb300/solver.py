@@ -98,14 +98,57 @@ class _HostBuffers:
     and unmapping a call, on GB300 with its fast host link the copy itself 0.9 ms.  Memory that
     the GPU alone goes on using is moved about by the driver, and every few copies then take
     15 to 35 ms; one access by the host to each page before the copy keeps it where it is
-    (`_touch`, 0.05 ms).  Arrays below 4 MB come from numpy (its heap reuses them); at most KEEP
-    bytes are kept idle, by the solver that made them (any thread may drop an array or ask for
-    one)."""
+    (`_touch`, 0.05 ms).  Arrays below 4 MB come from numpy (its heap reuses them).  At most
+    KEEP bytes are kept idle, counted whenever an array is dropped or asked for, the longest
+    idle given back first, and none once the last solver is closed (any thread may drop an
+    array or ask for one)."""
     MIN, KEEP = 4 << 20, 1 << 30
 
     def __init__(self):
         self._lock = threading.Lock()
         self._bufs = []   # [mapping, weak reference to the object that its arrays hold], oldest first
+        self._dropped = False   # an array died since the idle mappings were last counted
+        self._users, self._closed = 0, False
+
+    def open(self):
+        """One more solver."""
+        with self._lock:
+            self._users += 1
+            self._closed = False
+
+    def close(self):
+        """One solver less; after the last nothing is kept idle."""
+        with self._lock:
+            self._users -= 1
+            self._closed = self._users <= 0
+        self._dropped = True
+        self._settle()
+
+    def _settle(self):
+        # runs in whatever thread drops an array, at any moment (within empty() too, by the
+        # collector): it never waits; who holds the lock settles again after giving it back
+        while self._dropped and self._lock.acquire(blocking=False):
+            try:
+                self._dropped = False
+                idle = [b for b in self._bufs if b[1]() is None]
+                kept = sum(len(b[0]) for b in idle)
+                for b in idle:
+                    if kept <= (0 if self._closed else self.KEEP):
+                        break
+                    self._bufs.remove(b)
+                    kept -= len(b[0])
+            finally:
+                self._lock.release()
+
+    def _watch(self, raw):
+        pool = weakref.ref(self)
+
+        def dropped(_):
+            p = pool()
+            if p is not None:
+                p._dropped = True
+                p._settle()
+        return weakref.ref(raw, dropped)
 
     def empty(self, shape, dtype=np.float64):
         dtype = np.dtype(dtype)
@@ -115,35 +158,35 @@ class _HostBuffers:
         size = count * dtype.itemsize
         if size < self.MIN:
             return np.empty(shape, dtype)
+        # mappings come in sixteen sizes an octave, so that records that grow from call to call
+        # find one again
+        step = 1 << (size.bit_length() - 5)
+        whole = (size + step - 1) // step * step
         with self._lock:
-            idle = [b for b in self._bufs if b[1]() is None]
-            buf = next((b for b in idle if len(b[0]) == size), None)
+            buf = next((b for b in self._bufs if len(b[0]) == whole and b[1]() is None), None)
             again = buf is not None
-            if buf is None:
-                try:
-                    m = mmap.mmap(-1, size, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS)
-                except (OSError, OverflowError, ValueError):   # not to be had: numpy's own answer
-                    return np.empty(shape, dtype)
-                try:   # (as numpy does for its own arrays)
-                    m.madvise(mmap.MADV_HUGEPAGE)
-                except (AttributeError, OSError):
-                    pass
-                buf = [m, None]
-            else:
-                idle.remove(buf)
+            if again:
                 self._bufs.remove(buf)
-            self._bufs.append(buf)
-            kept = sum(len(b[0]) for b in idle)
-            for b in idle:
-                if kept <= self.KEEP:
-                    break
-                self._bufs.remove(b)
-                kept -= len(b[0])
-            raw = (ctypes.c_char * size).from_buffer(buf[0])
-            buf[1] = weakref.ref(raw)   # dead when the last array on the mapping is gone
+            else:
+                try:
+                    buf = [mmap.mmap(-1, whole, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS), None]
+                    # (as numpy does for its own arrays)
+                    buf[0].madvise(mmap.MADV_HUGEPAGE)
+                except (AttributeError, OSError, OverflowError, ValueError):
+                    pass
+            if buf is not None:
+                raw = (ctypes.c_char * size).from_buffer(buf[0])
+                buf[1] = self._watch(raw)   # dead when the last array on the mapping is gone
+                self._bufs.append(buf)
+        self._settle()
+        if buf is None:   # no mapping to be had: numpy's own answer
+            return np.empty(shape, dtype)
         if again:
             np.frombuffer(raw, np.uint8)[::mmap.PAGESIZE] = 0
         return np.frombuffer(raw, dtype, count).reshape(shape)
+
+
+_HOST = _HostBuffers()   # of every solver of the process
 
 
 def _touch(u):
@@ -154,14 +197,18 @@ def _touch(u):
 
 
 class TeukSolver:
-    """One context of one or more instances (see teuk_create)."""
+    """One context of one or more instances (see teuk_create).
+
+    Result arrays of 4 MB and more (get_state, extract, mode_sum) lie in host memory that is
+    used again once every view of them is dropped; up to 1 GB of it stays idle while a solver
+    of the process is open.  Such an array does not own its data: `ndarray.resize` refuses it
+    (resize a copy)."""
 
     def __init__(self, params, stream=None):
         if isinstance(params, dict):
             params = [params]
         plist = [p if isinstance(p, _lib.teuk_params) else make_params(**p) for p in params]
         self.n = len(plist)
-        self._host = _HostBuffers()
         arr = (_lib.teuk_params * self.n)(*plist)
         self.params = plist
         self._stream = stream
@@ -170,6 +217,8 @@ class TeukSolver:
         st = lib.teuk_create(arr, self.n, ctypes.c_void_p(_stream_handle(stream)), ctypes.byref(h))
         check(st, None)
         self.ctx = h
+        self._host = _HOST
+        self._host.open()
         self._steps_per_launch = 1
 
     # -- lifetime
@@ -177,6 +226,7 @@ class TeukSolver:
         if getattr(self, "ctx", None):
             _lib.load().teuk_destroy(self.ctx)
             self.ctx = None
+            self._host.close()
 
     def __del__(self):
         try:
