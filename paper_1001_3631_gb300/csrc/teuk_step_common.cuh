@@ -101,8 +101,7 @@ __device__ __forceinline__ Cx<DF> neg(Cx<DF> a) {
     return up2({p_neg(A.hi), p_neg(A.lo)});
 }
 // a * b + c per component, a given as pairs (hi, lo): the double-float tfma without its last
-// normalisation, so that lo may reach a few units in the last place of hi (one per link of a
-// chain of such sums)
+// normalisation (see Lin<DF> for how large lo may get)
 __device__ __forceinline__ DF2 p_tfma(DF2 A, DF2 B, DF2 C) {
     const float2 p = __fmul2_rn(A.hi, B.hi);
     float2 e = __ffma2_rn(A.hi, B.hi, p_neg(p));
@@ -425,9 +424,15 @@ template <> struct Lin<double> {
 };
 // Double-float: the sums, differences and products of a step's chain stay unnormalised (three
 // operations saved in each; as in Ogita, Rump and Oishi's compensated dot product, the
-// residues are summed apart), only the state that is stored is normalised (update).  The
-// error against 64 bits is the same (8192 x 128, 300 steps: 1.83e-14 both; 3001 x 300: 1.60e-14
-// both).  us per step: 16384 x 256 148 -> 136 (the tables and the state alone take 129 at the
+// residues are summed apart), only the state that is stored is normalised (update).  With
+// u = 2^-24, n links and M the sum of the moduli of a chain's terms, a partial sum's lo stays
+// within (n + 8) u M and the error within (38 + n + 2 n (n + 8)) u^2 M, also where hi cancels
+// and lo holds the rest (the bounds count M, not the sum).  Measured on 2e6 chains of n = 10,
+// half of them cancelling: rms 0.51, at most 13 u^2 M; normalised 0.31 and 4.9.  In a run the
+// rounding of the state outweighs it: the error against 64 bits over 36 runs of 241 x 32 to
+// 16384 x 256, in proportion to the normalised form's, is on average 1.002 (state, L2), 0.994
+// (state, largest), 0.966 (waveform, L2) and 0.962 (waveform, largest).
+// us per step: 16384 x 256 148 -> 136 (the tables and the state alone take 129 at the
 // measured copy rate), 8192 x 128 43.5 -> 37.9, 800 x 64 5.4 -> 4.8.
 template <> struct Lin<DF> {
     using C = Cx<DF>;
