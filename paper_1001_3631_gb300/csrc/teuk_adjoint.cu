@@ -37,11 +37,6 @@ template <typename R>
 __device__ __forceinline__ Z<R> zadd(Z<R> a, Z<R> b) { return {a.x + b.x, a.y + b.y}; }
 template <typename R>
 __device__ __forceinline__ Z<R> zscale(R s, Z<R> a) { return {s * a.x, s * a.y}; }
-// conj(cr + i ci) * z
-template <typename R>
-__device__ __forceinline__ Z<R> zconjmul(R cr, R ci, Z<R> z) {
-    return {cr * z.x + ci * z.y, cr * z.y - ci * z.x};
-}
 
 template <typename R> struct R2T;
 template <> struct R2T<double> { using V = double2; };

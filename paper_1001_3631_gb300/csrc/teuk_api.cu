@@ -276,7 +276,6 @@ InstDev dev_of(const teuk_ctx* c, const Instance& I) {
     const DF h2(d.hdt), q2(d.qdt);
     d.hdt2 = make_float2(h2.hi, h2.lo);
     d.qdt2 = make_float2(q2.hi, q2.lo);
-    d.dt_f = (float)I.dt;
     for (int b = 0; b < 2; ++b)
         for (int k = 0; k < 2; ++k) d.buf[b][k] = I.state[b][k];
     d.coef_h = I.coef_h;
@@ -409,15 +408,14 @@ teuk_status refresh_partitions(teuk_ctx* c) {
     return TEUK_OK;
 }
 
-// The 2D coefficient tables [9][n_rstar][pitch] at half and integer nodes, in the
-// instance's precision: read by the FP64 and double-float step kernels and their adjoint,
-// built at creation.  FP32 instances form their coefficients from 1D tables, forward and
+// The 2D coefficient tables (coef_index) at half and integer nodes, in the instance's
+// precision: read by the FP64 and double-float step kernels and their adjoint, built at
+// creation.  FP32 instances form their coefficients from 1D tables, forward and
 // adjoint, and have none.
 teuk_status coef_tables(teuk_ctx* c, Instance& I) {
     if (I.coef_h) return TEUK_OK;
     const teuk_params& q = I.p;
-    const size_t cs = q.prec == TEUK_FP64 ? sizeof(double) : q.prec == TEUK_FP64_DF ? sizeof(float2) : sizeof(float);
-    const size_t cbytes = (size_t)kNCoef * q.n_rstar * I.pitch * cs;
+    const size_t cbytes = (size_t)kNCoef * q.n_rstar * I.pitch * 8;   // double or (hi, lo)
     TK_CUDA(c, dmalloc(c, &I.coef_h, cbytes, c->stream));
     TK_CUDA(c, dmalloc(c, &I.coef_i, cbytes, c->stream));
     launch_coefficients(c->stream, q.prec, q.M, q.a, q.s, q.m, q.rstar_min, I.drs, I.dth, I.dt,
@@ -2167,7 +2165,7 @@ extern "C" teuk_status teuk_adjoint_n(teuk_ctx* c, int instance, int64_t step0, 
         TK_CUDA(c, B.get(&lam[b].F, plane));
         TK_CUDA(c, B.get(co32 ? &lam[b].Fc : &lam[b].P, plane));
     }
-    // the fused reverse step's strip; with a source, a ring of window co-states that
+    // the fused reverse step's cut; with a source, a ring of window co-states that
     // adj_src_grad_kernel turns into gradients every `slots` steps (32 MB at most)
     const AdjCut adj_cut = adj_step_plan(dev_of(c, I));
     const bool src_on = I.src_on;

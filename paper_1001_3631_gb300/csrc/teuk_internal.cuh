@@ -111,7 +111,6 @@ struct InstDev {
     // 14 (double-float) instructions a node on the FP64 pipe (see step_hdt)
     double hdt, qdt;
     float2 hdt2, qdt2;        // (hi, lo)
-    float dt_f, pad_f;
     void* buf[2][2];          // [ping-pong buffer][plane]
     const void* coef_h;       // tiles of double or (hi, lo) float pairs (coef_index)
     const void* coef_i;

@@ -6,8 +6,8 @@
 // by bulk-async (TMA) copies several columns ahead of use; at each column the block
 // computes the predictor (Eq. 13) at the half node just behind it and the corrector
 // (Eq. 14) at the column behind that, and stores u^{n+1}.  Radial neighbours are the
-// registers of the previous column; the theta neighbours of the input state are read
-// from the ring slot, and those of the predictor's results through a small shared
+// registers of the previous column; the theta neighbours of the input state (FP32 paths) are
+// read from the ring slot, and those of the predictor's results through a small shared
 // exchange buffer (one barrier per column).  A strip reads two extra columns, so every
 // input is read from HBM about once per step.  The angular ghost
 // rows of the pole condition (Sec. 2.2) mirror row 0 / row n_theta-1 with sign +1
@@ -21,21 +21,20 @@
 // Arithmetic of the FP32 paths, in differences so that the compensated FP32 state keeps its
 // accuracy (a difference of two (hi, c) pairs is formed as (hi_a - hi_b) - (c_a - c_b)
 // before anything cancels):
-//   predictor at (i+1/2, j), with Fb = (Phi_i + Phi_{i+1})/2, dF = Phi_{i+1} - Phi_i,
-//   Dp(j) = Fb(j+1) - Fb(j) and the same for Pi:
-//     dh_Phi = -g dF + (dt/2) Pb
-//     dh_Pi  =  g dPi + E1 Pb + E2 dF + ep Dp(j) - em Dp(j-1) + E3 Fb + (dt/2) tau(t_n)
-//   corrector at (i, j) from the half nodes R = i+1/2, L = i-1/2:
-//     h_R - h_L = (dF_R + dF_L)/2 + dh_R - dh_L,  u~ = (Fb_R + Fb_L)/2 + (dh_R + dh_L)/2,
-//     Delta Phi = -g d(h_Phi) + dt Pi~
-//     Delta Pi  =  g d(h_Pi) + E1 Pi~ + E2 d(h_Phi) + ep D+ - em D- + E3 Phi~ + dt tau(t_n+dt/2)
+//   predictor at (i+1/2, j), with the undivided sums Fb = Phi_i + Phi_{i+1}, Pb of Pi, the
+//   differences dF = Phi_{i+1} - Phi_i, dP of Pi, and Dp = -(Fb(j+1) - 2 Fb(j) + Fb(j-1)),
+//   D1 = Fb(j+1) - Fb(j-1) formed from the state's own theta differences:
+//     dh_Phi = -g dF + (dt/4) Pb
+//     dh_Pi  =  g dP + E1 Pb + E2 dF + A Dp + B D1 + E3 Fb + (dt/2) tau(t_n)
+//   corrector at (i, j) from the half nodes R = i+1/2, L = i-1/2 (h = Fb/2 + dh):
+//     h_R - h_L = (dF_R + dF_L)/2 + dh_R - dh_L,  4 u~ = Fb_R + Fb_L + 2 (dh_R + dh_L),
+//     Delta Phi = -g d(h_Phi) + (dt/4) 4 Pi~
+//     Delta Pi  =  g d(h_Pi) + E1 4 Pi~ + E2 d(h_Phi) + A D2 + B D1 + E3 4 Phi~ + dt tau(t_n+dt/2)
 //     u^{n+1} = u^n + Delta   (Kahan-compensated for the FP32_KAHAN state)
-// with the scaled coefficients g, E1, E2, ep, em, E3 (see RTab2; the two
-// sub-steps differ only by the factor 1/2 versus 1 of dt).  This is Eqs. (13)-(14)
-// with S_Pi = -c_t Pi + P* Phi_* + w Theta[Phi] + q Phi + tau, rearranged, not
-// approximated.  The FP32 paths write the angular part ep D+ - em D- in the split form
-// A (D+ - D-) + B (D+ + D-) (A = (ep + em)/2, B = (ep - em)/2, see split_angular), with
-// the second and two-cell differences formed directly from the state.
+// (D2, D1: the same theta differences of 4 u~), with the scaled coefficients of RTab2, which
+// carry the powers of two of the undivided sums; A and B are the split form of the angular
+// part (see split_angular).  This is Eqs. (13)-(14) with S_Pi = -c_t Pi + P* Phi_* + w
+// Theta[Phi] + q Phi + tau, rearranged, not approximated.
 #include <type_traits>
 
 #include "teuk_internal.cuh"
@@ -354,10 +353,9 @@ __device__ __forceinline__ void strip_columns_x(const InstDev& d, int64_t step, 
 }
 
 // One work item: the columns [c0, c1) of one instance for one step, one thread per row.
-// Per column c: theta differences of Phi(c), dl = Phi(j+1) - Phi(j) and dlm = Phi(j) -
-// Phi(j-1), from the ring slot; predictor at the half node c-1/2; exchange of its
-// results with the rows above and below (the one barrier of the column); corrector at
-// column c-1.  The first two columns are peeled so the steady-state loop has no
+// Per column c (FP32 paths; strip_columns_x has the others): theta differences of Phi(c) from
+// the ring slot; predictor at the half node c-1/2; exchange of its results with the rows
+// above and below (the one barrier of the column); corrector at column c-1.  The first two columns are peeled so the steady-state loop has no
 // per-column mode switches, and it is unrolled by two so the rotation of the
 // previous / current column is register renaming (by two: measured faster than one,
 // three or six on GB300).  Columns c0-1 .. c1 are read.
@@ -473,8 +471,8 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
         // own node of the column in slot s (rows past nth read slot padding: their results
         // are never stored or exchanged)
         auto node = [&](int s) { return ring.planes(s).load((size_t)j); };
-        // theta differences of Phi in the column in slot s (own node u): forward and backward
-        // (expanded angular form) or second and two-cell (split form, see split_angular)
+        // theta differences of Phi in the column in slot s (own node u): second (negated) and
+        // two-cell (see split_angular)
         auto theta_diffs = [&](int s, const NodeV<P>& u, C& dl, C& dlm) {
             const Planes<P> pl = ring.planes(s);
             const NodeV<P> dn = pl.load_phi((size_t)jp), upn = pl.load_phi((size_t)jm);
@@ -486,9 +484,9 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
             const Half<T> hp = half_prep<P>(ul, ur);
             return predictor<T>(hp, dll + dlr, dlml + dlmr, cf, qdt, src);
         };
-        // coefficients of column col: the half node col+1/2 into cfh and, on the FP32 paths
-        // (formed together in paired instructions), the node col into cfi
-        auto coefs = [&](int slot, int col, T* cfh, T* cfi) {
+        // coefficients of the column whose tables are in slot: the half node to its right into
+        // cfh and the node into cfi, formed together in paired instructions
+        auto coefs = [&](int slot, T* cfh, T* cfi) {
             float2 cf2[kNCoef];
             form_coefs2(ring.tab2(slot), rt.t, cf2);
 #pragma unroll
@@ -497,11 +495,10 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
                 cfi[k] = cf2[k].y;
             }
         };
-        // corrector at column cc from the half nodes L = cc-1/2 and R = cc+1/2; xb is the
-        // exchange buffer of this column's parity, srcc the source term at (cc, j); cfi the
-        // node's coefficients on the FP32 paths (the FP64 path reads them here)
+        // corrector at a column from the half nodes L and R on its two sides; xb is the exchange
+        // buffer of the column's parity, srcc the node's source term, cfi its coefficients
         auto correct = [&](const HalfRec<T>& Rh, const HalfRec<T>& Lh, const NodeV<P>& uc,
-                           const T* cfi, int cc, T* xb, size_t o, C srcc) {
+                           const T* cfi, T* xb, size_t o, C srcc) {
             const CRow<T> row = combine_lr<T>(Rh, Lh);
             // publish this row's exchange entry (the split form needs Hs alone: its averaged
             // differences are the row's own), then read the rows above and below
@@ -527,7 +524,7 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
         NodeV<P> u_cur = node(1);
         theta_diffs(1, u_cur, dl, dlm);
         T cfh[kNCoef], cfi[kNCoef];
-        coefs(0, c0 - 1, cfh, cfi);
+        coefs(0, cfh, cfi);
         C s_first = C::zero();
         if constexpr (kMov) {
             if (gr) s_first = msrc_h(c0 - 1);
@@ -560,7 +557,7 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
             C nxt_h = C::zero(), nxt_i = C::zero();
             load_src(c0, nxt_h, nxt_i);
             int sf = 0, sp = 1, sc = 2;
-    #pragma unroll 2
+#pragma unroll 2
             for (int c = c0 + 1; c <= c1; ++c) {
                 const C s_h = nxt_h, s_i = nxt_i;
                 if constexpr (kSrc != 0) {
@@ -569,9 +566,9 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
                 ring.wait(sc);
                 u_cur = node(sc);
                 theta_diffs(sc, u_cur, dl, dlm);
-                coefs(sp, c - 1, cfh, cfi);
+                coefs(sp, cfh, cfi);
                 const HalfRec<T> Rh = predict(u_prev, u_cur, dl_prev, dl, dlm_prev, dlm, cfh, s_h);
-                correct(Rh, L, u_prev, cfi, c - 1, xbuf + (c & 1) * xstride, o, s_i);
+                correct(Rh, L, u_prev, cfi, xbuf + (c & 1) * xstride, o, s_i);
                 if (threadIdx.x == 0 && c - 2 + R <= c1) ring.template fill<kSrc != 0>(d, bin, c - 2 + R, sf);
                 L = Rh;
                 u_prev = u_cur;
@@ -608,8 +605,8 @@ __device__ __forceinline__ bool strip_step(const InstDev& d, int64_t step, int b
 
 // Four register budgets: columns of up to 256 rows (the common case, P::blocks256
 // blocks per SM), of up to 320 rows (FP32 paths, two blocks per SM, 96 registers), of
-// up to 512 rows (one block per SM, 128 registers a thread) and of up to 1024 rows.  Dynamic shared memory:
-// StepShared<P, R>::bytes(blockDim.x).
+// up to 512 rows (one block per SM, 128 registers a thread) and of up to 1024 rows.
+// Dynamic shared memory: StepShared<P, R>::bytes(blockDim.x).
 // part (may be null): the block's columns are [part[b], part[b+1]), of `strip` pieces, instead
 // of uniform strips of `strip` columns; it is written by the host before the launch sequence
 // and never changes while a step runs, so it is read before griddepcontrol.wait.
@@ -662,7 +659,7 @@ __host__ __device__ constexpr bool has_wide() { return split_angular<P>(); }
 template <class P, bool kMov>
 __global__ void __launch_bounds__(kWideRows, 2) step_kernel_w(InstDev d, int64_t step, int bin, int strip,
                                                              const int* part) {
-    if constexpr (has_wide<P>()) step_body<P, kRingS, kMov>(d, step, bin, strip, part);
+    step_body<P, kRingS, kMov>(d, step, bin, strip, part);
 }
 
 template <class P, bool kMov>
@@ -922,7 +919,7 @@ static void launch_step_m(cudaStream_t st, const InstDev& d, int64_t step, int b
         cudaLaunchKernelEx(&cfg, step_kernel_s<P, kMov>, d, step, bin, strip, part);
     } else if (threads <= kWideRows && has_wide<P>()) {
         cfg.dynamicSmemBytes = StepShared<P, kRingS>::bytes(threads);
-        cudaLaunchKernelEx(&cfg, step_kernel_w<P, kMov>, d, step, bin, strip, part);
+        if constexpr (has_wide<P>()) cudaLaunchKernelEx(&cfg, step_kernel_w<P, kMov>, d, step, bin, strip, part);
     } else if (threads <= 512) {
         cfg.dynamicSmemBytes = StepShared<P, kRingS>::bytes(threads);
         cudaLaunchKernelEx(&cfg, step_kernel_m<P, kMov>, d, step, bin, strip, part);
@@ -945,10 +942,11 @@ static int resident_p(int threads) {
     if (threads <= 256)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel_s<P, false>, threads,
                                                       StepShared<P, kRingS>::bytes(threads));
-    else if (threads <= kWideRows && has_wide<P>())
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel_w<P, false>, threads,
-                                                      StepShared<P, kRingS>::bytes(threads));
-    else if (threads <= 512)
+    else if (threads <= kWideRows && has_wide<P>()) {
+        if constexpr (has_wide<P>())
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel_w<P, false>, threads,
+                                                          StepShared<P, kRingS>::bytes(threads));
+    } else if (threads <= 512)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel_m<P, false>, threads,
                                                       StepShared<P, kRingS>::bytes(threads));
     else
@@ -992,8 +990,10 @@ static cudaError_t prepare_m() {
               l = (int)StepShared<P, kRingL>::bytes(1024);
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(step_kernel_s<P, kMov>, a, s);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(step_kernel_w<P, kMov>, a, (int)StepShared<P, kRingS>::bytes(kWideRows));
+    if constexpr (has_wide<P>()) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(step_kernel_w<P, kMov>, a, (int)StepShared<P, kRingS>::bytes(kWideRows));
+    }
     if (e == cudaSuccess) e = cudaFuncSetAttribute(step_kernel_m<P, kMov>, a, m);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(step_kernel_l<P, kMov>, a, l);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(batched_step_kernel<P, 256, P::blocks256, kRingS, kMov>, a, s);

@@ -36,9 +36,6 @@ template <typename T>
 __device__ __forceinline__ Cx<T> rmac(Cx<T> acc, T s, Cx<T> z) {
     return {tfma(s, z.re, acc.re), tfma(s, z.im, acc.im)};
 }
-// -a
-template <typename T>
-__device__ __forceinline__ Cx<T> neg(Cx<T> a) { return {-a.re, -a.im}; }
 
 // FP32 complex values in paired instructions (sm_100 and later: FADD2 / FMUL2 / FFMA2
 // act on both components of a register pair).  Each component rounds exactly as the
@@ -54,7 +51,6 @@ __device__ __forceinline__ Cx<float> operator+(Cx<float> a, Cx<float> b) {
 __device__ __forceinline__ Cx<float> operator-(Cx<float> a, Cx<float> b) {
     return up(__ffma2_rn(bc(-1.0f), pk(b), pk(a)));
 }
-__device__ __forceinline__ Cx<float> neg(Cx<float> a) { return up(__fmul2_rn(bc(-1.0f), pk(a))); }
 __device__ __forceinline__ Cx<float> operator*(float s, Cx<float> a) {
     return up(__fmul2_rn(bc(s), pk(a)));
 }
@@ -95,10 +91,6 @@ __device__ __forceinline__ Cx<DF> operator-(Cx<DF> x, Cx<DF> y) {
     const DF2 X = pk2(x), Y = pk2(y);
     const DF2 S = p_two_diff(X.hi, Y.hi);
     return up2(p_fast_two_sum(S.hi, p_add(S.lo, p_sub(X.lo, Y.lo))));
-}
-__device__ __forceinline__ Cx<DF> neg(Cx<DF> a) {
-    const DF2 A = pk2(a);
-    return up2({p_neg(A.hi), p_neg(A.lo)});
 }
 // a * b + c per component, a given as pairs (hi, lo): the double-float tfma without its last
 // normalisation (see Lin<DF> for how large lo may get)
