@@ -223,7 +223,7 @@ void launch_trajectory(cudaStream_t st, double M, double a, int m, double rstar_
                        const double* x_half, const double* traj, int64_t n_samples,
                        const SourceDev& src, int prec);
 // teuk_step.cu
-cudaError_t prepare_step_kernels();
+cudaError_t prepare_step_kernels(int prec);
 int step_resident_blocks(int prec, int threads);  // blocks of the step kernel the GPU holds at once
 // How a per-step launch cuts the columns: uniform strips of `strip` columns (part null), or
 // nb pieces, block b covering [part[b], part[b+1]) (part: device); cap > 0: at most cap

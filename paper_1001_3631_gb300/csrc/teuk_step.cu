@@ -980,8 +980,8 @@ void launch_step(cudaStream_t st, const InstDev& d, int64_t step, int bin, const
 // through the L1), 70 per cent leaves 132 KB, too little.
 constexpr int kBatchCarveout = 72;
 
-// Opt the step kernels in to the dynamic shared memory of their largest blocks (on the
-// current device; called when a context is created).
+// Opt the step kernels of one precision in to the dynamic shared memory of their largest
+// blocks (on the current device; called when a context of that precision is created).
 template <class P, bool kMov>
 static cudaError_t prepare_m() {
     // (a capped launch, FP64 and double-float, takes more than its blocks need)
@@ -1011,12 +1011,11 @@ static cudaError_t prepare_p() {
     return e;
 }
 
-cudaError_t prepare_step_kernels() {
-    cudaError_t e = prepare_p<P64>();
-    if (e == cudaSuccess) e = prepare_p<P32>();
-    if (e == cudaSuccess) e = prepare_p<PK>();
-    if (e == cudaSuccess) e = prepare_p<PD>();
-    return e;
+cudaError_t prepare_step_kernels(int prec) {
+    if (prec == 0) return prepare_p<P64>();
+    if (prec == 1) return prepare_p<P32>();
+    if (prec == 3) return prepare_p<PD>();
+    return prepare_p<PK>();
 }
 
 void launch_extract(cudaStream_t st, const InstDev& d, int64_t step, int bin) {
