@@ -2,9 +2,10 @@
 kept whatever its value, and the autotuner knows the automatic cut."""
 import json
 
+import numpy as np
 import pytest
 
-from paper_1001_3631_gb300 import TeukSolver
+from paper_1001_3631_gb300 import TeukSolver, inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -70,3 +71,27 @@ def test_tables_of_other_cuts_are_not_used(tmp_path):
         cache.write_text(json.dumps({old: 3}))
         s.autotune(trial_steps=2, cache_path=str(cache))
         assert json.loads(cache.read_text()).keys() == {old, key}
+
+
+# the record at the two ends of the grid, beside them and inside, by the piece that holds it (a
+# launch with a piece for every place) and by a block of its own (one piece)
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp64_df", 1e-12), ("fp32_kahan", 1e-5), ("fp32", 1e-5)])
+@pytest.mark.parametrize("ext", [-10.0, -9.99, 14.0, 29.99, 30.0])
+def test_record_in_a_launch_that_takes_every_place(orc, prec, tol, ext):
+    nr, nth, n = 2500, 100, 3
+    p = dict(params_of(nr, nth, prec), rstar_ext=ext)
+    u0 = inputs.random_state(nth, nr, seed=5)
+    po = orc.params(**{k: v for k, v in p.items() if k != "prec"}, r0=7.5)
+    _, wo = orc.run(po, u0, n, orc.orbit_source(po))
+    waves = []
+    for strip in (0, nr):
+        with TeukSolver(p) as s:
+            s.set_tiling(strip, 1)
+            pieces = s.tiling()["pieces"]
+            assert pieces == 1 if strip else pieces % 152 == 0 and pieces >= 3 * 152   # 152 SMs
+            s.set_source(7.5)
+            s.set_state(u0)
+            s.step(n)
+            waves.append(s.extract()[0])
+    assert np.array_equal(waves[0], waves[1])
+    assert np.abs(waves[0] - wo).max() <= tol * max(np.abs(wo).max(), 1.0)
