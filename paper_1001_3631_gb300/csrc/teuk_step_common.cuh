@@ -395,7 +395,7 @@ __host__ __device__ constexpr bool split_angular() { return P::kind == kFP32 || 
 // FP32 operations a node, and no register spills: the record of a half node is two complex
 // values instead of eight); with the time steps formed on the host and the pole factor
 // applied to the sign bits (85 -> 75 FP64 instructions a node, and 14 -> 0 on the
-// double-float path) and double-float coefficients loaded ahead: FP64 570, double-float 148.
+// double-float path) and double-float coefficients loaded ahead: FP64 570 to 576, double-float 148.
 
 // Complex sums and differences.  FP64: as DFMA with a factor one that the compiler cannot
 // see (DADD and DMUL take 19 clocks of the SM's FP64 pipe, DFMA 16; the rounding is the
