@@ -105,20 +105,22 @@ class _HostBuffers:
     MIN, KEEP = 4 << 20, 1 << 30
 
     def __init__(self):
-        self._lock = threading.Lock()
+        self._lock = threading.Lock()   # of _bufs
+        self._count = threading.RLock()   # of _users and _closed
         self._bufs = []   # [mapping, weak reference to the object that its arrays hold], oldest first
         self._dropped = False   # an array died since the idle mappings were last counted
         self._users, self._closed = 0, False
 
     def open(self):
         """One more solver."""
-        with self._lock:
+        with self._count:
             self._users += 1
             self._closed = False
 
     def close(self):
-        """One solver less; after the last nothing is kept idle."""
-        with self._lock:
+        """One solver less; after the last nothing is kept idle.  (A solver's finalizer may run
+        in a thread that is within empty(): the lock of _bufs is never waited for here.)"""
+        with self._count:
             self._users -= 1
             self._closed = self._users <= 0
         self._dropped = True
@@ -162,22 +164,28 @@ class _HostBuffers:
         # find one again
         step = 1 << (size.bit_length() - 5)
         whole = (size + step - 1) // step * step
-        with self._lock:
-            buf = next((b for b in self._bufs if len(b[0]) == whole and b[1]() is None), None)
-            again = buf is not None
-            if again:
-                self._bufs.remove(buf)
-            else:
-                try:
-                    buf = [mmap.mmap(-1, whole, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS), None]
-                    # (as numpy does for its own arrays)
-                    buf[0].madvise(mmap.MADV_HUGEPAGE)
-                except (AttributeError, OSError, OverflowError, ValueError):
-                    pass
-            if buf is not None:
-                raw = (ctypes.c_char * size).from_buffer(buf[0])
-                buf[1] = self._watch(raw)   # dead when the last array on the mapping is gone
-                self._bufs.append(buf)
+        buf = None
+        # (not waited for without end: a finalizer that asks for an array may have interrupted
+        # this very thread's call)
+        if self._lock.acquire(timeout=0.1):
+            try:
+                buf = next((b for b in self._bufs if len(b[0]) == whole and b[1]() is None), None)
+                again = buf is not None
+                if again:
+                    self._bufs.remove(buf)
+                else:
+                    try:
+                        buf = [mmap.mmap(-1, whole, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS), None]
+                        # (as numpy does for its own arrays)
+                        buf[0].madvise(mmap.MADV_HUGEPAGE)
+                    except (AttributeError, OSError, OverflowError, ValueError):
+                        pass
+                if buf is not None:
+                    raw = (ctypes.c_char * size).from_buffer(buf[0])
+                    buf[1] = self._watch(raw)   # dead when the last array on the mapping is gone
+                    self._bufs.append(buf)
+            finally:
+                self._lock.release()
         self._settle()
         if buf is None:   # no mapping to be had: numpy's own answer
             return np.empty(shape, dtype)

@@ -99,3 +99,24 @@ def test_many_threads_drop_and_ask():
         t.join()
     gc.collect()
     assert not bad and idle(h) <= h.KEEP and not h._lock.locked()
+
+
+def test_a_finalizer_within_a_call_does_not_wait_for_it():
+    # the collector may close a solver, drop an array or ask for one while this thread is in
+    # empty(): the lock is then held by the thread itself
+    h = solver._HostBuffers()
+    h.open()
+    a = h.empty(BIG)
+    got = []
+
+    def finalizer():
+        with h._lock:
+            h.close()
+            got.append(h.empty(BIG))
+
+    t = threading.Thread(target=finalizer, daemon=True)
+    t.start()
+    t.join(20)
+    assert not t.is_alive() and got[0].flags["OWNDATA"]
+    del a
+    assert not h._bufs
