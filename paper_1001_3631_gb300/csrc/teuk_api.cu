@@ -1056,10 +1056,10 @@ void form_classes(const teuk_ctx* c, Batch& B) {
 // order; blocks are added where a block has most columns.  Measured on 54 batches of two to
 // four classes of 1 to 10 warps, in each precision: one class after the other / side by side.
 //   longest share up to 1.3 of the even one and up to 70 columns a place: 0.99 to 2.5 (FP32-Kahan
-//     6 modes of 1024..4100 columns and 64, 128, 192 rows, 47 columns: 46.2 -> 37.0 us; 20, 50,
+//     6 modes of 1024..4100 columns and 64, 128, 192 rows, 29 columns: 46.2 -> 37.0 us; 20, 50,
 //     70 rows, 0.3 columns: 24.9 -> 10.3; FP64 3000 columns of 32 and 64 rows, 4.9: 63.2 -> 55.8)
 //   86 columns a place: 0.83 to 0.89, 104: 0.99 to 1.05; 2000 (128 instances): 0.94
-//   longest share 1.35 to 1.5: 0.99 to 3.1; 1.6 to 1.9 with 24 columns and more: 0.75 to 1.05
+//   longest share 1.35 to 1.5: 0.98 to 3.1; 1.58 to 1.91 with 29 columns and more: 0.75 to 1.05
 void plan_branches(teuk_ctx* c, Batch& B) {
     constexpr int kThreads = 512;
     std::vector<double> work(B.cls.size(), 0.0);
