@@ -108,7 +108,16 @@ class _HostBuffers:
         self._lock = threading.Lock()   # of _bufs
         self._count = threading.RLock()   # of _users and _closed
         self._bufs = []   # [mapping, weak reference to the object that its arrays hold], oldest first
+        self._mapped = 0   # bytes of _bufs
         self._dropped = False   # an array died since the idle mappings were last counted
+        pool = weakref.ref(self)
+
+        def dropped(_):
+            p = pool()
+            if p is not None:
+                p._dropped = True
+                p._settle()
+        self._watch = dropped
         self._users, self._closed = 0, False
 
     def open(self):
@@ -129,7 +138,7 @@ class _HostBuffers:
     def _settle(self):
         # runs in whatever thread drops an array, at any moment (within empty() too, by the
         # collector): it never waits; who holds the lock settles again after giving it back
-        while self._dropped and self._lock.acquire(blocking=False):
+        while self._dropped and (self._closed or self._mapped > self.KEEP) and self._lock.acquire(blocking=False):
             try:
                 self._dropped = False
                 idle = [b for b in self._bufs if b[1]() is None]
@@ -139,18 +148,9 @@ class _HostBuffers:
                         break
                     self._bufs.remove(b)
                     kept -= len(b[0])
+                    self._mapped -= len(b[0])
             finally:
                 self._lock.release()
-
-    def _watch(self, raw):
-        pool = weakref.ref(self)
-
-        def dropped(_):
-            p = pool()
-            if p is not None:
-                p._dropped = True
-                p._settle()
-        return weakref.ref(raw, dropped)
 
     def empty(self, shape, dtype=np.float64):
         dtype = np.dtype(dtype)
@@ -180,9 +180,11 @@ class _HostBuffers:
                         buf[0].madvise(mmap.MADV_HUGEPAGE)
                     except (AttributeError, OSError, OverflowError, ValueError):
                         pass
+                    if buf is not None:
+                        self._mapped += whole
                 if buf is not None:
                     raw = (ctypes.c_char * size).from_buffer(buf[0])
-                    buf[1] = self._watch(raw)   # dead when the last array on the mapping is gone
+                    buf[1] = weakref.ref(raw, self._watch)   # dead when the last array on the mapping is gone
                     self._bufs.append(buf)
             finally:
                 self._lock.release()
